@@ -20,8 +20,8 @@
  * summed as a zero-padded FFT convolution; pairs in different patches either
  * by level convolutions (every level on the finest lattice, fractional-offset
  * kernel tables) or by a direct sum (the corner form in FP64; in FP32 plans
- * FP64 near cells and a cell-centred expansion of far cells). All give the sum
- * above to rounding.
+ * tabulated FP64 integrals of near cells, a cell-centred expansion of the cells
+ * around them and clusters of cells beyond). All give the sum above to rounding.
  *
  * Conventions
  *  - Every entry point returns an sg_status; no exception or signal crosses
@@ -107,9 +107,9 @@ typedef struct {
 
 typedef enum {
     SG_CROSS_AUTO = 0,          /* level convolutions when the hierarchy fits, else direct */
-    SG_CROSS_DIRECT = 1,        /* per-patch FFT convolutions + the direct sum across patches (corner
-                                   form in FP64 plans; FP64 near cells and a far-field expansion,
-                                   or quadrature off the plane, in FP32 plans) */
+    SG_CROSS_DIRECT = 1,        /* per-patch FFT convolutions + the sum across patches (corner form in
+                                   FP64 plans; tabulated near cells, a cell expansion, or quadrature
+                                   off the plane, and clusters of far cells in FP32 plans) */
     SG_CROSS_LEVELS = 2         /* level convolutions (SG_EINVAL if the hierarchy does not fit):
                                    every level's composite source on the finest lattice, every
                                    ordered pair of levels one zero-padded FFT convolution with
@@ -212,8 +212,8 @@ sg_status sg_force(sg_plan *plan, const void *sigma, const void *deltax, const v
  * K^{z,x} = (x - xc) K^{z,0} - z K^{x,0}, K^{z,y} = (y - yc) K^{z,0} - z K^{y,0};
  * a hierarchy (or masked patch) takes each patch's own convolution with its
  * height-z tables plus the cross-patch sum: the corner form of the off-plane
- * antiderivatives in FP64 (every pair in FP64 plans; the near cells in FP32
- * plans, whose far cells take Gauss-Legendre quadrature of the cell integrals).
+ * antiderivatives in FP64 plans; in FP32 plans tabulated integrals of the near
+ * cells, Gauss-Legendre quadrature of those around them, clusters beyond.
  * For a z = 0 plan Fx, Fy are those of sg_force and Fz is the limit from
  * above the plane, -2 pi G sigma0 of the target's own cell (the other cells'
  * normal forces vanish in the plane). Errors: as sg_force.
@@ -228,8 +228,8 @@ sg_status sg_force3(sg_plan *plan, const void *sigma, const void *deltax, const 
  * (z == 0): one unmasked patch, with the plan's slope mode (central slopes are
  * formed in the row transform here), or a hierarchy (patches, masks) on either
  * path of its plan (level convolutions, or each patch's own convolution plus
- * the cross-patch direct sum: the corner form in FP64 plans, FP64 near cells
- * and a moment expansion of far cells in FP32 plans), summed over the leaf
+ * the cross-patch sum: the corner form in FP64 plans, tabulated near cells, a
+ * moment expansion and clusters of far cells in FP32 plans), summed over the leaf
  * cells as for sg_force (the output at covered cells is unspecified):
  *   Phi(t) = -G sum_i [sigma0_i P^0_i(t) + deltax_i P^x_i(t) + deltay_i P^y_i(t)],
  *   P^0, P^x, P^y = integrals over cell i of 1/r, (xbar - xc_i)/r, (ybar - yc_i)/r,
@@ -281,8 +281,7 @@ sg_status sg_plan_wait(sg_plan *plan, void *stream);
 
 /*
  * Bounded waits (not in the paper). Kernels that wait for bulk copies into
- * shared memory (the column passes' kernel spectra, the FP32 direct sum's
- * source tiles) give up after a number of attempts, record the failure in the
+ * shared memory (the column passes' kernel spectra) give up after a number of attempts, record the failure in the
  * workspace's device error word, wait for their copies in flight (with the
  * default limit) and return early; the solve's outputs are then invalid.
  *
@@ -468,12 +467,12 @@ sg_status sg_autotune(int precision, int min_pad, int max_pad, int reps, double 
 
 /* Tune the cross-patch direct sum of one plan (hierarchies on the direct
  * path; a no-op returning *best_ms = 0 for other plans): the source-tile
- * ranges per target block (the plan's value, a half or a quarter of it) and,
- * for FP32 plans, the CTAs of the persistent far-field launch (1, 2, 3, 4, 6
- * or 8 per SM), each timed as the median of `reps` solves on zero fields with
- * the plan's own workspace; the fastest pair stays in the plan. The split only
- * regroups the FP64 partial sums of the far field (results agree to FP64
- * rounding; the far-field grid changes nothing). Synchronous; call with no
+ * ranges per target block of FP64 plans (the plan's value, a half or a quarter
+ * of it; 1 in FP32 plans) and, for FP32 plans, the CTAs of the far-field launch
+ * (one per target block, or 1, 2, 3, 4, 6 or 8 per SM that share the blocks),
+ * each timed as the median of `reps` solves on zero fields with the plan's own
+ * workspace; the fastest pair stays in the plan. The split only regroups the FP64
+ * partial sums (results agree to FP64 rounding; the far-field grid changes nothing). Synchronous; call with no
  * solve of the plan in flight and before capturing the plan into a batch.
  * sg_plan_direct_shape reads the pair. best_ms may be NULL. Errors: SG_EINVAL,
  * SG_ENOMEM, SG_ECUDA. */

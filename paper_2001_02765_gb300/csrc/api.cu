@@ -241,16 +241,15 @@ sg_status analyse(const sg_geom *g, geom_info &gi)
 size_t elem_size(sg_precision prec) { return prec == SG_FP64 ? 8 : 4; }
 
 // Source tiles of every patch (the composite sources cover whole patches):
-// 16 x 16 corners for the FP64 corner-form sum, 16 x 16 cells for the FP32
-// near/far sum. With masks, tiles that touch no existing cell carry zero
-// weights and are left out.
-void build_tiles(const sg_geom *g, const geom_info &gi, bool cell_tiles, std::vector<sg_tile_desc> &tiles,
-                 std::vector<int> &first, std::vector<int> &count)
+// 16 x 16 corners for the FP64 corner-form sum. With masks, tiles that touch no
+// existing cell carry zero weights and are left out.
+void build_tiles(const sg_geom *g, const geom_info &gi, std::vector<sg_tile_desc> &tiles, std::vector<int> &first,
+                 std::vector<int> &count)
 {
     first.assign(gi.n, 0);
     count.assign(gi.n, 0);
     std::vector<int64_t> sat;  // summed-area table of existing cells, (ny + 1) x (nx + 1)
-    const int extra = cell_tiles ? 0 : 1;  // a patch has nx + 1 corners per row, nx cells
+    const int extra = 1;  // a patch has nx + 1 corners per row
     for (int k = 0; k < gi.n; ++k) {
         const sg_patch &p = g->patches[k];
         const bool masked = g->masks && g->masks[k];
@@ -268,8 +267,7 @@ void build_tiles(const sg_geom *g, const geom_info &gi, bool cell_tiles, std::ve
             for (int a = 0; a < ntx; ++a) {
                 const int ci0 = a * SG_TILE_X, cj0 = b * SG_TILE_Y;
                 if (masked) {
-                    // cells of the tile (cell tiles: i in [ci0, ci0 + TILE_X - 1]) or around
-                    // its corners (corner tiles: i in [ci0 - 1, ci0 + TILE_X - 1]); same in j
+                    // cells around the tile's corners: i in [ci0 - 1, ci0 + TILE_X - 1]; same in j
                     const int i0 = ci0 - extra > 0 ? ci0 - extra : 0, j0 = cj0 - extra > 0 ? cj0 - extra : 0;
                     const int i1 = ci0 + SG_TILE_X < p.nx ? ci0 + SG_TILE_X : p.nx;
                     const int j1 = cj0 + SG_TILE_Y < p.ny ? cj0 + SG_TILE_Y : p.ny;
@@ -499,13 +497,12 @@ bool lv_params(const sg_geom *g, const geom_info &gi, sg_precision prec, sg_lv_s
     return true;
 }
 
-// Source-tile ranges per target block. FP64 plans: enough (block, range) CTAs
-// for two per SM. FP32 plans: work items of the persistent far-field launch,
-// about 32 per SM so that dynamic scheduling evens out their unequal costs.
+// Source-tile ranges per target block of FP64 plans: enough (block, range) CTAs
+// for two per SM. FP32 plans have one CTA per block (no ranges).
 int choose_nsplit(int nblocks, int ntiles, int nsm, sg_precision prec)
 {
-    if (nblocks <= 0) return 1;
-    const int want = prec == SG_FP64 ? 2 * nsm : 32 * nsm;
+    if (nblocks <= 0 || prec == SG_FP32) return 1;
+    const int want = 2 * nsm;
     int s = (want + nblocks - 1) / nblocks;
     const int cap = ntiles / 4 > 1 ? ntiles / 4 : 1;
     if (s > cap) s = cap;
@@ -514,13 +511,21 @@ int choose_nsplit(int nblocks, int ntiles, int nsm, sg_precision prec)
 }
 
 struct sizes {
-    int64_t spectra = 0, twiddles = 0, work = 0, direct = 0, geometry = 0;
+    int64_t spectra = 0, twiddles = 0, work = 0, direct = 0, geometry = 0, near = 0;
     int max_pad = SG_MIN_PAD;
-    int64_t total() const { return spectra + twiddles + work + direct + geometry; }
+    int64_t total() const { return spectra + twiddles + work + direct + geometry + near; }
 };
 
+std::vector<int64_t> level_leaves(const sg_geom *g, const geom_info &gi)
+{
+    std::vector<int64_t> n(gi.lmax + 1, 0);
+    for (int k = 0; k < gi.n; ++k) n[g->patches[k].level] += gi.nleaf[k];
+    return n;
+}
+
+// gmax: the largest width ratio 2^gmax with near tables (FP32 plans on the direct path)
 sizes plan_sizes(const sg_geom *g, const geom_info &gi, sg_precision prec, int ntiles, int nblocks, int nsplit,
-                 int64_t lv_bytes = -1)
+                 int64_t lv_bytes = -1, int gmax = SG_NT_GMAX)
 {
     sizes s;
     const size_t es = elem_size(prec);
@@ -538,13 +543,24 @@ sizes plan_sizes(const sg_geom *g, const geom_info &gi, sg_precision prec, int n
     if (gi.n > 1 || gi.masked) s.direct = 3 * gi.ncells * (int64_t)es + gi.ncells * (int64_t)sizeof(int);
     if ((gi.n > 1 || gi.masked) && g->slope_mode == SG_SLOPES_CENTRAL) s.direct += 40 * gi.ncells;  // links, centres
     if (gi.n > 1 && lv_bytes < 0) {
-        // off the plane: three partial components per split (and the near field in FP32 plans)
-        const bool off = g->z != 0.0;
-        const int64_t slices = off ? ((int64_t)nsplit + (prec == SG_FP32 ? 1 : 0)) * 3 / 2 + 1
-                                   : (prec == SG_FP64 ? (nsplit > 1 ? nsplit : 0) : nsplit + 1);
-        s.direct += (int64_t)ntiles * ((int64_t)sizeof(sg_tile_desc) + SG_TILE_N * 4 * (int64_t)es) +
-                    gi.nleaves * (int64_t)sizeof(int4) + (int64_t)nblocks * (int64_t)sizeof(sg_target_block) +
-                    slices * gi.nleaves * 16;
+        s.direct += gi.nleaves * (int64_t)sizeof(int4) + (int64_t)nblocks * (int64_t)sizeof(sg_target_block);
+        if (prec == SG_FP32) {
+            // clusters of 8 x 8 cells and their parents (up to 4/3 of them), the near field
+            int64_t ncl = 0;
+            for (int k = 0; k < gi.n; ++k)
+                for (int w = SG_CL_CELLS;; w *= 2) {
+                    const int64_t cx = (g->patches[k].nx + w - 1) / w, cy = (g->patches[k].ny + w - 1) / w;
+                    ncl += cx * cy;
+                    if (cx == 1 && cy == 1) break;
+                }
+            s.direct += sg_far_bytes(ncl, gi.nleaves, g->z);
+            s.near = sg_near_table_bytes(gi.lmax + 1, level_leaves(g, gi).data(), g->z, gmax);
+        } else {
+            // off the plane: three partial components per split
+            const int64_t slices = g->z != 0.0 ? (int64_t)nsplit * 3 / 2 + 1 : (nsplit > 1 ? nsplit : 0);
+            s.direct += (int64_t)ntiles * ((int64_t)sizeof(sg_tile_desc) + SG_TILE_N * 4 * (int64_t)es) +
+                        slices * gi.nleaves * 16;
+        }
     }
     s.geometry = (int64_t)gi.n * (int64_t)sizeof(sg_patch_dev) + 16 * (int64_t)gi.n;
     return s;
@@ -613,6 +629,7 @@ void plan_free(sg_plan *plan)
         sg_workspace_free(plan->ws, 0, false);
         delete plan->ws;
     }
+    sg_far_free(plan);
     cudaFree(plan->tiles);
     cudaFree(plan->targets);
     cudaFree(plan->blocks);
@@ -643,15 +660,19 @@ sg_status plan_build(const sg_geom *g, sg_precision prec, size_t budget, sg_plan
     }
     std::vector<sg_tile_desc> tiles;
     std::vector<int> tfirst, tcount;
-    // corner tiles for the corner form (FP64 plans), cell tiles for the FP32 far field
-    const bool corner_form = prec == SG_FP64;
-    if (gi.n > 1 && !use_lv) build_tiles(g, gi, !corner_form, tiles, tfirst, tcount);
+    // corner tiles for the corner form (FP64 plans); FP32 plans sum by clusters
+    const bool direct = gi.n > 1 && !use_lv;
+    if (direct && prec == SG_FP64) build_tiles(g, gi, tiles, tfirst, tcount);
     int dev = 0, nsm = 152;
     SG_CUDA_TRY(cudaGetDevice(&dev));
     SG_CUDA_TRY(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
     const int nblocks = use_lv ? 0 : count_blocks(g, gi);
-    const int nsplit = choose_nsplit(nblocks, (int)tiles.size(), nsm, corner_form ? SG_FP64 : prec);
-    const sizes sz = plan_sizes(g, gi, prec, (int)tiles.size(), nblocks, nsplit, lv_bytes);
+    const int nsplit = choose_nsplit(nblocks, (int)tiles.size(), nsm, prec);
+    // near tables as far as the budget goes (pairs of levels without one take the corner form)
+    int gmax = SG_NT_GMAX;
+    sizes sz = plan_sizes(g, gi, prec, (int)tiles.size(), nblocks, nsplit, lv_bytes, gmax);
+    while (budget && sz.near > 0 && (size_t)sz.total() > budget && gmax > -2)
+        sz = plan_sizes(g, gi, prec, (int)tiles.size(), nblocks, nsplit, lv_bytes, --gmax);
     if (budget && (size_t)sz.total() > budget) {
         set_error("plan exceeds the device-memory budget");
         return SG_EBUDGET;
@@ -784,36 +805,29 @@ sg_status plan_build(const sg_geom *g, sg_precision prec, size_t budget, sg_plan
     plan->ws_fwd_bytes = wf;
     plan->ws_inv_bytes = wi;
     // cross-patch direct sum
-    if (st == SG_OK && gi.n > 1 && !tiles.empty()) {
-        plan->ntiles = (int)tiles.size();
-        st = dev_alloc(plan, &plan->tiles, tiles.size() * sizeof(sg_tile_desc));
-        if (st == SG_OK)
-            st = cudaMemcpy(plan->tiles, tiles.data(), tiles.size() * sizeof(sg_tile_desc), cudaMemcpyHostToDevice) ==
-                         cudaSuccess ? SG_OK : SG_ECUDA;
-        const size_t nw = (size_t)plan->ntiles * SG_TILE_N;
-        // FP64 corner weights (FP64 plans), FP32 cell coefficients (FP32 plans)
-        const bool wide = prec == SG_FP64;
-        plan->ws_tile_bytes = (int64_t)nw * (wide ? (int64_t)sizeof(sg_dvec4) : (int64_t)sizeof(float4));
+    if (st == SG_OK && direct) {
         // targets: every leaf, in blocks of the leaves of 16 x 16 cells
         std::vector<int4> tg;
         std::vector<sg_target_block> blocks;
         build_targets(g, gi, tg, blocks);
         plan->ntargets = (int)tg.size();
         plan->nblocks = (int)blocks.size();
-        if (st == SG_OK) st = dev_alloc(plan, &plan->targets, tg.size() * sizeof(int4));
+        st = sg_plan_upload(plan, (void **)&plan->targets, tg.data(), tg.size() * sizeof(int4));
         if (st == SG_OK)
-            st = cudaMemcpy(plan->targets, tg.data(), tg.size() * sizeof(int4), cudaMemcpyHostToDevice) == cudaSuccess
-                     ? SG_OK : SG_ECUDA;
-        if (st == SG_OK) st = dev_alloc(plan, &plan->blocks, blocks.size() * sizeof(sg_target_block));
-        if (st == SG_OK)
-            st = cudaMemcpy(plan->blocks, blocks.data(), blocks.size() * sizeof(sg_target_block),
-                            cudaMemcpyHostToDevice) == cudaSuccess ? SG_OK : SG_ECUDA;
-        const int64_t slices = prec == SG_FP64 ? (nsplit > 1 ? nsplit : 0) : nsplit + 1;
-        plan->ws_partial_bytes = slices * (int64_t)tg.size() * 2 * (int64_t)sizeof(double);
-        if (g->z != 0.0)  // off the plane: three components per split (FP32: and one slice for the near field)
-            plan->ws_partial_bytes =
-                ((int64_t)nsplit + (prec == SG_FP32 ? 1 : 0)) * (int64_t)tg.size() * 3 * (int64_t)sizeof(double);
-        if (st == SG_OK && prec == SG_FP32) st = sg_cross_far_grid(plan, nsm);
+            st = sg_plan_upload(plan, (void **)&plan->blocks, blocks.data(), blocks.size() * sizeof(sg_target_block));
+        if (st == SG_OK && prec == SG_FP64) {
+            plan->ntiles = (int)tiles.size();
+            st = sg_plan_upload(plan, (void **)&plan->tiles, tiles.data(), tiles.size() * sizeof(sg_tile_desc));
+            plan->ws_tile_bytes = (int64_t)plan->ntiles * SG_TILE_N * (int64_t)sizeof(sg_dvec4);  // corner weights
+            // partial sums per split (off the plane: three components, one split too)
+            plan->ws_partial_bytes = (g->z != 0.0 ? (int64_t)nsplit * 3 : (nsplit > 1 ? nsplit * 2LL : 0)) *
+                                     (int64_t)tg.size() * (int64_t)sizeof(double);
+        } else if (st == SG_OK) {
+            std::vector<const int *> codes(gi.n);
+            for (int k = 0; k < gi.n; ++k) codes[k] = gi.code[k].data();
+            st = sg_far_setup(plan, codes.data(), gi.lmax + 1, level_leaves(g, gi).data(), gmax);
+            if (st == SG_OK) plan->ntiles = plan->far->first[1];
+        }
     }
     if (st == SG_OK) st = sg_twiddles_build(plan);
     if (st == SG_OK) st = sg_phase_build(plan);
@@ -827,9 +841,10 @@ sg_status plan_build(const sg_geom *g, sg_precision prec, size_t budget, sg_plan
         if (plan->composite) {
             n += gi.lmax > 0 ? gi.lmax : 1;  // composite sources: covered cells of levels 1 .. lmax-1, then all S_l
             if (plan->amr_central) n += (gi.lmax > 1 ? gi.lmax - 1 : 0) + gi.lmax + 1;  // fills, then slopes per level
-            // direct sum: corner weights, pair sum (+ split reduction) in FP64; cell coefficients,
-            // far field, near field and the combination in FP32
-            if (plan->ntiles > 0) n += prec == SG_FP64 ? 2 + (nsplit > 1) : 4;
+            // direct sum: corner weights, pair sum (+ split reduction) in FP64; the charges of
+            // every cluster level, near field (tables, and the corner form where there is none)
+            // and far field in FP32
+            if (plan->ntiles > 0) n += prec == SG_FP64 ? 2 + (nsplit > 1) : plan->far->nlev + 2 + plan->far->untabled;
         }
         plan->launches = n;
     }
@@ -1016,10 +1031,9 @@ sg_status sg_plan_bytes(const sg_geom *geom, sg_precision prec, int64_t *bytes)
         lv_bytes = -1;
     std::vector<sg_tile_desc> tiles;
     std::vector<int> tf, tc;
-    const bool corner_form = prec == SG_FP64;
-    if (gi.n > 1 && lv_bytes < 0) build_tiles(geom, gi, !corner_form, tiles, tf, tc);
+    if (gi.n > 1 && lv_bytes < 0 && prec == SG_FP64) build_tiles(geom, gi, tiles, tf, tc);
     const int nblocks = lv_bytes < 0 ? count_blocks(geom, gi) : 0;
-    const int nsplit = choose_nsplit(nblocks, (int)tiles.size(), 152, corner_form ? SG_FP64 : prec);
+    const int nsplit = choose_nsplit(nblocks, (int)tiles.size(), 152, prec);
     *bytes = plan_sizes(geom, gi, prec, (int)tiles.size(), nblocks, nsplit, lv_bytes).total();
     return SG_OK;
 }
@@ -1108,6 +1122,7 @@ sg_status sg_potential(sg_plan *plan, const void *sigma, const void *deltax, con
         // hierarchy on the direct path: composite sources, each patch's own
         // convolution with its potential spectra, then the cross-patch sum
         SG_TRY(sg_potential_spectra_build(plan));
+        SG_TRY(sg_far_potential_tables(plan));
         SG_TRY(ensure_ws(plan));
         sg_timing_reset(plan->timing);
         plan->ws->timing = plan->timing;

@@ -107,27 +107,32 @@ struct __align__(32) sg_dvec4 {
 #define SG_MAX_PATCH_SIDE 2048
 #define SG_MAX_LEVELS 12
 
-// Source tiles of the cross-patch direct sum: TILE_X x TILE_Y corners (FP64
-// plans, corner form) or cells (FP32 plans, near/far split).
+// Source tiles of the cross-patch direct sum of FP64 plans (corner form):
+// TILE_X x TILE_Y corners.
 #define SG_TILE_X 16
 #define SG_TILE_Y 16
 #define SG_TILE_N (SG_TILE_X * SG_TILE_Y)
 // Leaf targets per CTA of the direct sum (a block covers 16 x 16 cells of one patch).
 #define SG_DIRECT_THREADS 256
-// FP32 direct sum: a source cell whose centre lies less than SG_NEAR_R of its
-// own widths from the target along both axes is summed exactly in FP64 (near
-// field); every other cell by the expansion of its integrals about its centre,
-// through H^6 for tiles closer than SG_FAR_R4 cell widths to a block, through
-// H^4 beyond.
+// FP32 plans (cross32.cu): a source cell whose centre lies less than SG_NEAR_R of
+// its own widths from the target along both axes is summed from closed forms
+// (near field); other cells by the expansion of their integrals about their
+// centre, or in clusters of SG_CL_CELLS 2^k cells per side.
 #define SG_NEAR_R 6
-#define SG_FAR_R4 32
+#define SG_CL_CELLS 8
+#define SG_CL_LEVELS 9          // clusters of a patch: 2048 / 8 = 2^8 per side, nine levels
+// Near tables: targets up to 2^SG_NT_GMAX times narrower than the source cells
+// (4^g positions of 6.9 KB each: 7 MB at 5), keyed by log2 of the source cell
+// width in lattice units (below SG_NT_STEPS) and the width ratio's exponent (-1 .. SG_NT_GMAX).
+#define SG_NT_GMAX 5
+#define SG_NT_KEYS (SG_NT_GMAX + 2)
+#define SG_NT_STEPS (SG_MAX_LEVELS + 1)
 
 struct sg_tile_desc {
     int patch;          // source patch
-    int ox, oy;         // lattice coordinates of corner (0, 0) of the tile (corner tiles) or of
-                        // the lower-left corner of its cell (0, 0) (cell tiles)
+    int ox, oy;         // lattice coordinates of corner (0, 0) of the tile
     int step;           // corner spacing (cell width) in lattice units
-    int ci0, cj0;       // first corner (cell) index (i, j) of the tile in its patch
+    int ci0, cj0;       // first corner index (i, j) of the tile in its patch
     int pad0, pad1;
 };
 
@@ -183,6 +188,33 @@ struct sg_lv {
     void *cphase;                            // exp(-i pi j / P), j in [0, P], x then y, complex T
     void *pspectra;                          // potential: [nkeys][3][px/2+1][sg_spec_stride(py)] T, built at the first call
     int64_t fwd_elems, spec_elems, inv_elems;
+};
+
+// Clusters of a patch (cross32.cu): level k has nx[k] x ny[k] squares of
+// SG_CL_CELLS 2^k cells, the first at index off[k] of the slot table.
+struct sg_cl_patch {
+    int nlev;
+    int nx[SG_CL_LEVELS], ny[SG_CL_LEVELS];
+    int off[SG_CL_LEVELS];
+};
+
+struct sg_near_tab {
+    void *data;         // device: float2 [class][plane][12 x 12]
+};
+
+// Cross-patch sum of an FP32 plan: clusters and near tables.
+struct sg_far {
+    sg_cl_patch *patch;     // device, per patch
+    int *slot;              // device: cluster -> charges (64 floats each), -1 where no cell exists
+    int4 *desc;             // device, per charged cluster: patch, x, y, level; sorted by level
+    int first[SG_CL_LEVELS + 1];  // first charged cluster of each level
+    int nlev, ncl;
+    float *mat;             // device: interpolation matrices
+    int *keys;              // device copy of keys_host: first class of a table, -1 for none
+    int keys_host[SG_NT_STEPS * SG_NT_KEYS];
+    int nclass;
+    bool untabled;          // some pair of levels has no table (corner form)
+    sg_near_tab tab, ptab;  // force (or off-plane force); potential (built at its first call)
 };
 
 struct sg_patch_plan {
@@ -262,8 +294,9 @@ struct sg_plan {
     // cross-patch direct sum
     int ntiles;
     sg_tile_desc *tiles;            // device
-    int nsplit;                     // source-tile ranges per target block
-    int far_grid;                   // CTAs of the persistent far-field launch (FP32 plans)
+    int nsplit;                     // source-tile ranges per target block (FP64 plans; 1 in FP32)
+    int far_grid;                   // CTAs of the far-field launch (FP32 plans)
+    sg_far *far;                    // FP32 plans: clusters and near tables (cross32.cu)
     int wait_tries;                 // attempts of the kernels' bounded waits (SG_MBAR_MAX_TRIES by default)
     int ntargets;
     int4 *targets;                  // device: (lattice x, lattice y, output index, patch)
@@ -286,13 +319,12 @@ struct sg_workspace {
     void *work_fwd;         // uniform-transform scratch: 3 x (px/2+1) x ny complex (largest patch)
     void *work_inv;         // 2 x (px/2+1) x ny complex
     void *sfield;           // AMR composite source fields, 3 x ncells of T
-    void *tile_w;           // AMR corner weights (FP64 plans) or cell coefficients (FP32 plans),
-                            // ntiles x SG_TILE_N x 4 of T
+    void *tile_w;           // AMR corner weights (FP64 plans: ntiles x SG_TILE_N x 4) or cluster
+                            // charges (FP32 plans: 64 per charged cluster)
     double *partial;        // AMR direct-sum partial sums: nsplit x ntargets x 2 (FP64 plans, nsplit > 1);
-                            // (nsplit + 1) x ntargets x 2, the last slice the near field (FP32 plans)
+                            // the near field, ntargets x 2 or 3 (FP32 plans)
     void *zone_buf;         // zone plans: inputs (3 planes) and outputs (2 planes) in patch layout
-    int *err;               // device words: err[0] nonzero after a bounded wait in a kernel ran out;
-                            // err[1] the work-item counter of the persistent far-field launch
+    int *err;               // device word: err[0] nonzero after a bounded wait in a kernel ran out
     struct sg_timing *timing;  // stage timers, or NULL
 };
 
@@ -344,8 +376,19 @@ sg_status sg_potential_spectra_build(sg_plan *plan);   // synchronous, every pat
 void sg_tune_shape(sg_precision prec, int pad, int *shape);
 sg_status sg_cross_solve(sg_plan *plan, const struct sg_workspace *ws, const void *sigma, const void *dx, const void *dy,
                          void *fx, void *fy, void *fz, cudaStream_t st);  // fz: z != 0 plans only
-// Grid of the persistent far-field launch of an FP32 plan (sets plan->far_grid).
-sg_status sg_cross_far_grid(sg_plan *plan, int nsm);
+// FP32 plans (cross32.cu): clusters and near tables (codes: per patch the cell
+// codes; level_targets: leaf cells per level; gmax: largest width ratio 2^gmax
+// with near tables), the solves, the tables of the potential (built at its first
+// call, synchronously).
+sg_status sg_far_setup(sg_plan *plan, const int *const *codes, int nlevels, const int64_t *level_targets, int gmax);
+int64_t sg_near_table_bytes(int nlevels, const int64_t *level_targets, double z, int gmax);
+int64_t sg_far_bytes(int64_t nclusters, int64_t ntargets, double z);
+void sg_far_free(sg_plan *plan);
+sg_status sg_far_solve(sg_plan *plan, const struct sg_workspace *ws, const float *sigma, const float *dx, const float *dy,
+                       float *fx, float *fy, float *fz, cudaStream_t st);
+sg_status sg_far_potential_tables(sg_plan *plan);
+sg_status sg_far_potential(sg_plan *plan, const struct sg_workspace *ws, const float *sigma, const float *dx,
+                           const float *dy, float *phi, cudaStream_t st);
 // the potential's cross-patch sum, added into phi (the patches' own convolutions already there)
 sg_status sg_cross_potential(sg_plan *plan, const struct sg_workspace *ws, const void *sigma, const void *dx,
                              const void *dy, void *phi, cudaStream_t st);

@@ -66,34 +66,6 @@ namespace {
 
 // --------------------------------------------------------------- tables --
 
-__device__ __forceinline__ bool line_diff(double t1, double t2, double &out)
-{
-    // sgn(t2) ln|t2| - sgn(t1) ln|t1|; diverges when the span [t1, t2] holds 0
-    if (t1 == 0.0 || t2 == 0.0 || (t1 < 0.0 && t2 > 0.0)) return false;
-    out = (t2 > 0.0 ? log(t2) : -log(-t2)) - (t1 > 0.0 ? log(t1) : -log(-t1));
-    return true;
-}
-
-// x-family of the unit cell centred at (cx, cy), target at the origin.
-__device__ bool unit_x_family(double cx, double cy, double &x0, double &xx, double &xy)
-{
-    const double u1 = cx - 0.5, u2 = cx + 0.5, v1 = cy - 0.5, v2 = cy + 0.5;
-    double d1, d2;
-    if (u1 != 0.0) d1 = asinh_span(v1, v2, fabs(u1));
-    else if (!line_diff(v1, v2, d1)) return false;
-    if (u2 != 0.0) d2 = asinh_span(v1, v2, fabs(u2));
-    else if (!line_diff(v1, v2, d2)) return false;
-    x0 = d1 - d2;
-    const double g2 = v2 != 0.0 ? v2 * asinh_span(u1, u2, fabs(v2)) : 0.0;
-    const double g1 = v1 != 0.0 ? v1 * asinh_span(u1, u2, fabs(v1)) : 0.0;
-    xx = -cx * x0 + (g2 - g1);
-    const double r22 = sqrt(u2 * u2 + v2 * v2), r12 = sqrt(u1 * u1 + v2 * v2);
-    const double r21 = sqrt(u2 * u2 + v1 * v1), r11 = sqrt(u1 * u1 + v1 * v1);
-    const double ddr = (u2 + u1) / (r22 + r12) - (u2 + u1) / (r21 + r11);
-    xy = -cy * x0 - ddr;
-    return true;
-}
-
 // Packed wrapped tables of one kernel key: z0 = Kr^x0 + i Kr^y0, z1 = Kr^xx + i Kr^xy,
 // z2 = Kr^yy + i Kr^yx, each [py][px], for a source cell w = 2^s finest cells wide
 // and sample shift d = d2 / 2: Kr[e] = K(centre offset -e - d). The stored period
