@@ -54,8 +54,8 @@
 //
 // The direct sum over all pairs that this replaces cost 17.3 ms (far) + 8.9 ms
 // (near, FP64 pipe) on three nested 256^2 levels. Measured per solve: six nested
-// 256^2 levels 121.5 -> 4.83 ms, three off the plane 50.4 -> 1.89 ms, with the same
-// error against FP64 (3.5e-7, 1.2e-7).
+// 256^2 levels 121.5 -> 3.74 ms, three off the plane 50.4 -> 1.64 ms; error against
+// FP64 3.5e-7 -> 1.6e-7 and 1.3e-7 -> 7e-8.
 #include "common.cuh"
 #include "kmath.cuh"
 
@@ -64,6 +64,7 @@
 
 #include <algorithm>
 #include <new>
+#include <utility>
 #include <vector>
 
 namespace {
@@ -404,7 +405,9 @@ struct far_args {
 // first (the finest patches, with the most coarser cells near them, first).
 // Bound by FP32 issue (middle cells: 62 operations each) and the special-function
 // unit (far field). Six nested 256^2 levels: 1.9e9 block-point evaluations, 0.2e9
-// at targets, 1.0e9 middle pairs in 3.8 ms; three off the plane 1.49 ms.
+// at targets and 1.0e9 middle pairs, of which half on the block's points (a quarter
+// of the work): 2.7 ms, 3.8 with every middle cell on the targets; three levels off
+// the plane 1.25 against 1.49 ms.
 template <int Q>
 __global__ void __launch_bounds__(256, 3) k_far(far_args A)
 {
@@ -477,48 +480,67 @@ __global__ void __launch_bounds__(256, 3) k_far(far_args A)
                 if (!some) break;
             }
             if (pi0 > pi1 || pj0 > pj1) continue;
-            // the cells of the near level-0 clusters, 256 at a time
-            const int i0 = CL * pi0, i1 = min(p.nx, CL * (pi1 + 1)), j0 = CL * pj0, j1 = min(p.ny, CL * (pj1 + 1));
-            const int L = p.step, w = i1 - i0, total = w * (j1 - j0);
+            // the cells of the near level-0 clusters, in two passes: those whose field is
+            // smooth over the block (two block widths from its centre, and no target's near
+            // cell) on the block's points, a quarter per group of threads; the others on the targets
+            const int L = p.step;
+            const int i0 = CL * pi0, i1 = min(p.nx, CL * (pi1 + 1)) - 1, j0 = CL * pj0, j1 = min(p.ny, CL * (pj1 + 1)) - 1;
+            const int M2 = max(4 * b2 + L, 2 * SG_NEAR_R * L + b2);  // twice the distance, doubled
+            const int ii0 = max(i0, floor_div(-(int64_t)M2 - ox2 - L, 2 * L) + 1), ii1 = min(i1, -floor_div(-((int64_t)M2 - ox2 - L), 2 * L) - 1);
+            const int ij0 = max(j0, floor_div(-(int64_t)M2 - oy2 - L, 2 * L) + 1), ij1 = min(j1, -floor_div(-((int64_t)M2 - oy2 - L), 2 * L) - 1);
+            const bool inner = ii0 <= ii1 && ij0 <= ij1;
             const float invL = 1.f / (float)L;  // a power of two: exact
-            const float ux = tx * invL, uy = ty * invL;
             const double h8 = L * A.lambda * 0.125;
             const float zeta = Q == Q_OFF ? (float)(A.zl / (double)L) : 0.f;
-            for (int e0 = 0; e0 < total; e0 += 256) {
-                const int e = e0 + tid;
-                __syncthreads();  // the previous cells have been used
-                if (e < total) {
-                    const int jr = e / w, i = i0 + e - jr * w, j = j0 + jr;
-                    const int64_t o = p.cell_off + (int64_t)j * p.nx + i;
-                    mc[tid] = make_float4(A.sigma[o], (float)((double)A.dx[o] * h8), (float)((double)A.dy[o] * h8), 0.f);
-                    mp[tid] = make_float2(0.5f * (float)(ox2 + (2 * i + 1) * L) * invL,
-                                          0.5f * (float)(oy2 + (2 * j + 1) * L) * invL);
+            for (int pass = 0; pass < 2; ++pass) {
+                const bool outer = pass == 0;
+                if (outer && inner && ii0 == i0 && ii1 == i1 && ij0 == j0 && ij1 == j1) continue;
+                if (!outer && !inner) continue;
+                const int a0 = outer ? i0 : ii0, b0 = outer ? j0 : ij0;
+                const int w = (outer ? i1 : ii1) - a0 + 1, total = w * ((outer ? j1 : ij1) - b0 + 1);
+                const float ux = (outer ? px : tx) * invL, uy = (outer ? py : ty) * invL;
+                for (int e0 = 0; e0 < total; e0 += 256) {
+                    const int e = e0 + tid;
+                    __syncthreads();  // the previous cells have been used
+                    if (e < total) {
+                        const int jr = e / w, i = a0 + e - jr * w, j = b0 + jr;
+                        const int64_t o = p.cell_off + (int64_t)j * p.nx + i;
+                        float4 c = make_float4(0.f, 0.f, 0.f, 0.f);
+                        if (!(outer && inner && i >= ii0 && i <= ii1 && j >= ij0 && j <= ij1))
+                            c = make_float4(A.sigma[o], (float)((double)A.dx[o] * h8), (float)((double)A.dy[o] * h8), 0.f);
+                        mc[tid] = c;
+                        mp[tid] = make_float2(0.5f * (float)(ox2 + (2 * i + 1) * L) * invL,
+                                              0.5f * (float)(oy2 + (2 * j + 1) * L) * invL);
+                    }
+                    __syncthreads();
+                    if (!outer && (tid & ~31) >= blk.count) continue;  // no target in this warp
+                    const int nc = min(256, total - e0), dc = outer ? 4 : 1;
+                    float s[NO];
+#pragma unroll
+                    for (int o = 0; o < NO; ++o) s[o] = 0.f;
+                    for (int c = outer ? grp : 0; c < nc; c += dc) {
+                        const float4 cc = mc[c];
+                        if (cc.x == 0.f && cc.y == 0.f && cc.z == 0.f) continue;  // no density (the same in the warp)
+                        const float a = mp[c].x - ux, b = mp[c].y - uy;  // at targets exact: half-cell multiples
+                        const bool nearc = fabsf(a) < (float)SG_NEAR_R && fabsf(b) < (float)SG_NEAR_R;
+                        float t[NO];
+#pragma unroll
+                        for (int o = 0; o < NO; ++o) t[o] = s[o];
+                        if constexpr (Q == Q_FORCE) cell_far(a, b, cc, t[0], t[1]);
+                        else if constexpr (Q == Q_POT) t[0] += cell_far_pot(a, b, cc);
+                        else cell_far_z(a, b, zeta * zeta, cc, t[0], t[1], t[2]);
+#pragma unroll
+                        for (int o = 0; o < NO; ++o) s[o] = nearc ? s[o] : t[o];
+                    }
+                    if constexpr (Q == Q_FORCE) s[1] = -s[1];    // Q = Fx - i Fy
+                    if constexpr (Q == Q_POT) s[0] *= (float)L;  // per lattice unit
+                    if constexpr (Q == Q_OFF) s[2] *= -zeta;
+#pragma unroll
+                    for (int o = 0; o < NO; ++o) {
+                        if (outer) add2(nh[o], nl[o], s[o]);
+                        else add2(th[o], tl[o], s[o]);
+                    }
                 }
-                __syncthreads();
-                if ((tid & ~31) >= blk.count) continue;  // no target in this warp
-                const int nc = min(256, total - e0);
-                float s[NO];
-#pragma unroll
-                for (int o = 0; o < NO; ++o) s[o] = 0.f;
-                for (int c = 0; c < nc; ++c) {
-                    const float4 cc = mc[c];
-                    const float a = mp[c].x - ux, b = mp[c].y - uy;  // exact: half-cell multiples
-                    if (cc.x == 0.f && cc.y == 0.f && cc.z == 0.f) continue;  // no density (the same in every thread)
-                    const bool nearc = fabsf(a) < (float)SG_NEAR_R && fabsf(b) < (float)SG_NEAR_R;
-                    float t[NO];
-#pragma unroll
-                    for (int o = 0; o < NO; ++o) t[o] = s[o];
-                    if constexpr (Q == Q_FORCE) cell_far(a, b, cc, t[0], t[1]);
-                    else if constexpr (Q == Q_POT) t[0] += cell_far_pot(a, b, cc);
-                    else cell_far_z(a, b, zeta * zeta, cc, t[0], t[1], t[2]);
-#pragma unroll
-                    for (int o = 0; o < NO; ++o) s[o] = nearc ? s[o] : t[o];
-                }
-                if constexpr (Q == Q_FORCE) s[1] = -s[1];      // Q = Fx - i Fy
-                if constexpr (Q == Q_POT) s[0] *= (float)L;    // per lattice unit
-                if constexpr (Q == Q_OFF) s[2] *= -zeta;
-#pragma unroll
-                for (int o = 0; o < NO; ++o) add2(th[o], tl[o], s[o]);
             }
         }
         // the field at the block's points, then its interpolation to the targets:
@@ -604,18 +626,32 @@ __host__ __device__ __forceinline__ int near_first(int f, int g)
     return g >= 0 && 2 * f + 1 > (1 << g) ? -SG_NEAR_R + 1 : -SG_NEAR_R;
 }
 
-// One near table: the closed-form integrals of the 12 x 12 cells around one
-// position (fx, fy), scaled, in two FP32 parts, [plane][cell]; zero outside the
-// near box and where the integral diverges (a target on a corner or inside an
-// edge of a cell: never a leaf target with a cell that carries density).
+// The tables to build: key k holds the classes first[k] .. first[k + 1] for cells
+// of width H[k] and ratio exponent g[k].
+struct near_list {
+    int n;
+    int first[SG_NT_STEPS * SG_NT_KEYS + 1];
+    int g[SG_NT_STEPS * SG_NT_KEYS];
+    double H[SG_NT_STEPS * SG_NT_KEYS];
+};
+
+// Near tables, every key in one launch (the smallest have 144 entries, whose FP64
+// latency alone is 0.1 ms: one launch per key added 2.7 ms to a plan of six levels):
+// the closed-form integrals of the 12 x 12 cells around each position (fx, fy),
+// scaled, in two FP32 parts, [plane][cell]; zero outside the near box and where
+// the integral diverges (a target on a corner or inside an edge of a cell: never a
+// leaf target with a cell that carries density).
 template <int Q>
-__global__ void k_near_table(float2 *__restrict__ out, int g, double H, double G, double zeta)
+__global__ void k_near_table(float2 *__restrict__ out, near_list L, double G, double z)
 {
-    const int ncls = g < 0 ? 1 : 1 << (2 * g);
-    const int64_t total = (int64_t)ncls * NEAR_CELLS;
+    const int64_t total = (int64_t)L.first[L.n] * NEAR_CELLS;
     for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
         const int cls = (int)(e / NEAR_CELLS), c = (int)(e % NEAR_CELLS);
-        const int fx = g < 0 ? 0 : cls & ((1 << g) - 1), fy = g < 0 ? 0 : cls >> g;
+        int k0 = 0;
+        while (cls >= L.first[k0 + 1]) ++k0;
+        const int g = L.g[k0], pos = cls - L.first[k0];
+        const double H = L.H[k0];
+        const int fx = g < 0 ? 0 : pos & ((1 << g) - 1), fy = g < 0 ? 0 : pos >> g;
         const double w = g < 0 ? 0.0 : 1.0 / (double)(1 << g);
         const double cx = near_first(fx, g) + c % NEAR_BOX + 0.5 - (g < 0 ? 0.0 : (fx + 0.5) * w);
         const double cy = near_first(fy, g) + c / NEAR_BOX + 0.5 - (g < 0 ? 0.0 : (fy + 0.5) * w);
@@ -628,7 +664,7 @@ __global__ void k_near_table(float2 *__restrict__ out, int g, double H, double G
                 v[1] *= -G * H * H;
                 v[2] *= -G * H * H;
             } else if constexpr (Q == Q_OFF) {
-                unit_cell_offplane(cx, cy, zeta, v);
+                unit_cell_offplane(cx, cy, z / H, v);
                 for (int k = 0; k < 9; ++k) v[k] *= k % 3 == 0 ? G : G * H;
             } else {
                 // unit_x_family: K^{x,0}, K^{x,x}, K^{x,y} at (cx, cy); the y family by exchange
@@ -927,17 +963,24 @@ sg_status build_tables(sg_plan *plan, sg_near_tab &nt)
         return e == cudaErrorMemoryAllocation ? SG_ENOMEM : SG_ECUDA;
     }
     plan->device_bytes += (int64_t)bytes;
-    for (int s = 0; s < SG_NT_STEPS; ++s)
-        for (int g = -1; g <= SG_NT_GMAX; ++g) {
-            const int key = F.keys_host[s * SG_NT_KEYS + g + 1];
-            if (key < 0) continue;
-            const double H = (double)(1LL << s) * plan->lattice_unit;
-            const int64_t n = (g < 0 ? 1LL : 1LL << (2 * g)) * NEAR_CELLS;
-            const int grid = (int)std::min<int64_t>((n + 127) / 128, 4096);
-            k_near_table<Q><<<grid, 128>>>((float2 *)((char *)nt.data + (size_t)key * cls), g, H, plan->geom.G,
-                                           plan->geom.z / H);
-            SG_CUDA_TRY(cudaGetLastError());
-        }
+    // the keys in the order of their classes
+    near_list L;
+    memset(&L, 0, sizeof(L));
+    std::vector<std::pair<int, int>> order;  // first class, key
+    for (int k = 0; k < SG_NT_STEPS * SG_NT_KEYS; ++k)
+        if (F.keys_host[k] >= 0) order.push_back({F.keys_host[k], k});
+    std::sort(order.begin(), order.end());
+    for (const auto &o : order) {
+        L.first[L.n] = o.first;
+        L.g[L.n] = o.second % SG_NT_KEYS - 1;
+        L.H[L.n] = (double)(1LL << (o.second / SG_NT_KEYS)) * plan->lattice_unit;
+        ++L.n;
+    }
+    L.first[L.n] = F.nclass;
+    if (F.nclass == 0) return SG_OK;
+    const int grid = (int)std::min<int64_t>(((int64_t)F.nclass * NEAR_CELLS + 127) / 128, 1 << 16);
+    k_near_table<Q><<<grid, 128>>>((float2 *)nt.data, L, plan->geom.G, plan->geom.z);
+    SG_CUDA_TRY(cudaGetLastError());
     return SG_OK;
 }
 
