@@ -125,7 +125,7 @@ typedef struct {
     int64_t cross_pairs;        /* leaf-target x leaf-source pairs summed directly */
     int64_t device_bytes;       /* device memory held by the plan now */
     int64_t scratch_bytes;      /* per-call scratch (workspace) of one solve */
-    int max_pad;                /* largest padded FFT length */
+    int max_pad;                /* largest padded FFT length, rounded up to a power of two */
     int64_t nzones;             /* zones of a plan made by sg_plan_create_zones, else 0 */
     int launches;               /* kernels one sg_force (sg_force_zones for zone plans) enqueues */
     int cross_mode;             /* the path chosen: SG_CROSS_DIRECT or SG_CROSS_LEVELS (0 for a
@@ -440,7 +440,8 @@ sg_status sg_zones_links(const sg_zones *zones, int64_t *parent, uint8_t *leaf, 
  * three compiled launch shapes per padded length: half, the measured default
  * and twice the default number of row sequences (forward and inverse row
  * passes) or columns (column passes) per CTA, where shared memory and CTA size
- * allow. A process-wide table, initially the defaults, selects one per
+ * allow (lengths 5/4 and 3/2 of a power of two, from 320 on, have one shape).
+ * A process-wide table, initially the defaults, selects one per power-of-two
  * (precision, padded length); results are bit-identical under every shape
  * (only the grouping of sequences into CTAs changes). Solves read the table
  * when they enqueue (a graph captures the shapes in force at capture).

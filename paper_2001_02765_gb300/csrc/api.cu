@@ -532,8 +532,7 @@ sizes plan_sizes(const sg_geom *g, const geom_info &gi, sg_precision prec, int n
     int64_t work = 0;
     for (int k = 0; k < gi.n; ++k) {
         const int px = sg_pad_length(g->patches[k].nx), py = sg_pad_length(g->patches[k].ny);
-        if (px > s.max_pad) s.max_pad = px;
-        if (py > s.max_pad) s.max_pad = py;
+        s.max_pad = std::max(s.max_pad, sg_pow2_length(std::max(px, py)));
         if (lv_bytes < 0) s.spectra += (g->z != 0.0 ? 9LL : 6LL) * (px / 2 + 1) * sg_spec_stride(py) * (int64_t)es;
         const int64_t w = 5LL * (px / 2 + 1) * g->patches[k].ny * (int64_t)(2 * es);
         if (w > work) work = w;

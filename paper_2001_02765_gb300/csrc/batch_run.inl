@@ -25,6 +25,12 @@ inline int batch_smem(int px, int py)
     case 512: c = batch_col_smem_t<T, 512>(); break;
     case 1024: c = batch_col_smem_t<T, 1024>(); break;
     case 2048: c = batch_col_smem_t<T, 2048>(); break;
+    case 320: c = batch_col_smem_t<T, 320>(); break;
+    case 384: c = batch_col_smem_t<T, 384>(); break;
+    case 640: c = batch_col_smem_t<T, 640>(); break;
+    case 768: c = batch_col_smem_t<T, 768>(); break;
+    case 1280: c = batch_col_smem_t<T, 1280>(); break;
+    case 1536: c = batch_col_smem_t<T, 1536>(); break;
     default: return -1;
     }
     const int r = batch_row_smem<T>(px), e = batch_edge_smem<T>(py);
@@ -96,6 +102,12 @@ __device__ __forceinline__ void batch_run_item(const batch_item &it, const batch
     case 256: batch_item_len<T, 256>(it, m, err); break;
     case 512: batch_item_len<T, 512>(it, m, err); break;
     case 1024: batch_item_len<T, 1024>(it, m, err); break;
+    case 320: batch_item_len<T, 320>(it, m, err); break;
+    case 384: batch_item_len<T, 384>(it, m, err); break;
+    case 640: batch_item_len<T, 640>(it, m, err); break;
+    case 768: batch_item_len<T, 768>(it, m, err); break;
+    case 1280: batch_item_len<T, 1280>(it, m, err); break;
+    case 1536: batch_item_len<T, 1536>(it, m, err); break;
     default: batch_item_len<T, 2048>(it, m, err); break;
     }
 }

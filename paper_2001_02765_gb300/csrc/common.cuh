@@ -104,6 +104,9 @@ struct __align__(32) sg_dvec4 {
 // Largest padded length of the level convolutions (FP32; FP64 stops at SG_MAX_PAD).
 #define SG_LV_MAX_PAD 8192
 #define SG_MIN_PAD 64
+// Smallest power of two B whose multiples 5/4 B and 3/2 B are transform lengths.
+#define SG_SMOOTH_MIN 256
+#define SG_LEN_SLOTS 48
 #define SG_MAX_PATCH_SIDE 2048
 #define SG_MAX_LEVELS 12
 
@@ -244,11 +247,11 @@ struct sg_plan {
     double lattice_unit;            // lambda: half of the finest cell width
     double lattice_x0, lattice_y0;  // physical position of lattice coordinate 0
 
-    // twiddle tables exp(-2 pi i k / L), k < L, for each power of two L in
-    // [SG_MIN_PAD, max_pad]: FP64 copies then FP32 copies, back to back
+    // compact twiddle tables (fft.cuh) of each power of two in [SG_MIN_PAD, max_pad]
+    // and of the patches' other lengths: FP64 copies then FP32 copies, back to back
     void *twiddles;
-    int64_t tw64_off[16];           // byte offsets, indexed by log2 L
-    int64_t tw32_off[16];
+    int64_t tw64_off[SG_LEN_SLOTS];  // byte offsets, indexed by sg_len_index(L)
+    int64_t tw32_off[SG_LEN_SLOTS];
 
     // per cell (device, ncells): SG_CELL_ABSENT, SG_CELL_LEAF, or the index of the
     // child patch that covers the cell
@@ -435,9 +438,33 @@ static inline int sg_lv_cexp(int s, int p)
 // every row starts on a 16-byte boundary (bulk copies need it).
 static inline __host__ __device__ int sg_spec_stride(int py) { return ((py / 2 + 1) + 3) & ~3; }
 
+// Transform lengths of the uniform patches: the powers of two, and from 256 on
+// 5/4 and 3/2 of each (320, 384, 640, 768, ...). With powers of two alone a patch of
+// N cells is padded to 1.44 times 2N - 1 on average (over log N), 2.1 times its area;
+// with the two more lengths per octave to 1.13 times, 1.28 times its area. Below 256
+// points a solve is bound by its launches, and the lengths stay the powers of two.
+static inline __host__ __device__ constexpr bool sg_pow2(int L) { return (L & (L - 1)) == 0; }
+
+static inline int sg_next_length(int L)
+{
+    const int b = sg_pow2(L) ? L : 1 << (sg_ilog2(L) - 1);  // the power of two at or below
+    if (b < SG_SMOOTH_MIN) return 2 * b;
+    return L == b ? b / 4 * 5 : (L == b / 4 * 5 ? b / 2 * 3 : 2 * b);
+}
+
 static inline int sg_pad_length(int n)
 {
     int p = SG_MIN_PAD;
-    while (p < 2 * n - 1) p <<= 1;
+    while (p < 2 * n - 1) p = sg_next_length(p);
     return p;
+}
+
+// The power of two at or above a length.
+static inline int sg_pow2_length(int L) { return 1 << sg_ilog2(L); }
+
+// Slot of a length 2^k, 5 2^k or 3 2^k in the plan's twiddle tables.
+static inline int sg_len_index(int L)
+{
+    const int k = sg_pow2(L) ? sg_ilog2(L) : sg_ilog2(L) - 1, b = 1 << k;
+    return 3 * k + (L == b ? 0 : (L == b / 4 * 5 ? 1 : 2));
 }

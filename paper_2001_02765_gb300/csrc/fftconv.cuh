@@ -1,7 +1,7 @@
 // Kernels of the uniform-patch force as a zero-padded 2-D FFT convolution (introduction and
 // conclusion of Tseng, Shang & Yen; the uniform-grid route of Yen et al. 2012).
 //
-// For a patch of nx x ny cells padded to Px x Py (powers of two, P >= 2n - 1):
+// For a patch of nx x ny cells padded to Px x Py (P >= 2n - 1, see sg_pad_length):
 //   1. k_row_fwd : per row j < ny, the three input fields (sigma0, deltax,
 //                  deltay; the slopes either read or formed by central
 //                  differences on the fly, covered cells masked to zero) are
@@ -223,7 +223,7 @@ __device__ __forceinline__ void row_fwd_body(const row_fwd_args<T> &args, int bx
         if (j >= ny) continue;
         const int s = r >> 1;
         const C z = buf[spad<C>(s * PX + kx)];
-        const C w = buf[spad<C>(s * PX + ((PX - kx) & (PX - 1)))];
+        const C w = buf[spad<C>(s * PX + (kx == 0 ? 0 : PX - kx))];
         C out;
         if ((r & 1) == 0) out = cmake<C>(half * (z.x + w.x), half * (z.y - w.y));
         else out = cmake<C>(half * (z.y + w.y), half * (w.x - z.x));
@@ -252,6 +252,15 @@ __global__ void __launch_bounds__(THREADS) k_row_fwd(row_fwd_args<T> one, const 
 // barrier before each transform's first exchange).
 template <typename T, int PY>
 __host__ __device__ constexpr int col_nbuf() { return sizeof(T) == 8 && PY >= 4096 ? 1 : 2; }
+// Columns per CTA of the column passes: 256 threads for the powers of two up to
+// 2048, one column above; fewer for the lengths 3 2^k and 5 2^k, whose grids fill
+// the SMs sooner that way (a 160^2 solve, 320 points: 11.8 us with 3 columns and 4
+// row sequences per CTA, 16.0 with 6 and 12; 300^2, 640 points: 15.0 against 16.0).
+__host__ __device__ constexpr int col_cb_default(int py)
+{
+    if (!sg_pow2(py)) return py < 512 ? 3 : (py < 768 ? 2 : 1);
+    return py >= 2048 ? 1 : 2048 / py;
+}
 // The central-slope pass kernel on FP32 2048-point columns, one column per CTA,
 // runs four CTAs per SM instead of three (1025 columns in 1.7 waves instead of
 // 2.25): 64 registers (one spilled) and one exchange buffer, so that four CTAs'
@@ -260,6 +269,12 @@ __host__ __device__ constexpr int col_nbuf() { return sizeof(T) == 8 && PY >= 40
 // spills 100 bytes at 64 registers and keeps three.
 template <typename T, int PY, int CB>
 __host__ __device__ constexpr bool col_central_four() { return sizeof(T) == 4 && PY == 2048 && CB == 1; }
+// 768 and 1536 points likewise take 64 registers (both buffers fit): five CTAs of
+// 192 threads at 1536 points (a 700^2 solve 37.4 -> 35.6 us). At 1280 and 2560 the
+// radix-5 stage spills 60 bytes there and the pass is slower (600^2: 34.2 us at 64
+// registers, 30.9 at 80).
+template <typename T, int PY, int CB>
+__host__ __device__ constexpr bool col_central_lean() { return sizeof(T) == 4 && (PY == 768 || PY == 1536); }
 template <typename T, int PY, int CB>
 __host__ __device__ constexpr int col_central_nbuf() { return col_central_four<T, PY, CB>() ? 1 : col_nbuf<T, PY>(); }
 template <typename T, int PY, int CB, int NB = col_nbuf<T, PY>()>
@@ -297,22 +312,33 @@ __device__ __forceinline__ bool spectra_ready(uint64_t *bar, int *err, int tries
     return true;
 }
 
+
 // resident CTAs per SM asked of the register allocator (spill-free choices at
 // the default shapes, scaled by the CTA size for the other candidates). FP32
 // 2048-point columns: the two exchange buffers and six spectrum planes take
 // 59.5 KB of shared memory, so three CTAs fit per SM: 80 registers each (the
 // central-slope pass kernel's four-CTA form, above, overrides this).
+// The other lengths: as many CTAs as leave 80 registers a thread (three outputs
+// and FP64: 128).
 template <typename T, int PY, int NOUT>
 constexpr int col_min_blocks_def()
 {
+    if (!sg_pow2(PY)) return 65536 / ((sizeof(T) == 4 && NOUT < 3 ? 80 : 128) * (col_cb_default(PY) * PY / 8));
     return sizeof(T) == 4 ? (PY == 2048 ? (NOUT == 3 ? 2 : 3) : (PY == 4096 ? 1 : 2)) : 1;
 }
 template <typename T, int PY, int THREADS, int NOUT = 2>
 constexpr int col_min_blocks()
 {
-    constexpr int def_threads = (PY >= 2048 ? 1 : 2048 / PY) * PY / 8;
+    constexpr int def_threads = col_cb_default(PY) * PY / 8;
     constexpr int d = col_min_blocks_def<T, PY, NOUT>();
     return d * def_threads / THREADS >= 1 ? d * def_threads / THREADS : 1;
+}
+template <typename T, int PY, int CB, int THREADS>
+constexpr int col_central_blocks()
+{
+    if (col_central_four<T, PY, CB>()) return 4;
+    if (col_central_lean<T, PY, CB>()) return 65536 / (64 * THREADS);
+    return col_min_blocks<T, PY, THREADS>();
 }
 
 template <typename T, int PY, int CB, int THREADS, int NOUT, bool CO = false>
@@ -328,13 +354,14 @@ __device__ __forceinline__ void col_body(const col_args<T> &args, int bx, int qx
     C *bufs = reinterpret_cast<C *>(smem_raw);
     T *ssp = reinterpret_cast<T *>(smem_raw + col_buf_bytes<T, PY, CB>());
     __shared__ uint64_t bar;
-    static_assert(CB * PY / THREADS == 8, "eight elements per thread");
+    static_assert(CB * PY / 8 <= THREADS, "eight elements per thread");
     constexpr int QS = (PY / 2 + 1 + 3) & ~3;
     constexpr int STEP = PY / 8;
     const int kx0 = bx * CB;
-    // this thread's column and the rows it holds: jt + m PY/8, m = 0..7
+    // this thread's column and the rows it holds: jt + m PY/8, m = 0..7 (threads past
+    // the last column only join the barriers: their column counts as out of range)
     const int c = threadIdx.x / STEP, jt = threadIdx.x % STEP;
-    const int kx = kx0 + c;
+    const int kx = CB * STEP == THREADS || c < CB ? kx0 + c : qx;
     constexpr int NPL = NOUT == 3 ? 9 : (NOUT == 1 ? 3 : 6);
     if (threadIdx.x == 0) mbar_init(&bar, 1);
     __syncthreads();
@@ -536,7 +563,7 @@ __device__ __forceinline__ void edge_body(const edge_args<T> &args, const cplx_t
     const T half = (T)0.5;
     for (int k = threadIdx.x; k < PY; k += THREADS) {
         const C z = buf[spad<C>(k)];
-        const C w = buf[spad<C>((PY - k) & (PY - 1))];
+        const C w = buf[spad<C>(k == 0 ? 0 : PY - k)];
         edge[2 * k] = cmake<C>(half * (z.x + w.x), half * (z.y - w.y));
         edge[2 * k + 1] = cmake<C>(half * (z.y + w.y), half * (w.x - z.x));
     }
@@ -574,12 +601,13 @@ __device__ __forceinline__ void col_central_body(const col_args<T> &args, int bx
     T *ssp = reinterpret_cast<T *>(smem_raw + col_buf_bytes<T, PY, CB>());
     __shared__ uint64_t bar;
     __shared__ C rows[CB][2];  // R0, R1 of each column
-    static_assert(CB * PY / THREADS == 8, "eight elements per thread");
+    static_assert(CB * PY / 8 <= THREADS, "eight elements per thread");
     constexpr int QS = (PY / 2 + 1 + 3) & ~3;
     constexpr int STEP = PY / 8;
     const int kx0 = bx * CB;
+    // (threads past the last column only join the barriers)
     const int c = threadIdx.x / STEP, jt = threadIdx.x % STEP;
-    const int kx = kx0 + c;
+    const int kx = CB * STEP == THREADS || c < CB ? kx0 + c : qx;
     if (threadIdx.x == 0) mbar_init(&bar, 1);
     __syncthreads();
     if (threadIdx.x == 0) fetch_spectra<T, PY, CB, 6, CO>(ssp, spec, kx0, qx, &bar);
@@ -594,10 +622,12 @@ __device__ __forceinline__ void col_central_body(const col_args<T> &args, int bx
         v[m] = (m < 4 && j < ny && kx < qx) ? ld_plain<CO>(&work_fwd[(int64_t)kx * ny + j]) : cmake<C>((T)0, (T)0);
     }
     // the column's first and last rows (read after the transform's barriers)
-    if (jt == 0) rows[c][0] = v[0];
+    if (CB * STEP == THREADS || c < CB) {
+        if (jt == 0) rows[c][0] = v[0];
 #pragma unroll
-    for (int m = 0; m < 4; ++m)
-        if (jt + m * STEP == ny - 1) rows[c][1] = v[m];
+        for (int m = 0; m < 4; ++m)
+            if (jt + m * STEP == ny - 1) rows[c][1] = v[m];
+    }
     int par = 0;
     fft_regs<C, PY, CB, THREADS, col_nbuf<T, PY>(), false>(v, bufs, par, tw);
     if (!spectra_ready(&bar, err, args.tries)) return;
@@ -660,7 +690,7 @@ __device__ __forceinline__ void col_central_body(const col_args<T> &args, int bx
 // same registers, more time waiting on global loads). The batch tests check that
 // the persistent kernel (which runs the body) and this kernel agree bit for bit.
 template <typename T, int PY, int CB, int THREADS, bool BATCH = false>
-__global__ void __launch_bounds__(THREADS, (col_central_four<T, PY, CB>() ? 4 : col_min_blocks<T, PY, THREADS>())) k_col_conv_central(
+__global__ void __launch_bounds__(THREADS, (col_central_blocks<T, PY, CB, THREADS>())) k_col_conv_central(
     col_args<T> one, const col_args<T> *__restrict__ many, int qx, const cplx_t<T> *__restrict__ tw, int *err)
 {
     using C = cplx_t<T>;
@@ -759,15 +789,31 @@ __global__ void __launch_bounds__(THREADS, (col_central_four<T, PY, CB>() ? 4 : 
 
 // Default shapes (measured): row sequences (two rows each) per CTA of the
 // forward and inverse row passes, columns per CTA of the column passes.
-__host__ __device__ constexpr int row_nb_default(int px) { return px >= 4096 ? 2 : (4096 / px < 2 ? 2 : 4096 / px); }
-__host__ __device__ constexpr int row_nb_inv_default(int px) { return px >= 4096 ? 2 : (px == 2048 ? 4 : 4096 / px); }
-__host__ __device__ constexpr int col_cb_default(int py) { return py >= 2048 ? 1 : 2048 / py; }
+// (3 2^k and 5 2^k: small CTAs, see col_cb_default; even, so that a CTA's rows fill
+// whole 32-byte sectors of the transposed spectra)
+__host__ __device__ constexpr int row_nb_default(int px)
+{
+    if (!sg_pow2(px)) return px > 1024 ? 2 : 4;
+    return px >= 4096 ? 2 : (4096 / px < 2 ? 2 : 4096 / px);
+}
+__host__ __device__ constexpr int row_nb_inv_default(int px)
+{
+    if (!sg_pow2(px)) return px > 2048 ? 2 : 4;
+    return px >= 4096 ? 2 : (px == 2048 ? 4 : 4096 / px);
+}
 // Row-pass CTAs of 512 threads: a 1024² solve has only 256 row CTAs per pass,
 // and 512 threads (instead of 256) double the warps per SM; measured 2-3 %
 // faster per solve (potential, off-plane, central slopes), no spills.
 constexpr int ROW_THREADS = 512;
+// The other lengths: one butterfly of the radix-8 stages per thread and round.
+__host__ __device__ constexpr int row_threads(int px, int nb)
+{
+    if (sg_pow2(px)) return ROW_THREADS;
+    const int n = nb * px / 8, r = (n + 511) / 512;
+    return ((n + r - 1) / r + 31) / 32 * 32;
+}
 
-// Candidate shapes: half, the default, and twice the default, where feasible
+// Candidate shapes of the powers of two: half, the default, and twice the default, where feasible
 // (shared memory within 200 KB, 32..512 threads per CTA: 1024 would cap registers at 64).
 __host__ __device__ constexpr int shape_candidate(int def, int k) { return k == 0 ? def / 2 : (k == 1 ? def : 2 * def); }
 template <typename T>
@@ -860,8 +906,8 @@ inline uniform_passes<T> uniform_setup(const sg_plan *plan, const sg_workspace *
     C *wf = pot_spec ? (C *)wf_pot : (C *)ws->work_fwd;
     C *wi = (C *)ws->work_inv;
     const int64_t *twoff = sizeof(T) == 8 ? plan->tw64_off : plan->tw32_off;
-    u.twx = (const C *)((const char *)plan->twiddles + twoff[sg_ilog2(d.px)]);
-    u.twy = (const C *)((const char *)plan->twiddles + twoff[sg_ilog2(d.py)]);
+    u.twx = (const C *)((const char *)plan->twiddles + twoff[sg_len_index(d.px)]);
+    u.twy = (const C *)((const char *)plan->twiddles + twoff[sg_len_index(d.py)]);
     u.central = src.mode == SG_SLOPES_CENTRAL && pp.phase && !pot_spec;
     u.nf_rows = u.central ? 1 : nf;
     u.nf_cols = nf;
@@ -886,6 +932,14 @@ inline uniform_passes<T> uniform_setup(const sg_plan *plan, const sg_workspace *
     case 1024: { constexpr int PP = 1024; CALL; } break; \
     case 2048: { constexpr int PP = 2048; CALL; } break; \
     case 4096: { constexpr int PP = 4096; CALL; } break; \
+    case 320: { constexpr int PP = 320; CALL; } break;   \
+    case 384: { constexpr int PP = 384; CALL; } break;   \
+    case 640: { constexpr int PP = 640; CALL; } break;   \
+    case 768: { constexpr int PP = 768; CALL; } break;   \
+    case 1280: { constexpr int PP = 1280; CALL; } break; \
+    case 1536: { constexpr int PP = 1536; CALL; } break; \
+    case 2560: { constexpr int PP = 2560; CALL; } break; \
+    case 3072: { constexpr int PP = 3072; CALL; } break; \
     default: return SG_EINVAL;                 \
     }
 

@@ -36,10 +36,10 @@ sg_status cols_central_py(int cb, const col_args<T> &one, const col_args<T> *man
     constexpr int D = col_cb_default(PY);
     constexpr int A = shape_candidate(D, 0), C = shape_candidate(D, 2);
     if (cb == D) return launch_cols_central_any<T, PY, D>(one, many, bs, qx, tw, err, st, dep);
-    if constexpr (col_feasible_t<T, PY, A, 6>()) {
+    if constexpr (sg_pow2(PY) && col_feasible_t<T, PY, A, 6>()) {
         if (cb == A) return launch_cols_central_any<T, PY, A>(one, many, bs, qx, tw, err, st, dep);
     }
-    if constexpr (col_feasible_t<T, PY, C, 6>()) {
+    if constexpr (sg_pow2(PY) && col_feasible_t<T, PY, C, 6>()) {
         if (cb == C) return launch_cols_central_any<T, PY, C>(one, many, bs, qx, tw, err, st, dep);
     }
     return SG_EINVAL;
@@ -49,7 +49,7 @@ template <typename T, int PY>
 sg_status launch_edge_cols(const edge_args<T> &one, const edge_args<T> *many, batch_shape bs, const cplx_t<T> *tw,
                            cudaStream_t st)
 {
-    constexpr int THREADS = PY / 8 >= 64 ? PY / 8 : 64;
+    constexpr int THREADS = PY / 8 >= 64 ? (PY / 8 + 31) / 32 * 32 : 64;
     const size_t smem = (size_t)spad_size<cplx_t<T>>(PY) * sizeof(cplx_t<T>);
     // a dependent launch after the row pass (see k_edge_cols)
     if (many) {

@@ -14,12 +14,13 @@ sg_status launch_rows_fwd(const row_fwd_args<T> &one, const row_fwd_args<T> *man
                           const cplx_t<T> *tw, cudaStream_t st)
 {
     const size_t smem = (size_t)spad_size<cplx_t<T>>(NB * PX) * sizeof(cplx_t<T>);
-    auto kern = k_row_fwd<T, PX, NB, ROW_THREADS, BATCH, AFTER_EDGE>;
+    constexpr int THREADS = row_threads(PX, NB);
+    auto kern = k_row_fwd<T, PX, NB, THREADS, BATCH, AFTER_EDGE>;
     SG_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     const int ny = BATCH ? bs.maxny : one.src.ny;
     dim3 grid((ny + 2 * NB - 1) / (2 * NB), nf, BATCH ? bs.nmem : 1);
-    if (AFTER_EDGE) SG_CUDA_TRY(sg_launch_dep(kern, grid, dim3(ROW_THREADS), smem, st, one, many, tw));
-    else kern<<<grid, ROW_THREADS, smem, st>>>(one, many, tw);
+    if (AFTER_EDGE) SG_CUDA_TRY(sg_launch_dep(kern, grid, dim3(THREADS), smem, st, one, many, tw));
+    else kern<<<grid, THREADS, smem, st>>>(one, many, tw);
     SG_CUDA_TRY(cudaGetLastError());
     return SG_OK;
 }
@@ -43,10 +44,10 @@ sg_status rows_fwd_px(int nb, const row_fwd_args<T> &one, const row_fwd_args<T> 
     constexpr int D = row_nb_default(PX);
     constexpr int A = shape_candidate(D, 0), C = shape_candidate(D, 2);
     if (nb == D) return launch_rows_fwd_any<T, PX, D>(one, many, bs, nf, tw, st, after_edge);
-    if constexpr (row_feasible_t<T>(PX, A)) {
+    if constexpr (sg_pow2(PX) && row_feasible_t<T>(PX, A)) {
         if (nb == A) return launch_rows_fwd_any<T, PX, A>(one, many, bs, nf, tw, st, after_edge);
     }
-    if constexpr (row_feasible_t<T>(PX, C)) {
+    if constexpr (sg_pow2(PX) && row_feasible_t<T>(PX, C)) {
         if (nb == C) return launch_rows_fwd_any<T, PX, C>(one, many, bs, nf, tw, st, after_edge);
     }
     return SG_EINVAL;

@@ -11,11 +11,12 @@ sg_status launch_rows_inv(const row_inv_args<T> &one, const row_inv_args<T> *man
                           const cplx_t<T> *tw, cudaStream_t st)
 {
     const size_t smem = (size_t)spad_size<cplx_t<T>>(NB * PX) * sizeof(cplx_t<T>);
-    auto kern = k_row_inv<T, PX, NB, ROW_THREADS, BATCH>;
+    constexpr int THREADS = row_threads(PX, NB);
+    auto kern = k_row_inv<T, PX, NB, THREADS, BATCH>;
     SG_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     const int ny = BATCH ? bs.maxny : one.ny;
     dim3 grid((ny + 2 * NB - 1) / (2 * NB), nout, BATCH ? bs.nmem : 1);
-    SG_CUDA_TRY(sg_launch_dep(kern, grid, dim3(ROW_THREADS), smem, st, one, many, tw));
+    SG_CUDA_TRY(sg_launch_dep(kern, grid, dim3(THREADS), smem, st, one, many, tw));
     SG_CUDA_TRY(cudaGetLastError());
     return SG_OK;
 }
@@ -35,10 +36,10 @@ sg_status rows_inv_px(int nb, const row_inv_args<T> &one, const row_inv_args<T> 
     constexpr int D = row_nb_inv_default(PX);
     constexpr int A = shape_candidate(D, 0), C = shape_candidate(D, 2);
     if (nb == D) return launch_rows_inv_any<T, PX, D>(one, many, bs, nout, tw, st);
-    if constexpr (row_feasible_t<T>(PX, A)) {
+    if constexpr (sg_pow2(PX) && row_feasible_t<T>(PX, A)) {
         if (nb == A) return launch_rows_inv_any<T, PX, A>(one, many, bs, nout, tw, st);
     }
-    if constexpr (row_feasible_t<T>(PX, C)) {
+    if constexpr (sg_pow2(PX) && row_feasible_t<T>(PX, C)) {
         if (nb == C) return launch_rows_inv_any<T, PX, C>(one, many, bs, nout, tw, st);
     }
     return SG_EINVAL;

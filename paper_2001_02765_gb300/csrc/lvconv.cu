@@ -904,7 +904,7 @@ sg_status lv_solve_t(sg_plan *plan, const sg_workspace *ws, void *out0, void *ou
     const sg_lv &lv = *plan->lv;
     const int qx = lv.px / 2 + 1;
     const int64_t *twoff = sizeof(T) == 8 ? plan->tw64_off : plan->tw32_off;
-    auto twid = [&](int L) { return (const C *)((const char *)plan->twiddles + twoff[sg_ilog2(L)]); };
+    auto twid = [&](int L) { return (const C *)((const char *)plan->twiddles + twoff[sg_len_index(L)]); };
     const C *cphx = (const C *)lv.cphase, *cphy = cphx + lv.px + 1;
     C *wf = (C *)ws->work_fwd;
     C *wi = (C *)ws->work_inv;
@@ -1110,8 +1110,8 @@ sg_status sg_lv_setup(sg_plan *plan, const sg_lv_setup_args *a)
         sg_set_last_cuda_error(e, "cudaMalloc");
         return e == cudaErrorMemoryAllocation ? SG_ENOMEM : SG_ECUDA;
     }
-    const double2 *twx = (const double2 *)((const char *)plan->twiddles + plan->tw64_off[sg_ilog2(a->px)]);
-    const double2 *twy = (const double2 *)((const char *)plan->twiddles + plan->tw64_off[sg_ilog2(a->py)]);
+    const double2 *twx = (const double2 *)((const char *)plan->twiddles + plan->tw64_off[sg_len_index(a->px)]);
+    const double2 *twy = (const double2 *)((const char *)plan->twiddles + plan->tw64_off[sg_len_index(a->py)]);
     sg_status st = SG_OK;
     for (int k = 0; k < lv->nkeys && st == SG_OK; ++k) {
         k_lv_tables<<<2048, 256>>>(z, a->px, a->py, lv->key_s[k], lv->key_d2[k]);
@@ -1159,8 +1159,8 @@ sg_status sg_lv_potential_spectra_build(sg_plan *plan)
         sg_set_last_cuda_error(e, "cudaMalloc");
         return e == cudaErrorMemoryAllocation ? SG_ENOMEM : SG_ECUDA;
     }
-    const double2 *twx = (const double2 *)((const char *)plan->twiddles + plan->tw64_off[sg_ilog2(px)]);
-    const double2 *twy = (const double2 *)((const char *)plan->twiddles + plan->tw64_off[sg_ilog2(py)]);
+    const double2 *twx = (const double2 *)((const char *)plan->twiddles + plan->tw64_off[sg_len_index(px)]);
+    const double2 *twy = (const double2 *)((const char *)plan->twiddles + plan->tw64_off[sg_len_index(py)]);
     // Phi = -G sum [sigma0 P^0 + deltax P^x + deltay P^y]: P^0 in units of h_f, P^x, P^y of h_f^2
     const double sc0 = -plan->geom.G * lv->hf, sc1 = -plan->geom.G * lv->hf * lv->hf;
     sg_status st = SG_OK;

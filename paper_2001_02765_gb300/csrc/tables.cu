@@ -30,6 +30,9 @@
 
 #include <math.h>
 
+#include <algorithm>
+#include <vector>
+
 // unit-cell tables for m, n >= 0 (parity applied by the caller)
 struct k3 {
     double x0, xx, xy;
@@ -284,14 +287,16 @@ __global__ void k_extract_spectra(const double2 *z, T *planes, int px, int py, d
 // and radix R, entries W_{NS R}^k = exp(-2 pi i k / (NS R)), k < NS.
 __global__ void k_twiddles(double2 *tw64, float2 *tw32, int L)
 {
-    for (int ns = 8, off = 0; ns < L; off += ns, ns *= 8) {
-        const int span = L / ns >= 8 ? 8 * ns : L;  // NS R
+    for (int ns = stage_radix(L, 1), off = 0; ns < L;) {
+        const int r = stage_radix(L, ns);
         for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < ns; k += gridDim.x * blockDim.x) {
             double s, c;
-            sincospi(-2.0 * (double)k / (double)span, &s, &c);
+            sincospi(-2.0 * (double)k / (double)(ns * r), &s, &c);
             tw64[off + k] = make_double2(c, s);
             tw32[off + k] = make_float2((float)c, (float)s);
         }
+        off += ns;
+        ns *= r;
     }
 }
 
@@ -307,6 +312,7 @@ sg_status sg_fft_lines_fp64(double2 *data, int L, int count, int64_t seq_stride,
             data, seq_stride, elem_stride, tw);                                                               \
         break;
         SG_CASE(64) SG_CASE(128) SG_CASE(256) SG_CASE(512) SG_CASE(1024) SG_CASE(2048) SG_CASE(4096) SG_CASE(8192)
+        SG_CASE(320) SG_CASE(384) SG_CASE(640) SG_CASE(768) SG_CASE(1280) SG_CASE(1536) SG_CASE(2560) SG_CASE(3072)
 #undef SG_CASE
     default:
         return SG_EINVAL;
@@ -316,23 +322,29 @@ sg_status sg_fft_lines_fp64(double2 *data, int L, int count, int64_t seq_stride,
 }
 
 // Compact twiddle tables (see fft.cuh): FP64 for every power of two in
-// [SG_MIN_PAD, max_pad], then FP32 copies of each (read by FP32 plans).
+// [SG_MIN_PAD, max_pad] and the patches' other lengths, then FP32 copies of each
+// (read by FP32 plans).
 sg_status sg_twiddles_build(sg_plan *plan)
 {
+    std::vector<int> lens;
+    for (int L = SG_MIN_PAD; L <= plan->max_pad; L <<= 1) lens.push_back(L);
+    for (int p = 0; p < plan->npatches && !plan->lv; ++p)
+        for (int L : {plan->pp[p].d.px, plan->pp[p].d.py})
+            if (std::find(lens.begin(), lens.end(), L) == lens.end()) lens.push_back(L);
     int64_t off = 0;
-    for (int L = SG_MIN_PAD; L <= plan->max_pad; L <<= 1) {
-        plan->tw64_off[sg_ilog2(L)] = off;
+    for (int L : lens) {
+        plan->tw64_off[sg_len_index(L)] = off;
         off += ((int64_t)stage_table_size(L) * sizeof(double2) + 255) / 256 * 256;
     }
-    for (int L = SG_MIN_PAD; L <= plan->max_pad; L <<= 1) {
-        plan->tw32_off[sg_ilog2(L)] = off;
+    for (int L : lens) {
+        plan->tw32_off[sg_len_index(L)] = off;
         off += ((int64_t)stage_table_size(L) * sizeof(float2) + 255) / 256 * 256;
     }
     SG_CUDA_TRY(cudaMalloc(&plan->twiddles, (size_t)off));
     plan->device_bytes += off;
-    for (int L = SG_MIN_PAD; L <= plan->max_pad; L <<= 1) {
-        double2 *t64 = (double2 *)((char *)plan->twiddles + plan->tw64_off[sg_ilog2(L)]);
-        float2 *t32 = (float2 *)((char *)plan->twiddles + plan->tw32_off[sg_ilog2(L)]);
+    for (int L : lens) {
+        double2 *t64 = (double2 *)((char *)plan->twiddles + plan->tw64_off[sg_len_index(L)]);
+        float2 *t32 = (float2 *)((char *)plan->twiddles + plan->tw32_off[sg_len_index(L)]);
         k_twiddles<<<(L / 8 + 255) / 256, 256>>>(t64, t32, L);
         SG_CUDA_TRY(cudaGetLastError());
     }
@@ -362,8 +374,8 @@ sg_status sg_tables_build(sg_plan *plan)
         if (offplane) k_tables_wrapped_z<<<1024, 256>>>(z, pp.d.nx, pp.d.ny, px, py, plan->geom.z / pp.d.h);
         else k_tables_wrapped<<<1024, 256>>>(z, pp.d.nx, pp.d.ny, px, py);
         if (cudaGetLastError() != cudaSuccess) { st = SG_ECUDA; break; }
-        const double2 *twx = (const double2 *)((const char *)plan->twiddles + plan->tw64_off[sg_ilog2(px)]);
-        const double2 *twy = (const double2 *)((const char *)plan->twiddles + plan->tw64_off[sg_ilog2(py)]);
+        const double2 *twx = (const double2 *)((const char *)plan->twiddles + plan->tw64_off[sg_len_index(px)]);
+        const double2 *twy = (const double2 *)((const char *)plan->twiddles + plan->tw64_off[sg_len_index(py)]);
         for (int q = 0; q < npacked && st == SG_OK; ++q) {
             double2 *zq = z + q * plane;
             st = sg_fft_lines_fp64(zq, px, py, px, 1, twx);       // rows
@@ -479,8 +491,8 @@ static sg_status potential_spectra_patch(sg_plan *plan, int p)
     }
     k_tables_wrapped_pot<<<1024, 256>>>(z, pp.d.nx, pp.d.ny, px, py);
     sg_status st = cudaGetLastError() == cudaSuccess ? SG_OK : SG_ECUDA;
-    const double2 *twx = (const double2 *)((const char *)plan->twiddles + plan->tw64_off[sg_ilog2(px)]);
-    const double2 *twy = (const double2 *)((const char *)plan->twiddles + plan->tw64_off[sg_ilog2(py)]);
+    const double2 *twx = (const double2 *)((const char *)plan->twiddles + plan->tw64_off[sg_len_index(px)]);
+    const double2 *twy = (const double2 *)((const char *)plan->twiddles + plan->tw64_off[sg_len_index(py)]);
     for (int q = 0; q < 2 && st == SG_OK; ++q) {
         st = sg_fft_lines_fp64(z + q * plane, px, py, px, 1, twx);
         if (st == SG_OK) st = sg_fft_lines_fp64(z + q * plane, py, px, 1, px, twy);
