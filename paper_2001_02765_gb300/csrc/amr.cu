@@ -139,8 +139,7 @@ __global__ void k_fill_covered(const sg_patch_dev *__restrict__ gpd, const int *
                                int t1, const T *__restrict__ sigma, const T *__restrict__ dx, const T *__restrict__ dy,
                                T *__restrict__ F)
 {
-    sg_dep_trigger();
-    sg_dep_wait();  // the covered cells of the level above
+    sg_dep_first();  // the covered cells of the level above, or the previous solve
     const patch_table tab = stage_patch_table(gpd, gorder, gcpre, npatches);
     const sg_patch_dev *pd = tab.pd;
     const int *order = tab.order;
@@ -175,8 +174,7 @@ __global__ void k_composite(const sg_patch_dev *__restrict__ gpd, const int *__r
                             const T *__restrict__ sigma, const T *__restrict__ dx, const T *__restrict__ dy,
                             const T *__restrict__ F, T *__restrict__ s)
 {
-    sg_dep_trigger();
-    sg_dep_wait();  // the filled values of the covered cells
+    sg_dep_first();  // the filled values of the covered cells, or the previous solve
     const patch_table tab = stage_patch_table(gpd, gorder, gfpre, n);
     const sg_patch_dev *pd = tab.pd;
     const int *order = tab.order;
@@ -245,6 +243,8 @@ __global__ void k_amr_slopes(const int2 *__restrict__ nb, const int2 *__restrict
                              const T *__restrict__ sigma, const T *__restrict__ F, T *__restrict__ D, int64_t P,
                              int64_t c0, int64_t c1, int step, double lambda)
 {
+    sg_dep_trigger();
+    sg_dep_wait();  // the slopes of the level below, the filled values
     for (int64_t c = c0 + blockIdx.x * (int64_t)blockDim.x + threadIdx.x; c < c1; c += (int64_t)gridDim.x * blockDim.x) {
         if (code[c] != SG_CELL_LEAF) {
             D[c] = D[c + P] = (T)0;
@@ -303,28 +303,17 @@ sg_status prepare_t(sg_plan *plan, const sg_workspace *ws, const void *sigma, co
         const int t0 = plan->comp_lev_first[l], t1 = plan->comp_lev_first[l + 1];
         const int64_t n = plan->comp_cells_host[t1] - plan->comp_cells_host[t0];
         if (n <= 0) continue;
-        // the finest fill reads the caller's fields: an ordinary launch; the next ones depend on it
-        auto kf = k_fill_covered<T>;
-        if (l == lmax - 1)
-            kf<<<grid_for(n), 256, patch_table_bytes(plan->npatches), st>>>(
-                plan->patch_dev, plan->cell_code, plan->comp_order, plan->comp_cells, plan->npatches, t0, t1,
-                (const T *)sigma, sx, sy, F);
-        else
-            SG_CUDA_TRY(sg_launch_dep(kf, dim3(grid_for(n)), dim3(256), patch_table_bytes(plan->npatches), st,
-                                      plan->patch_dev, plan->cell_code, plan->comp_order, plan->comp_cells,
-                                      plan->npatches, t0, t1, (const T *)sigma, sx, sy, F));
+        // (dependent launches all: each waits for the stream's previous kernel at its start)
+        SG_CUDA_TRY(sg_launch_dep(k_fill_covered<T>, dim3(grid_for(n)), dim3(256), patch_table_bytes(plan->npatches), st,
+                                  plan->patch_dev, plan->cell_code, plan->comp_order, plan->comp_cells,
+                                  plan->npatches, t0, t1, (const T *)sigma, sx, sy, F));
         SG_CUDA_TRY(cudaGetLastError());
     }
     if (fill_only) return SG_OK;
     auto kc = k_composite<T>;
-    if (lmax >= 2)  // after the fills of the covered cells
-        SG_CUDA_TRY(sg_launch_dep(kc, dim3(grid_for(plan->comp_items)), dim3(256), patch_table_bytes(plan->npatches),
-                                  st, plan->patch_dev, plan->cell_code, plan->comp_order, plan->comp_item_off,
-                                  plan->npatches, (const T *)sigma, sx, sy, (const T *)F, s));
-    else
-        kc<<<grid_for(plan->comp_items), 256, patch_table_bytes(plan->npatches), st>>>(
-            plan->patch_dev, plan->cell_code, plan->comp_order, plan->comp_item_off, plan->npatches, (const T *)sigma,
-            sx, sy, F, s);
+    SG_CUDA_TRY(sg_launch_dep(kc, dim3(grid_for(plan->comp_items)), dim3(256), patch_table_bytes(plan->npatches), st,
+                              plan->patch_dev, plan->cell_code, plan->comp_order, plan->comp_item_off, plan->npatches,
+                              (const T *)sigma, sx, sy, (const T *)F, s));
     SG_CUDA_TRY(cudaGetLastError());
     return SG_OK;
 }
@@ -344,9 +333,9 @@ sg_status slopes_t(sg_plan *plan, const sg_workspace *ws, const void *sigma, cud
     for (int l = 0; l < plan->comp_depth; ++l) {
         const int64_t c0 = plan->lev_cells[l], c1 = plan->lev_cells[l + 1];
         if (c1 <= c0) continue;
-        k_amr_slopes<T><<<grid_for(c1 - c0), 256, 0, st>>>(plan->slope_nb, plan->cell_pos, plan->cell_code,
-                                                          (const T *)sigma, F, D, P, c0, c1, plan->lev_step[l],
-                                                          plan->lattice_unit);
+        SG_CUDA_TRY(sg_launch_dep(k_amr_slopes<T>, dim3(grid_for(c1 - c0)), dim3(256), 0, st, plan->slope_nb,
+                                  plan->cell_pos, plan->cell_code, (const T *)sigma, F, D, P, c0, c1, plan->lev_step[l],
+                                  plan->lattice_unit));
         SG_CUDA_TRY(cudaGetLastError());
     }
     return SG_OK;

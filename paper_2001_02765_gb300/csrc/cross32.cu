@@ -412,6 +412,8 @@ template <int Q>
 __global__ void __launch_bounds__(256, 3) k_far(far_args A)
 {
     constexpr int NO = q_out<Q>();
+    sg_dep_trigger();
+    sg_dep_wait();  // the charges, the near field, the patches' own results
     __shared__ float4 mc[256];
     __shared__ float2 mp[256];
     __shared__ float nodes[4][NQ][NO][2];
@@ -942,7 +944,7 @@ sg_status solve(sg_plan *plan, const sg_workspace *ws, const float *sigma, const
     A.out[0] = o0;
     A.out[1] = o1;
     A.out[2] = o2;
-    k_far<Q><<<plan->far_grid, 256, 0, st>>>(A);
+    SG_CUDA_TRY(sg_launch_dep(k_far<Q>, dim3(plan->far_grid), dim3(256), 0, st, A));
     SG_CUDA_TRY(cudaGetLastError());
     sg_timing_end(ws, SG_STAGE_DIRECT, st);
     return SG_OK;

@@ -217,6 +217,7 @@ template <typename T>
 __global__ void k_zone_gather(const int64_t *__restrict__ slot, int64_t n, const T *__restrict__ s, const T *__restrict__ dx,
                               const T *__restrict__ dy, T *__restrict__ buf, int64_t ncells)
 {
+    sg_dep_first();
     for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < n; k += (int64_t)gridDim.x * blockDim.x) {
         const int64_t o = slot[k];
         buf[o] = s[k];
@@ -232,6 +233,8 @@ __global__ void k_zone_scatter(const int64_t *__restrict__ slot, const int *__re
                                const T *__restrict__ fxp, const T *__restrict__ fyp, T *__restrict__ fx,
                                T *__restrict__ fy)
 {
+    sg_dep_trigger();
+    sg_dep_wait();
     for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < n; k += (int64_t)gridDim.x * blockDim.x) {
         const int64_t o = slot[k];
         const bool leaf = code[o] == SG_CELL_LEAF;
@@ -244,6 +247,8 @@ template <typename T>
 __global__ void k_zone_scatter1(const int64_t *__restrict__ slot, const int *__restrict__ code, int64_t n,
                                 const T *__restrict__ vp, T *__restrict__ v)
 {
+    sg_dep_trigger();
+    sg_dep_wait();
     for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < n; k += (int64_t)gridDim.x * blockDim.x) {
         const int64_t o = slot[k];
         v[k] = code[o] == SG_CELL_LEAF ? vp[o] : (T)0;
@@ -261,11 +266,13 @@ sg_status potential_zones_t(sg_plan *plan, const void *sigma, const void *dx, co
     const bool caller = plan->geom.slope_mode == SG_SLOPES_CALLER;
     int grid = (int)((plan->nzones + 255) / 256);
     if (grid > 8192) grid = 8192;
-    k_zone_gather<T><<<grid, 256, 0, st>>>(plan->zone_slot, plan->nzones, (const T *)sigma,
-                                           caller ? (const T *)dx : nullptr, caller ? (const T *)dy : nullptr, buf, nc);
+    SG_CUDA_TRY(sg_launch_dep(k_zone_gather<T>, dim3(grid), dim3(256), 0, st, plan->zone_slot, plan->nzones,
+                              (const T *)sigma, caller ? (const T *)dx : nullptr, caller ? (const T *)dy : nullptr,
+                              buf, nc));
     SG_CUDA_TRY(cudaGetLastError());
     SG_TRY(sg_potential(plan, buf, caller ? buf + nc : nullptr, caller ? buf + 2 * nc : nullptr, buf + 3 * nc, st));
-    k_zone_scatter1<T><<<grid, 256, 0, st>>>(plan->zone_slot, plan->cell_code, plan->nzones, buf + 3 * nc, (T *)phi);
+    SG_CUDA_TRY(sg_launch_dep(k_zone_scatter1<T>, dim3(grid), dim3(256), 0, st, plan->zone_slot, plan->cell_code,
+                              plan->nzones, (const T *)(buf + 3 * nc), (T *)phi));
     SG_CUDA_TRY(cudaGetLastError());
     return SG_OK;
 }
@@ -279,12 +286,13 @@ sg_status force_zones_t(sg_plan *plan, const void *sigma, const void *dx, const 
     const bool caller = plan->geom.slope_mode == SG_SLOPES_CALLER;
     int grid = (int)((plan->nzones + 255) / 256);
     if (grid > 8192) grid = 8192;
-    k_zone_gather<T><<<grid, 256, 0, st>>>(plan->zone_slot, plan->nzones, (const T *)sigma,
-                                           caller ? (const T *)dx : nullptr, caller ? (const T *)dy : nullptr, buf, nc);
+    SG_CUDA_TRY(sg_launch_dep(k_zone_gather<T>, dim3(grid), dim3(256), 0, st, plan->zone_slot, plan->nzones,
+                              (const T *)sigma, caller ? (const T *)dx : nullptr, caller ? (const T *)dy : nullptr,
+                              buf, nc));
     SG_CUDA_TRY(cudaGetLastError());
     SG_TRY(sg_force_ws(plan, plan->ws, buf, buf + nc, buf + 2 * nc, buf + 3 * nc, buf + 4 * nc, st));
-    k_zone_scatter<T><<<grid, 256, 0, st>>>(plan->zone_slot, plan->cell_code, plan->nzones, buf + 3 * nc,
-                                            buf + 4 * nc, (T *)fx, (T *)fy);
+    SG_CUDA_TRY(sg_launch_dep(k_zone_scatter<T>, dim3(grid), dim3(256), 0, st, plan->zone_slot, plan->cell_code,
+                              plan->nzones, (const T *)(buf + 3 * nc), (const T *)(buf + 4 * nc), (T *)fx, (T *)fy));
     SG_CUDA_TRY(cudaGetLastError());
     return SG_OK;
 }
