@@ -510,6 +510,9 @@ int choose_nsplit(int nblocks, int ntiles, int nsm, sg_precision prec)
     return s;
 }
 
+// rows of the column pass's output (whole blocks of eight, see fftconv.cuh)
+int64_t inv_rows(int ny) { return (ny + 7) & ~7; }
+
 struct sizes {
     int64_t spectra = 0, twiddles = 0, work = 0, direct = 0, geometry = 0, near = 0;
     int max_pad = SG_MIN_PAD;
@@ -534,7 +537,7 @@ sizes plan_sizes(const sg_geom *g, const geom_info &gi, sg_precision prec, int n
         const int px = sg_pad_length(g->patches[k].nx), py = sg_pad_length(g->patches[k].ny);
         s.max_pad = std::max(s.max_pad, sg_pow2_length(std::max(px, py)));
         if (lv_bytes < 0) s.spectra += (g->z != 0.0 ? 9LL : 6LL) * (px / 2 + 1) * sg_spec_stride(py) * (int64_t)es;
-        const int64_t w = 5LL * (px / 2 + 1) * g->patches[k].ny * (int64_t)(2 * es);
+        const int64_t w = (px / 2 + 1) * (3LL * g->patches[k].ny + 2LL * inv_rows(g->patches[k].ny)) * (int64_t)(2 * es);
         if (w > work) work = w;
     }
     s.work = lv_bytes < 0 ? work : lv_bytes;
@@ -799,7 +802,8 @@ sg_status plan_build(const sg_geom *g, sg_precision prec, size_t budget, sg_plan
         const int64_t f = central ? q + (2LL * pdev[k].py + 1) * (int64_t)(2 * es) : 3 * q;  // edge pairs, even start
         const int nout = g->z != 0.0 ? 3 : 2;
         if (f > wf) wf = f;
-        if (nout * q > wi) wi = nout * q;
+        const int64_t i = nout * (int64_t)(pdev[k].px / 2 + 1) * inv_rows(pdev[k].ny) * (int64_t)(2 * es);
+        if (i > wi) wi = i;
     }
     plan->ws_fwd_bytes = wf;
     plan->ws_inv_bytes = wi;

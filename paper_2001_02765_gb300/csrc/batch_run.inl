@@ -7,7 +7,7 @@ namespace sgk {
 
 // dynamic shared memory of one item of each kind at padded length p
 template <typename T>
-__host__ __device__ constexpr int batch_row_smem(int) { return spad_size<cplx_t<T>>(BATCH_MAX_PAD) * (int)sizeof(cplx_t<T>); }
+__host__ __device__ constexpr int batch_row_smem(int p) { return row_smem_bytes<T>(p, batch_nb(p), BATCH_THREADS); }
 template <typename T>
 __host__ __device__ constexpr int batch_edge_smem(int p) { return spad_size<cplx_t<T>>(p) * (int)sizeof(cplx_t<T>); }
 

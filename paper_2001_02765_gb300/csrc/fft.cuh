@@ -254,7 +254,7 @@ __device__ __forceinline__ void twiddle_powers(C *v, C w1)
 // IN_HALF: the first stage takes the inputs at logical positions >= L/2 as
 // zero without reading them (zero padding to at least twice the data length).
 // OUT_HALF: the last stage writes only the outputs at positions < L/2.
-template <typename C, int L, int NB, int THREADS, int NS, int R, bool INV, bool IN_HALF = false, bool OUT_HALF = false>
+template <typename C, int L, int NB, int THREADS, int NS, int R, bool INV, bool IN_HALF, bool OUT_HALF, int SEQ>
 __device__ __forceinline__ void fft_stage(C *buf, const C *__restrict__ tw)
 {
     constexpr int NBF = NB * (L / R);            // butterflies in the stage
@@ -269,12 +269,12 @@ __device__ __forceinline__ void fft_stage(C *buf, const C *__restrict__ tw)
         const int b = threadIdx.x + p * THREADS;
         if (NBF % THREADS == 0 || b < NBF) {
             const int seq = b / S, j = b % S;
-            const C *src = buf + spad<C>(seq * L + j);
+            const C *src = buf + seq * SEQ;
 #pragma unroll
             for (int r = 0; r < R; ++r) {
                 if (IN_HALF && NS == 1 && r >= R / 2) v[p][r] = cmake<C>(0, 0);
-                else if constexpr (SPAN_IN) v[p][r] = src[r * spad<C>(S)];
-                else v[p][r] = buf[spad<C>(seq * L + j + r * S)];
+                else if constexpr (SPAN_IN) v[p][r] = src[spad<C>(j) + r * spad<C>(S)];
+                else v[p][r] = src[spad<C>(j + r * S)];
             }
         }
     }
@@ -287,27 +287,27 @@ __device__ __forceinline__ void fft_stage(C *buf, const C *__restrict__ tw)
             const int k = j % NS;
             if constexpr (NS > 1) twiddle_powers<C, R>(v[p], twiddle<C, INV>(tw, stage_table_offset(L, NS) + k));
             dft<C, R, INV>(v[p]);
-            const int base = seq * L + (j / NS) * NS * R + k;
+            const int base = (j / NS) * NS * R + k;
             constexpr bool SPAN_OUT = NS % spad_group<C>() == 0;
-            C *dst = buf + spad<C>(base);
+            C *dst = buf + seq * SEQ;
 #pragma unroll
             for (int r = 0; r < R; ++r) {
                 if (OUT_HALF && NS * R == L && r >= R / 2) continue;  // position k + r NS >= L/2
-                if constexpr (SPAN_OUT) dst[r * spad<C>(NS)] = v[p][r];
-                else buf[spad<C>(base + r * NS)] = v[p][r];
+                if constexpr (SPAN_OUT) dst[spad<C>(base) + r * spad<C>(NS)] = v[p][r];
+                else dst[spad<C>(base + r * NS)] = v[p][r];
             }
         }
     }
     __syncthreads();
 }
 
-template <typename C, int L, int NB, int THREADS, int NS, bool INV, bool IN_HALF, bool OUT_HALF>
+template <typename C, int L, int NB, int THREADS, int NS, bool INV, bool IN_HALF, bool OUT_HALF, int SEQ>
 __device__ __forceinline__ void fft_stages(C *buf, const C *__restrict__ tw)
 {
     if constexpr (NS < L) {
         constexpr int R = stage_radix(L, NS);
-        fft_stage<C, L, NB, THREADS, NS, R, INV, IN_HALF, OUT_HALF>(buf, tw);
-        fft_stages<C, L, NB, THREADS, NS * R, INV, IN_HALF, OUT_HALF>(buf, tw);
+        fft_stage<C, L, NB, THREADS, NS, R, INV, IN_HALF, OUT_HALF, SEQ>(buf, tw);
+        fft_stages<C, L, NB, THREADS, NS * R, INV, IN_HALF, OUT_HALF, SEQ>(buf, tw);
     }
 }
 
@@ -315,11 +315,13 @@ __device__ __forceinline__ void fft_stages(C *buf, const C *__restrict__ tw)
 // Must be called by every thread of the CTA (it synchronises). The caller
 // synchronises before the call so that the inputs are visible. With IN_HALF
 // the inputs at positions >= L/2 are taken as zero (and need not be written);
-// with OUT_HALF only the outputs at positions < L/2 are produced.
-template <typename C, int L, int NB, int THREADS, bool INV, bool IN_HALF = false, bool OUT_HALF = false>
+// with OUT_HALF only the outputs at positions < L/2 are produced. SEQ: elements
+// from one sequence to the next (default: back to back, spad(s L + k) = s spad(L) + spad(k)).
+template <typename C, int L, int NB, int THREADS, bool INV, bool IN_HALF = false, bool OUT_HALF = false,
+          int SEQ = spad<C>(L)>
 __device__ __forceinline__ void fft_batch(C *buf, const C *__restrict__ tw)
 {
-    fft_stages<C, L, NB, THREADS, 1, INV, IN_HALF, OUT_HALF>(buf, tw);
+    fft_stages<C, L, NB, THREADS, 1, INV, IN_HALF, OUT_HALF, SEQ>(buf, tw);
 }
 
 // ------------------------------------------------- register-resident form --
@@ -348,7 +350,7 @@ __device__ __forceinline__ void fft_batch(C *buf, const C *__restrict__ tw)
 // threads of a sequence: its inputs and outputs go through the exchanges anyway,
 // so a thread takes butterflies jt, jt + L/8, ... below L/R. Threads beyond
 // NSEQ L / 8 only join the barriers.
-template <typename C, int L, int NSEQ, int THREADS, int NS, int NBUF, bool INV>
+template <typename C, int L, int NSEQ, int THREADS, int NS, int NBUF, bool INV, int SEQ>
 __device__ __forceinline__ void rfft_stages(C (&v)[8], C *bufs, int &par, const C *__restrict__ tw)
 {
     static_assert(THREADS >= NSEQ * L / 8, "eight elements per thread");
@@ -357,7 +359,7 @@ __device__ __forceinline__ void rfft_stages(C (&v)[8], C *bufs, int &par, const 
         constexpr bool EVEN = 8 % R == 0;    // whole butterflies of the thread's eight elements
         constexpr int PER = (8 + R - 1) / R;
         constexpr int S = L / R;
-        constexpr int BUF = spad_size<C>(NSEQ * L);
+        constexpr int BUF = SEQ == spad<C>(L) ? spad_size<C>(NSEQ * L) : NSEQ * SEQ;
         constexpr bool ALL = THREADS == NSEQ * L / 8;
         const int seq = threadIdx.x / (L / 8), jt = threadIdx.x % (L / 8);
         const bool live = ALL || seq < NSEQ;
@@ -371,16 +373,16 @@ __device__ __forceinline__ void rfft_stages(C (&v)[8], C *bufs, int &par, const 
                 if (!(live && j < S)) continue;
                 C u[R];
 #pragma unroll
-                for (int r = 0; r < R; ++r) u[r] = in[spad<C>(seq * L + j + r * S)];
+                for (int r = 0; r < R; ++r) u[r] = in[seq * SEQ + spad<C>(j + r * S)];
                 twiddle_powers<C, R>(u, twiddle<C, INV>(tw, stage_table_offset(L, NS) + j % NS));
                 dft<C, R, INV>(u);
-                const int base = seq * L + (j / NS) * NS * R + j % NS;
+                const int base = (j / NS) * NS * R + j % NS;
 #pragma unroll
-                for (int r = 0; r < R; ++r) out[spad<C>(base + r * NS)] = u[r];
+                for (int r = 0; r < R; ++r) out[seq * SEQ + spad<C>(base + r * NS)] = u[r];
             }
             __syncthreads();
             par ^= 1;
-            rfft_stages<C, L, NSEQ, THREADS, NS * R, NBUF, INV>(v, bufs, par, tw);
+            rfft_stages<C, L, NSEQ, THREADS, NS * R, NBUF, INV, SEQ>(v, bufs, par, tw);
             return;
         }
         C u[PER * R];
@@ -396,7 +398,7 @@ __device__ __forceinline__ void rfft_stages(C (&v)[8], C *bufs, int &par, const 
                 const int j = jt + p * (L / 8);
                 if (!(live && (EVEN || j < S))) continue;
 #pragma unroll
-                for (int r = 0; r < R; ++r) u[p * R + r] = in[spad<C>(seq * L + j + r * S)];
+                for (int r = 0; r < R; ++r) u[p * R + r] = in[seq * SEQ + spad<C>(j + r * S)];
             }
             if constexpr (NBUF == 1) __syncthreads();
         }
@@ -421,13 +423,13 @@ __device__ __forceinline__ void rfft_stages(C (&v)[8], C *bufs, int &par, const 
             for (int p = 0; p < PER; ++p) {
                 const int j = jt + p * (L / 8);
                 if (!(live && (EVEN || j < S))) continue;
-                const int base = seq * L + (j / NS) * NS * R + j % NS;
+                const int base = (j / NS) * NS * R + j % NS;
 #pragma unroll
-                for (int r = 0; r < R; ++r) out[spad<C>(base + r * NS)] = u[p * R + r];
+                for (int r = 0; r < R; ++r) out[seq * SEQ + spad<C>(base + r * NS)] = u[p * R + r];
             }
             __syncthreads();
             if constexpr (NBUF == 2) par ^= 1;
-            rfft_stages<C, L, NSEQ, THREADS, NS * R, NBUF, INV>(v, bufs, par, tw);
+            rfft_stages<C, L, NSEQ, THREADS, NS * R, NBUF, INV, SEQ>(v, bufs, par, tw);
         }
     }
 }
@@ -436,8 +438,8 @@ __device__ __forceinline__ void rfft_stages(C (&v)[8], C *bufs, int &par, const 
 // thread of the CTA calls it. bufs: NBUF buffers of spad_size(NSEQ L) elements.
 // With NBUF = 1 the caller must make sure that no thread still reads the
 // buffer from an earlier use when this call starts writing it.
-template <typename C, int L, int NSEQ, int THREADS, int NBUF, bool INV>
+template <typename C, int L, int NSEQ, int THREADS, int NBUF, bool INV, int SEQ = spad<C>(L)>
 __device__ __forceinline__ void fft_regs(C (&v)[8], C *bufs, int &par, const C *__restrict__ tw)
 {
-    rfft_stages<C, L, NSEQ, THREADS, 1, NBUF, INV>(v, bufs, par, tw);
+    rfft_stages<C, L, NSEQ, THREADS, 1, NBUF, INV, SEQ>(v, bufs, par, tw);
 }

@@ -15,7 +15,7 @@
 //                    Fy^ = sigma^ (i s d) + deltay^ e + deltax^ (s f)
 //                  (s = -1 for ky > Py/2: those planes are odd in ky); both are
 //                  transformed back along y and the first ny rows written:
-//                  work_inv[o][kx][j].
+//                  work_inv[o][j / 8][kx][j % 8].
 //   3. k_row_inv : per row j < ny, the two half spectra are inverse transformed
 //                  along x (two rows per complex FFT) and the first nx values
 //                  written to Fx, Fy. The spectra already carry G / (Px Py).
@@ -106,6 +106,19 @@ struct edge_args {
     cplx_t<T> *edge;
 };
 
+// The column pass's output, work_inv: blocks of INV_ROWS rows, [o][j / 8][kx][j % 8]
+// (rows rounded up to a whole block), so that the inverse row pass reads its rows
+// in one contiguous piece; the column pass scatters 64-byte segments instead, in
+// stores that nothing waits for. With [o][kx][j] the inverse pass gathered 64 bytes
+// per column and waited on them (long-scoreboard stalls 3.7 per issue).
+constexpr int INV_ROWS = 8;
+__host__ __device__ __forceinline__ int64_t inv_rows(int ny) { return (ny + INV_ROWS - 1) & ~(INV_ROWS - 1); }
+// (32-bit: at most 3 x 2049 x 2048 elements)
+__device__ __forceinline__ int inv_index(int o, int kx, int j, int qx, int ny)
+{
+    return ((o * ((ny + INV_ROWS - 1) / INV_ROWS) + j / INV_ROWS) * qx + kx) * INV_ROWS + j % INV_ROWS;
+}
+
 // Global-to-shared staging loops issue LOAD_UNROLL loads per thread before
 // their shared-memory stores, so that these loads are in flight together.
 constexpr int LOAD_UNROLL = 4;
@@ -171,6 +184,37 @@ __device__ __forceinline__ void ld_pair(const C *p, int k, C &a, C &b)
         b = ld_table<CO>(p + 2 * k + 1);
     }
 }
+// Elements from one row sequence to the next in shared memory: the padded length, a
+// multiple of 128 bytes, plus 128 / NB bytes, so that the sequences that a warp
+// stages and unpacks side by side (four in the inverse pass of 2048 points) fall in
+// distinct banks.
+template <typename T>
+__host__ __device__ constexpr int row_seq(int px, int nb)
+{
+    constexpr int cs = (int)sizeof(cplx_t<T>);
+    return spad<cplx_t<T>>(px) + (128 / nb > cs ? 128 / nb / cs : 1);
+}
+
+// Row passes of up to 1024 points and of the lengths 3 2^k and 5 2^k, with eight
+// elements per thread, keep the rows in registers between the stages (fft_regs, two
+// exchange buffers): four barriers for a 1536-point row instead of nine, and the
+// loads of the forward pass and the stores of the inverse one go straight to and
+// from registers (64^2 12.7 -> 11.9 us, 160^2 11.7 -> 10.8, 700^2 35.5 -> 34.1,
+// 500^2 23.0 -> 20.5, 1500^2 91.4 -> 88.2). 2048 points want four sequences per CTA in
+// the inverse pass for its loads, whose two buffers leave one CTA per SM (13.2 ->
+// 16.4 us), and 4096 points likewise (41.5 -> 47.7 us). Other launch shapes transform in shared memory (fft_batch), with the same results, as do FP64 rows (bound by the
+// FP64 pipe; two buffers would leave one CTA per SM).
+template <typename T>
+__host__ __device__ constexpr bool row_in_regs(int px, int nb, int threads)
+{
+    return sizeof(T) == 4 && (!sg_pow2(px) || px <= 1024) && nb * px / 8 <= threads && 2 * nb * px / 8 > threads;
+}
+template <typename T>
+__host__ __device__ constexpr int row_smem_bytes(int px, int nb, int threads)
+{
+    return (row_in_regs<T>(px, nb, threads) ? 2 : 1) * nb * row_seq<T>(px, nb) * (int)sizeof(cplx_t<T>);
+}
+
 template <typename T, int PX, int NB, int THREADS, bool WAIT_AT_END = false>
 __device__ __forceinline__ void row_fwd_body(const row_fwd_args<T> &args, int bx, int f,
                                              const cplx_t<T> *__restrict__ tw)
@@ -180,6 +224,7 @@ __device__ __forceinline__ void row_fwd_body(const row_fwd_args<T> &args, int bx
     C *buf = reinterpret_cast<C *>(smem_raw);
     constexpr int RB = 2 * NB;
     constexpr int QX = PX / 2 + 1;
+    constexpr int SEQ = row_seq<T>(PX, NB);
     const field_src<T> &src = args.src;
     cplx_t<T> *__restrict__ work = args.work;
     const int j0 = bx * RB;
@@ -192,28 +237,47 @@ __device__ __forceinline__ void row_fwd_body(const row_fwd_args<T> &args, int bx
     if constexpr (!WAIT_AT_END) sg_dep_wait();
 
     // two rows per complex sequence: z = row(2s) + i row(2s+1); positions >= PX/2 are zero
-    constexpr int NE = NB * (PX / 2);
-    for (int e0 = threadIdx.x; e0 < NE; e0 += LOAD_UNROLL * THREADS) {
-        T a[LOAD_UNROLL], b[LOAD_UNROLL];
+    if constexpr (row_in_regs<T>(PX, NB, THREADS)) {
+        constexpr int STEP = PX / 8;
+        const int q = threadIdx.x / STEP, jt = threadIdx.x % STEP, ja = j0 + 2 * q;
+        C v[8];
 #pragma unroll
-        for (int u = 0; u < LOAD_UNROLL; ++u) {
-            const int e = e0 + u * THREADS;
-            a[u] = b[u] = (T)0;
-            if (e < NE) {
-                const int s = e / (PX / 2), i = e % (PX / 2);
-                const int ja = j0 + 2 * s;
-                a[u] = field_value(src, f, ja, i);
-                b[u] = field_value(src, f, ja + 1, i);
+        for (int m = 0; m < 8; ++m)
+            v[m] = m < 4 && q < NB ? cmake<C>(field_value(src, f, ja, jt + m * STEP), field_value(src, f, ja + 1, jt + m * STEP))
+                                   : cmake<C>((T)0, (T)0);
+        int par = 0;
+        fft_regs<C, PX, NB, THREADS, 2, false, SEQ>(v, buf, par, tw);
+        // the transform into the buffer that no thread still reads, for the unpacking
+        buf += par * (NB * SEQ);
+        if (q < NB) {
+#pragma unroll
+            for (int m = 0; m < 8; ++m) buf[q * SEQ + spad<C>(jt + m * STEP)] = v[m];
+        }
+        __syncthreads();
+    } else {
+        constexpr int NE = NB * (PX / 2);
+        for (int e0 = threadIdx.x; e0 < NE; e0 += LOAD_UNROLL * THREADS) {
+            T a[LOAD_UNROLL], b[LOAD_UNROLL];
+#pragma unroll
+            for (int u = 0; u < LOAD_UNROLL; ++u) {
+                const int e = e0 + u * THREADS;
+                a[u] = b[u] = (T)0;
+                if (e < NE) {
+                    const int s = e / (PX / 2), i = e % (PX / 2);
+                    const int ja = j0 + 2 * s;
+                    a[u] = field_value(src, f, ja, i);
+                    b[u] = field_value(src, f, ja + 1, i);
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < LOAD_UNROLL; ++u) {
+                const int e = e0 + u * THREADS;
+                if (e < NE) buf[(e / (PX / 2)) * SEQ + spad<C>(e % (PX / 2))] = cmake<C>(a[u], b[u]);
             }
         }
-#pragma unroll
-        for (int u = 0; u < LOAD_UNROLL; ++u) {
-            const int e = e0 + u * THREADS;
-            if (e < NE) buf[spad<C>((e / (PX / 2)) * PX + e % (PX / 2))] = cmake<C>(a[u], b[u]);
-        }
+        __syncthreads();
+        fft_batch<C, PX, NB, THREADS, false, true, false, SEQ>(buf, tw);
     }
-    __syncthreads();
-    fft_batch<C, PX, NB, THREADS, false, true>(buf, tw);
 
     // unpack: A[k] = (Z[k] + conj Z[-k]) / 2, B[k] = (Z[k] - conj Z[-k]) / 2i
     const T half = (T)0.5;
@@ -222,8 +286,8 @@ __device__ __forceinline__ void row_fwd_body(const row_fwd_args<T> &args, int bx
         const int j = j0 + r;
         if (j >= ny) continue;
         const int s = r >> 1;
-        const C z = buf[spad<C>(s * PX + kx)];
-        const C w = buf[spad<C>(s * PX + (kx == 0 ? 0 : PX - kx))];
+        const C z = buf[s * SEQ + spad<C>(kx)];
+        const C w = buf[s * SEQ + spad<C>(kx == 0 ? 0 : PX - kx)];
         C out;
         if ((r & 1) == 0) out = cmake<C>(half * (z.x + w.x), half * (z.y - w.y));
         else out = cmake<C>(half * (z.y + w.y), half * (w.x - z.x));
@@ -236,9 +300,33 @@ template <typename T, int PX, int NB, int THREADS, bool BATCH = false, bool WAIT
 __global__ void __launch_bounds__(THREADS) k_row_fwd(row_fwd_args<T> one, const row_fwd_args<T> *__restrict__ many,
                                                      const cplx_t<T> *__restrict__ tw)
 {
-    sg_dep_trigger();
+    // the first kernel of a solve without an edge pass lets the next one start only
+    // once the stream's previous kernel has finished (see sg_dep_first)
+    if constexpr (WAIT_AT_END) sg_dep_trigger();
+    else sg_dep_first();
     const row_fwd_args<T> args = pass_args<BATCH>(one, many);
     row_fwd_body<T, PX, NB, THREADS, WAIT_AT_END>(args, blockIdx.x, blockIdx.y, tw);
+}
+
+// exp(2 pi i u / 8)
+template <typename T>
+__device__ __forceinline__ cplx_t<T> turn8(int u)
+{
+    const T h = (T)0.70710678118654752440;
+    const T s = (u & 4) ? (T)-1 : (T)1;            // half a turn
+    const T a = (u & 1) ? h : (T)1, b = (u & 1) ? h : (T)0;
+    return (u & 2) ? cmake<cplx_t<T>>(-s * b, s * a) : cmake<cplx_t<T>>(s * a, s * b);
+}
+// a exp(2 pi i q / 8) for a constant q, explicitly rounded
+template <typename C>
+__device__ __forceinline__ C rot8(C a, int q)
+{
+    using T = decltype(C::x);
+    const T h = (T)0.70710678118654752440;
+    if (q & 1) a = cmake<C>(mul_rn(h, add_rn(a.x, -a.y)), mul_rn(h, add_rn(a.x, a.y)));
+    if (q & 2) a = cmake<C>(-a.y, a.x);
+    if (q & 4) a = cmake<C>(-a.x, -a.y);
+    return a;
 }
 
 // Shared-memory layout of the column kernels: the padded FFT buffer, then the
@@ -261,22 +349,27 @@ __host__ __device__ constexpr int col_cb_default(int py)
     if (!sg_pow2(py)) return py < 512 ? 3 : (py < 768 ? 2 : 1);
     return py >= 2048 ? 1 : 2048 / py;
 }
-// The central-slope pass kernel on FP32 2048-point columns, one column per CTA,
-// runs four CTAs per SM instead of three (1025 columns in 1.7 waves instead of
-// 2.25): 64 registers (one spilled) and one exchange buffer, so that four CTAs'
-// buffers and spectrum planes (41 KB each) fit in an SM's shared memory.
-// Measured 28.3 -> 27.2 us per pass at 2048 x 2048; the caller-slope pass
-// spills 100 bytes at 64 registers and keeps three.
-template <typename T, int PY, int CB>
-__host__ __device__ constexpr bool col_central_four() { return sizeof(T) == 4 && PY == 2048 && CB == 1; }
+// The central-slope pass kernel takes 64 registers and one exchange buffer at the
+// default shape of FP32 columns of 2048 and 4096 points, so that 32 warps fit per SM
+// (four CTAs of 256 threads, or two of 512; 41 KB and 84 KB of shared memory each)
+// instead of 24 and 16: 28.3 -> 27.2 us per pass at 2048 x 2048, 112 -> 95 us at
+// 4096 x 4096. Batches do so at every length (64 disks of 64^2 to 512^2: 257 -> 234 us
+// per batch); single solves of the shorter lengths, bound by latency, are 3 % faster
+// at two CTAs without the spills (250^2 14.8 against 15.2 us). The caller-slope pass
+// spills 100 bytes at 64 registers and takes 80 (three CTAs).
+template <typename T, int PY, int CB, bool BATCH>
+__host__ __device__ constexpr bool col_central_four()
+{
+    return sizeof(T) == 4 && sg_pow2(PY) && CB == col_cb_default(PY) && (BATCH || PY >= 2048);
+}
 // 768 and 1536 points likewise take 64 registers (both buffers fit): five CTAs of
 // 192 threads at 1536 points (a 700^2 solve 37.4 -> 35.6 us). At 1280 and 2560 the
 // radix-5 stage spills 60 bytes there and the pass is slower (600^2: 34.2 us at 64
 // registers, 30.9 at 80).
 template <typename T, int PY, int CB>
 __host__ __device__ constexpr bool col_central_lean() { return sizeof(T) == 4 && (PY == 768 || PY == 1536); }
-template <typename T, int PY, int CB>
-__host__ __device__ constexpr int col_central_nbuf() { return col_central_four<T, PY, CB>() ? 1 : col_nbuf<T, PY>(); }
+template <typename T, int PY, int CB, bool BATCH>
+__host__ __device__ constexpr int col_central_nbuf() { return col_central_four<T, PY, CB, BATCH>() ? 1 : col_nbuf<T, PY>(); }
 template <typename T, int PY, int CB, int NB = col_nbuf<T, PY>()>
 __host__ __device__ constexpr int col_buf_bytes() { return NB * ((spad_size<cplx_t<T>>(CB * PY) * (int)sizeof(cplx_t<T>) + 15) & ~15); }
 template <typename T, int PY, int CB, int NPL = 6, int NB = col_nbuf<T, PY>()>
@@ -313,18 +406,20 @@ __device__ __forceinline__ bool spectra_ready(uint64_t *bar, int *err, int tries
 }
 
 
-// resident CTAs per SM asked of the register allocator (spill-free choices at
-// the default shapes, scaled by the CTA size for the other candidates). FP32
-// 2048-point columns: the two exchange buffers and six spectrum planes take
-// 59.5 KB of shared memory, so three CTAs fit per SM: 80 registers each (the
-// central-slope pass kernel's four-CTA form, above, overrides this).
-// The other lengths: as many CTAs as leave 80 registers a thread (three outputs
-// and FP64: 128).
+// resident CTAs per SM asked of the register allocator for the caller-slope and
+// multi-output passes (at the default shapes, scaled by the CTA size for the other
+// candidates). FP32 columns of up to 2048 points: three CTAs of 256 threads at 80
+// registers (two exchange buffers and six spectrum planes take 59.5 KB each; a 500^2
+// caller-slope solve 28.3 us with two CTAs below 2048 points, 25.0 with three), two
+// for three outputs.
+// The other lengths: as many CTAs as leave 96 registers a thread below 1536 points,
+// 80 from there (three outputs and FP64: 128).
 template <typename T, int PY, int NOUT>
 constexpr int col_min_blocks_def()
 {
-    if (!sg_pow2(PY)) return 65536 / ((sizeof(T) == 4 && NOUT < 3 ? 80 : 128) * (col_cb_default(PY) * PY / 8));
-    return sizeof(T) == 4 ? (PY == 2048 ? (NOUT == 3 ? 2 : 3) : (PY == 4096 ? 1 : 2)) : 1;
+    if (!sg_pow2(PY))
+        return 65536 / ((sizeof(T) == 4 && NOUT < 3 ? (PY < 1536 ? 96 : 80) : 128) * (col_cb_default(PY) * PY / 8));
+    return sizeof(T) == 4 ? (PY == 4096 ? 1 : (NOUT == 3 ? 2 : 3)) : 1;
 }
 template <typename T, int PY, int THREADS, int NOUT = 2>
 constexpr int col_min_blocks()
@@ -333,11 +428,12 @@ constexpr int col_min_blocks()
     constexpr int d = col_min_blocks_def<T, PY, NOUT>();
     return d * def_threads / THREADS >= 1 ? d * def_threads / THREADS : 1;
 }
-template <typename T, int PY, int CB, int THREADS>
+template <typename T, int PY, int CB, int THREADS, bool BATCH>
 constexpr int col_central_blocks()
 {
-    if (col_central_four<T, PY, CB>()) return 4;
+    if (col_central_four<T, PY, CB, BATCH>()) return 65536 / (64 * THREADS);
     if (col_central_lean<T, PY, CB>()) return 65536 / (64 * THREADS);
+    if (sizeof(T) == 4 && sg_pow2(PY) && PY < 2048) return 512 / THREADS >= 1 ? 512 / THREADS : 1;
     return col_min_blocks<T, PY, THREADS>();
 }
 
@@ -381,7 +477,7 @@ __device__ __forceinline__ void col_body(const col_args<T> &args, int bx, int qx
 #pragma unroll
         for (int m = 0; m < 8; ++m) {
             const int j = jt + m * STEP;
-            v[m] = (m < 4 && j < ny && kx < qx) ? ld_plain<CO>(&work_fwd[((int64_t)f * qx + kx) * ny + j])
+            v[m] = (m < 4 && j < ny && kx < qx) ? ld_plain<CO>(&work_fwd[(f * qx + kx) * ny + j])
                                                 : cmake<C>((T)0, (T)0);
         }
         if (col_nbuf<T, PY>() == 1 && f > 0) __syncthreads();
@@ -455,10 +551,10 @@ __device__ __forceinline__ void col_body(const col_args<T> &args, int bx, int qx
         }
         if (col_nbuf<T, PY>() == 1) __syncthreads();
         fft_regs<C, PY, CB, THREADS, col_nbuf<T, PY>(), true>(v, bufs, par, tw);
+        const int at = inv_index(o, kx, jt, qx, ny);  // STEP is a whole number of row blocks
 #pragma unroll
         for (int m = 0; m < 4; ++m) {
-            const int j = jt + m * STEP;
-            if (j < ny && kx < qx) work_inv[((int64_t)o * qx + kx) * ny + j] = v[m];
+            if (jt + m * STEP < ny && kx < qx) work_inv[at + m * (STEP * qx)] = v[m];
         }
     }
 }
@@ -478,7 +574,10 @@ __device__ __forceinline__ void row_inv_body(const row_inv_args<T> &args, int bx
 {
     using C = cplx_t<T>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    C *buf = reinterpret_cast<C *>(smem_raw);
+    // register form: staged in the second exchange buffer (the first exchange writes the first)
+    constexpr int SEQ = row_seq<T>(PX, NB);
+    constexpr bool REGS = row_in_regs<T>(PX, NB, THREADS);
+    C *buf = reinterpret_cast<C *>(smem_raw) + (REGS ? NB * SEQ : 0);
     constexpr int RB = 2 * NB;
     constexpr int QX = PX / 2 + 1;
     const cplx_t<T> *__restrict__ work_inv = args.wi;
@@ -487,26 +586,20 @@ __device__ __forceinline__ void row_inv_body(const row_inv_args<T> &args, int bx
     const int j0 = bx * RB;
     if (j0 >= ny) return;
     sg_dep_wait();
-    const C *w = work_inv + (int64_t)o * QX * ny;
     T *out = o == 0 ? fx : (o == 1 ? fy : fz);
 
-    // Z[k] = A[k] + i B[k] over the full length, from the half spectra of rows 2s, 2s+1.
-    // In FP32 with an even row count the two rows' values of a column are one
-    // aligned 16-byte pair (ja is even): one load instead of two.
+    // Z[k] = A[k] + i B[k] over the full length, from the half spectra of rows 2s, 2s+1:
+    // the two rows' values of a column are one aligned pair (ja is even), consecutive
+    // threads read consecutive pairs
     constexpr int NE = NB * QX;
-    const bool pairs = sizeof(C) == 8 && (ny & 1) == 0;
     for (int e0 = threadIdx.x; e0 < NE; e0 += LOAD_UNROLL * THREADS) {
         C av[LOAD_UNROLL], bv[LOAD_UNROLL];
 #pragma unroll
         for (int u = 0; u < LOAD_UNROLL; ++u) {
             const int e = e0 + u * THREADS, s = e % NB, k = e / NB, ja = j0 + 2 * s;
-            if (pairs) {
-                av[u] = bv[u] = cmake<C>((T)0, (T)0);
-                if (e < NE && ja < ny) ld_pair_plain<CO>(&w[(int64_t)k * ny + ja], av[u], bv[u]);
-            } else {
-                av[u] = (e < NE && ja < ny) ? ld_plain<CO>(&w[(int64_t)k * ny + ja]) : cmake<C>((T)0, (T)0);
-                bv[u] = (e < NE && ja + 1 < ny) ? ld_plain<CO>(&w[(int64_t)k * ny + ja + 1]) : cmake<C>((T)0, (T)0);
-            }
+            av[u] = bv[u] = cmake<C>((T)0, (T)0);
+            if (e < NE && ja < ny) ld_pair_plain<CO>(&work_inv[inv_index(o, k, ja, QX, ny)], av[u], bv[u]);
+            if (ja + 1 >= ny) bv[u] = cmake<C>((T)0, (T)0);  // a row of the last block past the patch
         }
 #pragma unroll
         for (int u = 0; u < LOAD_UNROLL; ++u) {
@@ -517,19 +610,40 @@ __device__ __forceinline__ void row_inv_body(const row_inv_args<T> &args, int bx
                 a.y = (T)0;
                 b.y = (T)0;
             }
-            buf[spad<C>(s * PX + k)] = cmake<C>(a.x - b.y, a.y + b.x);
-            if (k > 0 && k < PX / 2) buf[spad<C>(s * PX + PX - k)] = cmake<C>(a.x + b.y, b.x - a.y);  // conj(a) + i conj(b)
+            buf[s * SEQ + spad<C>(k)] = cmake<C>(a.x - b.y, a.y + b.x);
+            if (k > 0 && k < PX / 2) buf[s * SEQ + spad<C>(PX - k)] = cmake<C>(a.x + b.y, b.x - a.y);  // conj(a) + i conj(b)
         }
     }
     __syncthreads();
-    fft_batch<C, PX, NB, THREADS, true, false, true>(buf, tw);
-    for (int e = threadIdx.x; e < NB * PX; e += THREADS) {
-        const int s = e / PX, i = e % PX;
-        if (i >= nx) continue;
-        const int ja = j0 + 2 * s;
-        const C z = buf[spad<C>(e)];
-        if (ja < ny) out[(int64_t)ja * nx + i] = z.x;
-        if (ja + 1 < ny) out[(int64_t)(ja + 1) * nx + i] = z.y;
+    if constexpr (REGS) {
+        constexpr int STEP = PX / 8;
+        const int q = threadIdx.x / STEP, jt = threadIdx.x % STEP, ja = j0 + 2 * q;
+        C v[8];
+        if (q < NB) {
+#pragma unroll
+            for (int m = 0; m < 8; ++m) v[m] = buf[q * SEQ + spad<C>(jt + m * STEP)];
+        }
+        int par = 0;
+        fft_regs<C, PX, NB, THREADS, 2, true, SEQ>(v, reinterpret_cast<C *>(smem_raw), par, tw);
+        if (q < NB) {
+#pragma unroll
+            for (int m = 0; m < 4; ++m) {
+                const int i = jt + m * STEP;
+                if (i >= nx) continue;
+                if (ja < ny) out[(int64_t)ja * nx + i] = v[m].x;
+                if (ja + 1 < ny) out[(int64_t)(ja + 1) * nx + i] = v[m].y;
+            }
+        }
+    } else {
+        fft_batch<C, PX, NB, THREADS, true, false, true, SEQ>(buf, tw);
+        for (int e = threadIdx.x; e < NB * PX; e += THREADS) {
+            const int s = e / PX, i = e % PX;
+            if (i >= nx) continue;
+            const int ja = j0 + 2 * s;
+            const C z = buf[s * SEQ + spad<C>(i)];
+            if (ja < ny) out[(int64_t)ja * nx + i] = z.x;
+            if (ja + 1 < ny) out[(int64_t)(ja + 1) * nx + i] = z.y;
+        }
     }
 }
 
@@ -577,8 +691,7 @@ __global__ void __launch_bounds__(THREADS) k_edge_cols(edge_args<T> one, const e
     // kernel of the stream (its scratch is the solve's scratch), then lets the
     // row pass start beside it (k_row_fwd with WAIT_AT_END), whose completion
     // then implies this kernel's for the column pass after them
-    sg_dep_wait();
-    sg_dep_trigger();
+    sg_dep_first();
     const edge_args<T> args = pass_args<BATCH>(one, many);
     edge_body<T, PY, THREADS>(args, tw);
 }
@@ -633,6 +746,14 @@ __device__ __forceinline__ void col_central_body(const col_args<T> &args, int bx
     if (!spectra_ready(&bar, err, args.tries)) return;
     if (CO && threadIdx.x == 0) mbar_inval(&bar);  // every thread has passed its wait; the body runs again
 
+    // the slope factors of the column, and of the bins jt + q PY/8: those of bin jt
+    // turned by q (and -ny q) eighths, so one load instead of eight
+    C e1, e2, f1, f2;
+    ld_pair<false>(cpair, kx < qx ? kx : 0, e1, e2);
+    ld_pair<false>(rpair, jt, f1, f2);
+    C r0 = rows[c < CB ? c : 0][0], r1 = rows[c < CB ? c : 0][1];
+    r0 = cmul_rn(f1, r0);
+    r1 = cmul_rn(f2, r1);
     C accx[8], accy[8];
 #pragma unroll
     for (int q = 0; q < 8; ++q) {
@@ -645,15 +766,12 @@ __device__ __forceinline__ void col_central_body(const col_args<T> &args, int bx
         const T *sp = ssp + c * QS + kq;  // plane p at sp[p * CB * QS]
         const C S = v[q];
         // slope spectra
-        C e1, e2, f1, f2;
-        ld_pair<false>(cpair, kx, e1, e2);
-        ld_pair<false>(rpair, ky, f1, f2);
-        const T cs = (T)2 * e1.y, rs = (T)2 * f1.y;  // sin(2 pi k / P) / h, exactly
+        const T cs = (T)2 * e1.y, rs = (T)2 * rot8(f1, q).y;  // sin(2 pi k / P) / h
         C c0, c1;
         ld_pair<CO>(edge, ky, c0, c1);
         // every operation explicitly rounded (see mul_rn): the result must not depend on the launch shape
         const C p2 = cmul_rn(e2, c1), p1 = cmul_rn(e1, c0);
-        const C q2 = cmul_rn(f2, rows[c][1]), q1 = cmul_rn(f1, rows[c][0]);
+        const C q2 = cmul_rn(turn8<T>(-ny * q), r1), q1 = rot8(r0, q);
         const C X = cmake<C>(add_rn(add_rn(-mul_rn(cs, S.y), p2.x), -p1.x), add_rn(add_rn(mul_rn(cs, S.x), p2.y), -p1.y));
         const C Y = cmake<C>(add_rn(add_rn(-mul_rn(rs, S.y), q2.x), -q1.x), add_rn(add_rn(mul_rn(rs, S.x), q2.y), -q1.y));
         const T a = sp[0 * CB * QS];
@@ -669,18 +787,16 @@ __device__ __forceinline__ void col_central_body(const col_args<T> &args, int bx
     // inverse transforms: the products are already in the transform's input pattern
     if (col_nbuf<T, PY>() == 1) __syncthreads();
     fft_regs<C, PY, CB, THREADS, col_nbuf<T, PY>(), true>(accx, bufs, par, tw);
+    int at = inv_index(0, kx, jt, qx, ny);  // STEP is a whole number of row blocks
 #pragma unroll
-    for (int m = 0; m < 4; ++m) {
-        const int j = jt + m * STEP;
-        if (j < ny && kx < qx) work_inv[(int64_t)kx * ny + j] = accx[m];
-    }
+    for (int m = 0; m < 4; ++m)
+        if (jt + m * STEP < ny && kx < qx) work_inv[at + m * (STEP * qx)] = accx[m];
     if (col_nbuf<T, PY>() == 1) __syncthreads();
     fft_regs<C, PY, CB, THREADS, col_nbuf<T, PY>(), true>(accy, bufs, par, tw);
+    at = inv_index(1, kx, jt, qx, ny);
 #pragma unroll
-    for (int m = 0; m < 4; ++m) {
-        const int j = jt + m * STEP;
-        if (j < ny && kx < qx) work_inv[((int64_t)qx + kx) * ny + j] = accy[m];
-    }
+    for (int m = 0; m < 4; ++m)
+        if (jt + m * STEP < ny && kx < qx) work_inv[at + m * (STEP * qx)] = accy[m];
 }
 
 
@@ -690,7 +806,7 @@ __device__ __forceinline__ void col_central_body(const col_args<T> &args, int bx
 // same registers, more time waiting on global loads). The batch tests check that
 // the persistent kernel (which runs the body) and this kernel agree bit for bit.
 template <typename T, int PY, int CB, int THREADS, bool BATCH = false>
-__global__ void __launch_bounds__(THREADS, (col_central_blocks<T, PY, CB, THREADS>())) k_col_conv_central(
+__global__ void __launch_bounds__(THREADS, (col_central_blocks<T, PY, CB, THREADS, BATCH>())) k_col_conv_central(
     col_args<T> one, const col_args<T> *__restrict__ many, int qx, const cplx_t<T> *__restrict__ tw, int *err)
 {
     using C = cplx_t<T>;
@@ -704,7 +820,7 @@ __global__ void __launch_bounds__(THREADS, (col_central_blocks<T, PY, CB, THREAD
     const int ny = args.ny;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     C *bufs = reinterpret_cast<C *>(smem_raw);
-    T *ssp = reinterpret_cast<T *>(smem_raw + col_buf_bytes<T, PY, CB, col_central_nbuf<T, PY, CB>()>());
+    T *ssp = reinterpret_cast<T *>(smem_raw + col_buf_bytes<T, PY, CB, col_central_nbuf<T, PY, CB, BATCH>()>());
     __shared__ uint64_t bar;
     __shared__ C rows[CB][2];  // R0, R1 of each column
     static_assert(CB * PY / THREADS == 8, "eight elements per thread");
@@ -732,9 +848,17 @@ __global__ void __launch_bounds__(THREADS, (col_central_blocks<T, PY, CB, THREAD
     for (int m = 0; m < 4; ++m)
         if (jt + m * STEP == ny - 1) rows[c][1] = v[m];
     int par = 0;
-    fft_regs<C, PY, CB, THREADS, col_central_nbuf<T, PY, CB>(), false>(v, bufs, par, tw);
+    fft_regs<C, PY, CB, THREADS, col_central_nbuf<T, PY, CB, BATCH>(), false>(v, bufs, par, tw);
     if (!spectra_ready(&bar, err, args.tries)) return;
 
+    // the slope factors of the column, and of the bins jt + q PY/8: those of bin jt
+    // turned by q (and -ny q) eighths, so one load instead of eight
+    C e1, e2, f1, f2;
+    ld_pair<false>(cpair, kx < qx ? kx : 0, e1, e2);
+    ld_pair<false>(rpair, jt, f1, f2);
+    C r0 = rows[c < CB ? c : 0][0], r1 = rows[c < CB ? c : 0][1];
+    r0 = cmul_rn(f1, r0);
+    r1 = cmul_rn(f2, r1);
     C accx[8], accy[8];
 #pragma unroll
     for (int q = 0; q < 8; ++q) {
@@ -747,15 +871,12 @@ __global__ void __launch_bounds__(THREADS, (col_central_blocks<T, PY, CB, THREAD
         const T *sp = ssp + c * QS + kq;  // plane p at sp[p * CB * QS]
         const C S = v[q];
         // slope spectra
-        C e1, e2, f1, f2;
-        ld_pair<false>(cpair, kx, e1, e2);
-        ld_pair<false>(rpair, ky, f1, f2);
-        const T cs = (T)2 * e1.y, rs = (T)2 * f1.y;  // sin(2 pi k / P) / h, exactly
+        const T cs = (T)2 * e1.y, rs = (T)2 * rot8(f1, q).y;  // sin(2 pi k / P) / h
         C c0, c1;
         ld_pair<false>(edge, ky, c0, c1);
         // every operation explicitly rounded (see mul_rn): the result must not depend on the launch shape
         const C p2 = cmul_rn(e2, c1), p1 = cmul_rn(e1, c0);
-        const C q2 = cmul_rn(f2, rows[c][1]), q1 = cmul_rn(f1, rows[c][0]);
+        const C q2 = cmul_rn(turn8<T>(-ny * q), r1), q1 = rot8(r0, q);
         const C X = cmake<C>(add_rn(add_rn(-mul_rn(cs, S.y), p2.x), -p1.x), add_rn(add_rn(mul_rn(cs, S.x), p2.y), -p1.y));
         const C Y = cmake<C>(add_rn(add_rn(-mul_rn(rs, S.y), q2.x), -q1.x), add_rn(add_rn(mul_rn(rs, S.x), q2.y), -q1.y));
         const T a = sp[0 * CB * QS];
@@ -769,20 +890,18 @@ __global__ void __launch_bounds__(THREADS, (col_central_blocks<T, PY, CB, THREAD
     }
 
     // inverse transforms: the products are already in the transform's input pattern
-    if (col_central_nbuf<T, PY, CB>() == 1) __syncthreads();
-    fft_regs<C, PY, CB, THREADS, col_central_nbuf<T, PY, CB>(), true>(accx, bufs, par, tw);
+    if (col_central_nbuf<T, PY, CB, BATCH>() == 1) __syncthreads();
+    fft_regs<C, PY, CB, THREADS, col_central_nbuf<T, PY, CB, BATCH>(), true>(accx, bufs, par, tw);
+    int at = inv_index(0, kx, jt, qx, ny);  // STEP is a whole number of row blocks
 #pragma unroll
-    for (int m = 0; m < 4; ++m) {
-        const int j = jt + m * STEP;
-        if (j < ny && kx < qx) work_inv[(int64_t)kx * ny + j] = accx[m];
-    }
-    if (col_central_nbuf<T, PY, CB>() == 1) __syncthreads();
-    fft_regs<C, PY, CB, THREADS, col_central_nbuf<T, PY, CB>(), true>(accy, bufs, par, tw);
+    for (int m = 0; m < 4; ++m)
+        if (jt + m * STEP < ny && kx < qx) work_inv[at + m * (STEP * qx)] = accx[m];
+    if (col_central_nbuf<T, PY, CB, BATCH>() == 1) __syncthreads();
+    fft_regs<C, PY, CB, THREADS, col_central_nbuf<T, PY, CB, BATCH>(), true>(accy, bufs, par, tw);
+    at = inv_index(1, kx, jt, qx, ny);
 #pragma unroll
-    for (int m = 0; m < 4; ++m) {
-        const int j = jt + m * STEP;
-        if (j < ny && kx < qx) work_inv[((int64_t)qx + kx) * ny + j] = accy[m];
-    }
+    for (int m = 0; m < 4; ++m)
+        if (jt + m * STEP < ny && kx < qx) work_inv[at + m * (STEP * qx)] = accy[m];
 }
 
 // ------------------------------------------------------------ launch shapes --
@@ -819,6 +938,7 @@ __host__ __device__ constexpr int shape_candidate(int def, int k) { return k == 
 template <typename T>
 __host__ __device__ constexpr bool row_feasible_t(int px, int nb)
 {
+    // (the skew of row_seq is not counted: the same candidates as without it)
     return nb >= 1 && nb <= 64 && (int64_t)spad_size<cplx_t<T>>(nb * px) * (int64_t)sizeof(cplx_t<T>) <= 200 * 1024;
 }
 template <typename T, int PY, int CB, int NPL>

@@ -8,19 +8,20 @@ namespace {
 
 // after_edge: launched right after the edge-column transform of a central-slope
 // solve, as a dependent launch that runs beside it and waits for it at its end
-// (k_row_fwd with WAIT_AT_END); otherwise the first kernel of the solve.
+// (k_row_fwd with WAIT_AT_END); otherwise the first kernel of the solve, a dependent
+// launch too (it waits for the stream's previous kernel at its start): launched
+// normally, solves back to back started on a grid of 2.05 us steps.
 template <typename T, int PX, int NB, bool BATCH, bool AFTER_EDGE>
 sg_status launch_rows_fwd(const row_fwd_args<T> &one, const row_fwd_args<T> *many, batch_shape bs, int nf,
                           const cplx_t<T> *tw, cudaStream_t st)
 {
-    const size_t smem = (size_t)spad_size<cplx_t<T>>(NB * PX) * sizeof(cplx_t<T>);
     constexpr int THREADS = row_threads(PX, NB);
+    const size_t smem = (size_t)row_smem_bytes<T>(PX, NB, THREADS);
     auto kern = k_row_fwd<T, PX, NB, THREADS, BATCH, AFTER_EDGE>;
     SG_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     const int ny = BATCH ? bs.maxny : one.src.ny;
     dim3 grid((ny + 2 * NB - 1) / (2 * NB), nf, BATCH ? bs.nmem : 1);
-    if (AFTER_EDGE) SG_CUDA_TRY(sg_launch_dep(kern, grid, dim3(THREADS), smem, st, one, many, tw));
-    else kern<<<grid, THREADS, smem, st>>>(one, many, tw);
+    SG_CUDA_TRY(sg_launch_dep(kern, grid, dim3(THREADS), smem, st, one, many, tw));
     SG_CUDA_TRY(cudaGetLastError());
     return SG_OK;
 }

@@ -10,8 +10,8 @@ template <typename T, int PX, int NB, bool BATCH>
 sg_status launch_rows_inv(const row_inv_args<T> &one, const row_inv_args<T> *many, batch_shape bs, int nout,
                           const cplx_t<T> *tw, cudaStream_t st)
 {
-    const size_t smem = (size_t)spad_size<cplx_t<T>>(NB * PX) * sizeof(cplx_t<T>);
     constexpr int THREADS = row_threads(PX, NB);
+    const size_t smem = (size_t)row_smem_bytes<T>(PX, NB, THREADS);
     auto kern = k_row_inv<T, PX, NB, THREADS, BATCH>;
     SG_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     const int ny = BATCH ? bs.maxny : one.ny;
