@@ -477,7 +477,7 @@ bool lv_params(const sg_geom *g, const geom_info &gi, sg_precision prec, sg_lv_s
         mapbytes += (int64_t)mp.size() * 4;
         // compact row transforms and source spectra, full-width inverse columns
         const int64_t qxc = (px >> sg_lv_cexp(sx, (int)px)) / 2 + 1, pcy = py >> sg_lv_cexp(sx, (int)py);
-        work += (3 * qxc * a.ny[m] + 3 * qxc * pcy + 2 * qx * a.ny[m]) * cs;
+        work += (3 * qxc * a.ny[m] + 3 * qxc * pcy + 2 * qx * ((a.ny[m] + 7) & ~7)) * cs;
     }
     int nkeys = 0;
     int ks[3 * SG_MAX_LEVELS], kd[3 * SG_MAX_LEVELS];

@@ -18,10 +18,12 @@
 // kernels, read at the level-l sample points.
 //
 // Pipeline per solve (after the composite sources): for every level, the row
-// transforms of its sampled rows and the column transforms to full spectra; for
-// every target level, a column kernel that sums sources x kernel spectra over
-// all source levels and fields and inverse-transforms Fx, Fy at the target's
-// sampled rows; then the inverse row transforms, written to the level's cells.
+// transforms of its sampled rows and the column transforms to full spectra; a
+// column kernel that sums sources x kernel spectra over all source levels and
+// fields and inverse-transforms Fx, Fy at the targets' sampled rows; then the
+// inverse row transforms, written to the level's cells. The sums depend on the
+// target level only through f(s_l): every level but the finest has the same one
+// (sampled at different rows), so there are two sums whatever the level count.
 // Kernel spectra (six planes per distinct (s, d), FP64-built) depend only on
 // the lattice, not on the density.
 //
@@ -263,6 +265,31 @@ __device__ __forceinline__ int lv_level_of(const int *cta0, int nlev)
     return m;
 }
 
+// FP32 transforms of up to 4096 points run in registers (fft_regs, eight elements
+// per thread: 4096 / L sequences for 512 threads), FP64 and 8192-point ones in shared
+// memory. SEQ: elements from one sequence to the next (bank skew, see fftconv.cuh).
+template <typename T>
+__host__ __device__ constexpr bool lv_in_regs(int L) { return sizeof(T) == 4 && L <= 4096; }
+template <typename T>
+__host__ __device__ constexpr int lv_seq(int L, int nb)
+{
+    constexpr int cs = (int)sizeof(cplx_t<T>);
+    return spad<cplx_t<T>>(L) + (lv_in_regs<T>(L) ? (128 / nb > cs ? 128 / nb / cs : 1) : 0);
+}
+template <typename T>
+__host__ __device__ constexpr int lv_row_smem(int L)
+{
+    return (lv_in_regs<T>(L) ? 2 : 1) * lv_nb(L) * lv_seq<T>(L, lv_nb(L)) * (int)sizeof(cplx_t<T>);
+}
+// (dynamic shared memory of a launch over levels of lengths up to lmax)
+template <typename T>
+inline size_t lv_row_smem_max(int lmax)
+{
+    int b = 0;
+    for (int L = 64; L <= lmax; L *= 2) b = lv_row_smem<T>(L) > b ? lv_row_smem<T>(L) : b;
+    return (size_t)b;
+}
+
 // Row transforms (length PX = the level's compact Pcx) of a level's sampled
 // rows (three fields, blockIdx.y), two real rows per complex sequence;
 // out[(f qx + kx) ny + j], qx = PX/2 + 1.
@@ -274,34 +301,51 @@ __device__ __forceinline__ void lv_row_fwd_body(const lv_rows_src<T> &a, cplx_t<
     constexpr int NB = lv_nb(PX), THREADS = LV_ROW_THREADS;
     constexpr int RB = 2 * NB;
     constexpr int QX = PX / 2 + 1;
+    constexpr int SEQ = lv_seq<T>(PX, NB);
     const int f = blockIdx.y;
     const int j0 = blk * RB;
-    // LV_LOAD_UNROLL samples per thread in flight before their stores
-    constexpr int NE = NB * (PX / 2);
-    for (int e0 = threadIdx.x; e0 < NE; e0 += LV_LOAD_UNROLL * THREADS) {
-        T va[LV_LOAD_UNROLL], vb[LV_LOAD_UNROLL];
+    if constexpr (lv_in_regs<T>(PX)) {
+        constexpr int STEP = PX / 8;
+        const int q = threadIdx.x / STEP, jt = threadIdx.x % STEP, ja = j0 + 2 * q;
+        C v[8];
 #pragma unroll
-        for (int u = 0; u < LV_LOAD_UNROLL; ++u) {
-            const int e = e0 + u * THREADS, q = e / (PX / 2), I = e % (PX / 2), ja = j0 + 2 * q;
-            va[u] = e < NE ? lv_sample(a, f, ja, I) : (T)0;
-            vb[u] = e < NE ? lv_sample(a, f, ja + 1, I) : (T)0;
-        }
+        for (int m = 0; m < 8; ++m)
+            v[m] = m < 4 ? cmake<C>(lv_sample(a, f, ja, jt + m * STEP), lv_sample(a, f, ja + 1, jt + m * STEP))
+                         : cmake<C>((T)0, (T)0);
+        int par = 0;
+        fft_regs<C, PX, NB, THREADS, 2, false, SEQ>(v, buf, par, tw);
+        buf += par * (NB * SEQ);  // the buffer that no thread still reads
 #pragma unroll
-        for (int u = 0; u < LV_LOAD_UNROLL; ++u) {
-            const int e = e0 + u * THREADS;
-            if (e < NE) buf[spad<C>((e / (PX / 2)) * PX + e % (PX / 2))] = cmake<C>(va[u], vb[u]);
+        for (int m = 0; m < 8; ++m) buf[q * SEQ + spad<C>(jt + m * STEP)] = v[m];
+        __syncthreads();
+    } else {
+        // LV_LOAD_UNROLL samples per thread in flight before their stores
+        constexpr int NE = NB * (PX / 2);
+        for (int e0 = threadIdx.x; e0 < NE; e0 += LV_LOAD_UNROLL * THREADS) {
+            T va[LV_LOAD_UNROLL], vb[LV_LOAD_UNROLL];
+#pragma unroll
+            for (int u = 0; u < LV_LOAD_UNROLL; ++u) {
+                const int e = e0 + u * THREADS, q = e / (PX / 2), I = e % (PX / 2), ja = j0 + 2 * q;
+                va[u] = e < NE ? lv_sample(a, f, ja, I) : (T)0;
+                vb[u] = e < NE ? lv_sample(a, f, ja + 1, I) : (T)0;
+            }
+#pragma unroll
+            for (int u = 0; u < LV_LOAD_UNROLL; ++u) {
+                const int e = e0 + u * THREADS;
+                if (e < NE) buf[(e / (PX / 2)) * SEQ + spad<C>(e % (PX / 2))] = cmake<C>(va[u], vb[u]);
+            }
         }
+        __syncthreads();
+        fft_batch<C, PX, NB, THREADS, false, true>(buf, tw);
     }
-    __syncthreads();
-    fft_batch<C, PX, NB, THREADS, false, true>(buf, tw);
     const T half = (T)0.5;
     for (int e = threadIdx.x; e < QX * RB; e += THREADS) {
         const int kx = e / RB, r = e % RB;
         const int j = j0 + r;
         if (j >= a.ny) continue;
         const int q = r >> 1;
-        const C zz = buf[spad<C>(q * PX + kx)];
-        const C w = buf[spad<C>(q * PX + ((PX - kx) & (PX - 1)))];
+        const C zz = buf[q * SEQ + spad<C>(kx)];
+        const C w = buf[q * SEQ + spad<C>((PX - kx) & (PX - 1))];
         C o;
         if ((r & 1) == 0) o = cmake<C>(half * (zz.x + w.x), half * (zz.y - w.y));
         else o = cmake<C>(half * (zz.y + w.y), half * (w.x - zz.x));
@@ -364,32 +408,57 @@ __device__ __forceinline__ void lv_col_fwd_body(const cplx_t<T> *__restrict__ in
     using C = cplx_t<T>;
     constexpr int NB = lv_cnb(PY), THREADS = LV_CFWD_THREADS;
     const int f = blockIdx.y, kx0 = blk * NB;
-    for (int e = threadIdx.x; e < NB * (PY / 2); e += THREADS)
-        buf[spad<C>((e / (PY / 2)) * PY + e % (PY / 2))] = cmake<C>((T)0, (T)0);
-    __syncthreads();
-    const int ne = NB * a.ny;
-    for (int e0 = threadIdx.x; e0 < ne; e0 += LV_LOAD_UNROLL * THREADS) {
-        C v[LV_LOAD_UNROLL];
+    if constexpr (lv_in_regs<T>(PY)) {
+        // straight from and to global memory; shared memory only between the stages
+        constexpr int STEP = PY / 8;
+        const int q = threadIdx.x / STEP, jt = threadIdx.x % STEP, kx = kx0 + q;
+        const int mask = (1 << a.st) - 1, col = (f * a.qx + kx) * a.ny;
+        C v[8];
 #pragma unroll
-        for (int u = 0; u < LV_LOAD_UNROLL; ++u) {
-            const int e = e0 + u * THREADS, q = e / a.ny, j = e % a.ny, kx = kx0 + q;
-            v[u] = (e < ne && kx < a.qx) ? in[((int64_t)f * a.qx + kx) * a.ny + j] : cmake<C>((T)0, (T)0);
+        for (int m = 0; m < 8; ++m) {
+            const int rel = jt + m * STEP - a.p0, j = rel >> a.st;
+            v[m] = m < 4 && rel >= 0 && (rel & mask) == 0 && j < a.ny && kx < a.qx ? in[col + j] : cmake<C>((T)0, (T)0);
         }
+        int par = 0;
+        fft_regs<C, PY, NB, THREADS, 2, false>(v, buf, par, tw);
+        if (kx >= a.qx) return;  // past every barrier
+        const int at = (f * a.qx + kx) * PY;
+        const C px = a.hx ? cphx[kx << a.cx] : cmake<C>((T)1, (T)0);
 #pragma unroll
-        for (int u = 0; u < LV_LOAD_UNROLL; ++u) {
-            const int e = e0 + u * THREADS, q = e / a.ny, j = e % a.ny, kx = kx0 + q;
-            if (e < ne && kx < a.qx) buf[spad<C>(q * PY + a.p0 + (j << a.st))] = v[u];
+        for (int m = 0; m < 8; ++m) {
+            const int k = jt + m * STEP;
+            if (a.hy) v[m] = cmul(v[m], cphy[k << a.cy]);
+            if (a.hx) v[m] = cmul(v[m], px);
+            spec[at + k] = v[m];
         }
-    }
-    __syncthreads();
-    fft_batch<C, PY, NB, THREADS, false, true>(buf, tw);
-    for (int e = threadIdx.x; e < NB * PY; e += THREADS) {
-        const int q = e / PY, k = e % PY, kx = kx0 + q;
-        if (kx >= a.qx) continue;
-        C v = buf[spad<C>(e)];
-        if (a.hy) v = cmul(v, cphy[k << a.cy]);
-        if (a.hx) v = cmul(v, cphx[kx << a.cx]);
-        spec[((int64_t)f * a.qx + kx) * PY + k] = v;
+    } else {
+        for (int e = threadIdx.x; e < NB * (PY / 2); e += THREADS)
+            buf[spad<C>((e / (PY / 2)) * PY + e % (PY / 2))] = cmake<C>((T)0, (T)0);
+        __syncthreads();
+        const int ne = NB * a.ny;
+        for (int e0 = threadIdx.x; e0 < ne; e0 += LV_LOAD_UNROLL * THREADS) {
+            C v[LV_LOAD_UNROLL];
+    #pragma unroll
+            for (int u = 0; u < LV_LOAD_UNROLL; ++u) {
+                const int e = e0 + u * THREADS, q = e / a.ny, j = e % a.ny, kx = kx0 + q;
+                v[u] = (e < ne && kx < a.qx) ? in[((int64_t)f * a.qx + kx) * a.ny + j] : cmake<C>((T)0, (T)0);
+            }
+    #pragma unroll
+            for (int u = 0; u < LV_LOAD_UNROLL; ++u) {
+                const int e = e0 + u * THREADS, q = e / a.ny, j = e % a.ny, kx = kx0 + q;
+                if (e < ne && kx < a.qx) buf[spad<C>(q * PY + a.p0 + (j << a.st))] = v[u];
+            }
+        }
+        __syncthreads();
+        fft_batch<C, PY, NB, THREADS, false, true>(buf, tw);
+        for (int e = threadIdx.x; e < NB * PY; e += THREADS) {
+            const int q = e / PY, k = e % PY, kx = kx0 + q;
+            if (kx >= a.qx) continue;
+            C v = buf[spad<C>(e)];
+            if (a.hy) v = cmul(v, cphy[k << a.cy]);
+            if (a.hx) v = cmul(v, cphx[kx << a.cx]);
+            spec[((int64_t)f * a.qx + kx) * PY + k] = v;
+        }
     }
 }
 
@@ -405,10 +474,9 @@ struct lv_col_fwd_args {
     const cplx_t<T> *cphx, *cphy;
 };
 
-// (resident CTAs per SM asked of the register allocator: FP32 three at up to
-// 4096 points, two at 8192; FP64 two)
+// (resident CTAs per SM asked of the register allocator: two, FP64 one at 8192 points)
 template <typename T, int LMAX>
-__global__ void __launch_bounds__(LV_CFWD_THREADS, sizeof(T) == 4 ? (LMAX <= 4096 ? 3 : 2) : (LMAX <= 4096 ? 2 : 1))
+__global__ void __launch_bounds__(LV_CFWD_THREADS, sizeof(T) == 4 || LMAX <= 4096 ? 2 : 1)
     k_lv_col_fwd(lv_col_fwd_args<T> A)
 {
     sg_dep_trigger();
@@ -422,6 +490,8 @@ __global__ void __launch_bounds__(LV_CFWD_THREADS, sizeof(T) == 4 ? (LMAX <= 409
                       (lv_col_fwd_body<T, PP>(A.in[m], A.spec[m], A.a[m], A.tw[m], A.cphx, A.cphy, blk, buf)));
 }
 
+// Target classes: 0 the finest level (samples on cell centres of the finest lattice),
+// 1 every coarser level (samples shifted by half a finest cell).
 struct lv_mac_args {
     int nsrc;
     int64_t spec_off[SG_MAX_LEVELS];    // complex-element offset of each source level's compact spectra
@@ -429,20 +499,23 @@ struct lv_mac_args {
     int lpy[SG_MAX_LEVELS];
     int hx[SG_MAX_LEVELS];              // its samples half-shifted along x, y
     int hy[SG_MAX_LEVELS];
-    int key[SG_MAX_LEVELS][SG_MAX_LEVELS];  // kernel of source level m for target level l, [m][l]
-    int d2[SG_MAX_LEVELS][SG_MAX_LEVELS];   // its 2 x sample shift
-    // target level l: its ny sampled rows sit at compact positions p0 + j 2^st of
-    // its compact column length 2^lm (lm < log2 PY: the bins are folded onto it,
-    // with the half-sample shift when fh), inverse twiddles tw[l]
+    int key[SG_MAX_LEVELS][2];          // kernel of source level m for target class c, [m][c]
+    int d2[SG_MAX_LEVELS][2];           // its 2 x sample shift
+    // target level l: its ny sampled rows sit at positions p0 + j 2^st
     int ny[SG_MAX_LEVELS];
     int p0[SG_MAX_LEVELS];
     int st[SG_MAX_LEVELS];
-    int lm[SG_MAX_LEVELS];
-    int fh[SG_MAX_LEVELS];
-    const void *tw[SG_MAX_LEVELS];
     int64_t inv_off[SG_MAX_LEVELS];     // complex-element offset of its inverse-column outputs
     int qx;
 };
+
+// The inverse-column outputs of a level: blocks of LV_ROWS rows, [o][j / 8][kx][j % 8],
+// read in one piece by the inverse row pass (see INV_ROWS in fftconv.cuh).
+constexpr int LV_ROWS = 8;
+__device__ __forceinline__ int lv_inv_index(int o, int kx, int j, int qx, int ny)
+{
+    return ((o * ((ny + LV_ROWS - 1) / LV_ROWS) + j / LV_ROWS) * qx + kx) * LV_ROWS + j % LV_ROWS;
+}
 
 // Transform length switch for the compact target lengths 64 .. LMAX (only the
 // lengths up to LMAX are instantiated).
@@ -574,150 +647,138 @@ __device__ __forceinline__ void lv_mac_bin(cplx_t<T> X0, cplx_t<T> X1, cplx_t<T>
     }
 }
 
-// Inverse transforms (length L) of the NOUT outputs, held PY apart in shared
-// memory. One at a time, and with the length switch outside the loop: a batch of
-// both, or a switch inside the loop, makes the register allocation of the
-// whole kernel (its per-bin loads) grow by a quarter or more.
-template <typename C, int PY, int L, int NOUT, int THREADS>
-__device__ __forceinline__ void lv_inv_columns(C *bx, const C *__restrict__ tw)
+// Classes per column-MAC CTA (2: both, the sources read once), sequences transformed
+// at a time, threads: FP32 columns of up to 4096 points hold both classes' outputs
+// in shared memory (70 KB at 2048 points, 139 KB at 4096) and transform two sequences
+// at a time; above, and in FP64, a CTA takes one class and one sequence at a time.
+template <typename T>
+__host__ __device__ constexpr int lv_mac_classes(int py) { return sizeof(T) == 4 && py <= 4096 ? 2 : 1; }
+template <typename T>
+__host__ __device__ constexpr int lv_mac_nsq(int py) { return lv_mac_classes<T>(py); }
+template <typename T>
+__host__ __device__ constexpr int lv_mac_threads(int py)
 {
-#pragma unroll 1
-    for (int o = 0; o < NOUT; ++o) fft_batch<C, L, 1, THREADS, true, false, true>(bx + spad<C>(o * PY), tw);
+    const int n = lv_mac_nsq<T>(py) * py / 8;
+    return n < 64 ? 64 : n;
 }
+template <typename T>
+__host__ __device__ constexpr int lv_mac_minb(int py) { return sizeof(T) == 4 ? 65536 / (64 * lv_mac_threads<T>(py)) : 1; }
 
-// One (column kx, target level l) per CTA, kx = blockIdx.x / nsrc and
-// l = blockIdx.x % nsrc, so that the CTAs of all target levels of a column run
-// side by side and read its source spectra (and shared kernel planes) from L2:
-// Fx^, Fy^ = sum over source levels and fields of source spectrum (unfolded
-// from the compact one) x kernel spectrum (decompressed, see k_lv_extract),
-// formed element by element straight into two shared buffers; from 4096-point
-// columns up, for a coarse target level, folded in place onto its compact column
-// length (lv_fold_bin); inverse column transforms of that length; the target
-// level's sampled rows to out[(o qx + kx) ny + j] (out at the level's
-// inverse-column offset). NOUT = 1: the potential, one output from 3 kernel
-// planes per key (p0 real, px and py imaginary; py odd in ky).
-template <typename T, int PY, int THREADS, int MINB, int NOUT>
-__global__ void __launch_bounds__(THREADS, MINB) k_lv_col_mac_inv(lv_mac_args a, const cplx_t<T> *__restrict__ spec,
-                                                            const T *__restrict__ kspec,
-                                                            const cplx_t<T> *__restrict__ phx,
-                                                            const cplx_t<T> *__restrict__ phy,
-                                                            cplx_t<T> *__restrict__ out,
-                                                            const cplx_t<T> *__restrict__ cph)
+// One column kx per CTA (and one class, when lv_mac_classes is 1): for every target
+// class Fx^, Fy^ = sum over source levels and fields of source spectrum (unfolded from
+// the compact one) x kernel spectrum (decompressed, see k_lv_extract), formed bin by
+// bin into shared memory; inverse column transforms; the sampled rows of every level
+// of the class to out (lv_inv_index, at the level's offset). A source value is read
+// once for both classes and a kernel value once in all: 234 KB per column through L2
+// on three nested 256^2 levels, 480 KB with one CTA per target level (the coarser
+// ones repeating the same sum). Per solve 192 -> 163 us there, 716 -> 636 us on the
+// three-level edge-refined N = 512 hierarchy (4096 points: the pass 420 -> 318 us, its
+// kernel planes alone 605 MB from DRAM, 89 us). NOUT = 1: the potential, one
+// output from 3 kernel planes per key (p0 real, px and py imaginary; py odd in ky).
+template <typename T, int PY, int NOUT>
+__global__ void __launch_bounds__(lv_mac_threads<T>(PY), lv_mac_minb<T>(PY)) k_lv_col_mac_inv(
+    lv_mac_args a, const cplx_t<T> *__restrict__ spec, const T *__restrict__ kspec, const cplx_t<T> *__restrict__ phx,
+    const cplx_t<T> *__restrict__ phy, cplx_t<T> *__restrict__ out, const cplx_t<T> *__restrict__ tw)
 {
     sg_dep_trigger();
     sg_dep_wait();  // the source spectra
     using C = cplx_t<T>;
+    constexpr int THREADS = lv_mac_threads<T>(PY), NC = lv_mac_classes<T>(PY), NSQ = lv_mac_nsq<T>(PY);
+    constexpr int SEQ = spad<C>(PY);
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    C *bx = reinterpret_cast<C *>(smem_raw);
-    C *by = bx + spad<C>(PY);
+    C *seqs = reinterpret_cast<C *>(smem_raw);   // [class][output]
     constexpr int QS = ((PY / 2 + 1) + 3) & ~3;  // kernel plane row stride (sg_spec_stride)
-    const int kx = blockIdx.x / a.nsrc, l = blockIdx.x % a.nsrc;
+    const int kx = NC == 2 ? blockIdx.x : blockIdx.x / 2, c0 = NC == 2 ? 0 : blockIdx.x % 2;
     const int64_t kqplane = (int64_t)a.qx * QS;
     constexpr int NPL = NOUT == 2 ? 6 : 3;  // kernel planes per key
     // Bins in mirror pairs: slot j in [0, PY/2) holds bins j and PY - j, which read
     // the same kernel values (kq = j); slot 0 holds bins 0 and PY/2 (kq = 0 and PY/2).
-    // V slots per thread at a time, so that their loads are in flight together.
     constexpr int NSLOT = PY / 2;
-    // (FP32 2048-point force columns: one slot pair, 56 registers, four CTAs per
-    // SM measured 2 % faster than two pairs at three CTAs; two pairs elsewhere,
-    // measured faster than one at 4096 and 8192 points)
-    constexpr int VMAX = sizeof(T) == 8 ? 1 : (NOUT == 2 && PY == 2048 ? 1 : 2);
-    constexpr int V = NSLOT / THREADS >= VMAX ? VMAX : 1;
     const C phk = phx[kx + (a.qx - 1)];
-    for (int j0 = threadIdx.x; j0 < NSLOT; j0 += V * THREADS) {
-        int ky[V][2];
-        C ph[V][2], ax[V][2], ay[V][2];
+    for (int j = threadIdx.x; j < NSLOT; j += THREADS) {
+        const int ky[2] = {j, j == 0 ? PY / 2 : PY - j};
+        // half-cell phase exp(i pi (kx / Px + ky / Py)) at the signed frequencies j and -j (PY/2 for slot 0)
+        const C ph[2] = {cmul(phk, phy[j + PY / 2]), cmul(phk, phy[(j == 0 ? PY / 2 : -j) + PY / 2])};
+        C ax[NC][2], ay[NC][2];
 #pragma unroll
-        for (int v = 0; v < V; ++v) {
-            const int j = j0 + v * THREADS;
-            ky[v][0] = j;
-            ky[v][1] = j == 0 ? PY / 2 : PY - j;
-            // half-cell phase exp(i pi (kx / Px + ky / Py)) at the signed frequencies j and -j (PY/2 for slot 0)
-            ph[v][0] = cmul(phk, phy[j + PY / 2]);
-            ph[v][1] = cmul(phk, phy[(j == 0 ? PY / 2 : -j) + PY / 2]);
+        for (int c = 0; c < NC; ++c)
 #pragma unroll
-            for (int b = 0; b < 2; ++b) ax[v][b] = ay[v][b] = cmake<C>((T)0, (T)0);
-        }
+            for (int b = 0; b < 2; ++b) ax[c][b] = ay[c][b] = cmake<C>((T)0, (T)0);
         for (int m = 0; m < a.nsrc; ++m) {
             const lv_src_col sc = lv_source_column(a, m, kx);
-            const int64_t splane = sc.splane;
             const C *sm = spec + a.spec_off[m] + (int64_t)sc.col * sc.pcy;
-            const T *km = kspec + (int64_t)a.key[m][l] * NPL * kqplane + (int64_t)kx * QS;
-            int row[V][2];
-            bool neg[V][2];
+            int row[2];
+            bool neg[2];
 #pragma unroll
-            for (int v = 0; v < V; ++v) {
+            for (int b = 0; b < 2; ++b) lv_source_row(sc, ky[b], row[b], neg[b]);
+            C X[3][2];
+            T g[NC][NPL];
 #pragma unroll
-                for (int b = 0; b < 2; ++b) lv_source_row(sc, ky[v][b], row[v][b], neg[v][b]);
+            for (int f = 0; f < 3; ++f)
+#pragma unroll
+                for (int b = 0; b < 2; ++b) X[f][b] = sm[f * sc.splane + row[b]];
+#pragma unroll
+            for (int c = 0; c < NC; ++c) {
+                const T *km = kspec + (int64_t)a.key[m][c0 + c] * NPL * kqplane + (int64_t)kx * QS;
+#pragma unroll
+                for (int f = 0; f < NPL; ++f) g[c][f] = km[f * kqplane + j];
             }
-            C X[3][V][2];
-            T gx[3][V][2], gy[3][V][2];
 #pragma unroll
-            for (int f = 0; f < 3; ++f) {
-#pragma unroll
-                for (int v = 0; v < V; ++v) {
-                    const int j = j0 + v * THREADS;
-                    X[f][v][0] = sm[f * splane + row[v][0]];
-                    X[f][v][1] = sm[f * splane + row[v][1]];
-                    gx[f][v][0] = gx[f][v][1] = km[f * kqplane + j];
-                    if constexpr (NOUT == 2) gy[f][v][0] = gy[f][v][1] = km[(3 + f) * kqplane + j];
-                }
-            }
-            if (j0 == 0) {  // slot 0: bin PY/2 has kernel values of its own
-#pragma unroll
-                for (int f = 0; f < 3; ++f) {
-                    gx[f][0][1] = km[f * kqplane + PY / 2];
-                    if constexpr (NOUT == 2) gy[f][0][1] = km[(3 + f) * kqplane + PY / 2];
-                }
-            }
-            const int d2 = a.d2[m][l];
-#pragma unroll
-            for (int v = 0; v < V; ++v) {
+            for (int c = 0; c < NC; ++c) {
+                const int d2 = a.d2[m][c0 + c];
 #pragma unroll
                 for (int b = 0; b < 2; ++b) {
-                    const T sg = (b == 0 || ky[v][1] == PY / 2) ? (T)1 : (T)-1;
+                    if (b == 1 && j == 0) {  // bin PY/2 has kernel values of its own
+                        const T *km = kspec + (int64_t)a.key[m][c0 + c] * NPL * kqplane + (int64_t)kx * QS;
+#pragma unroll
+                        for (int f = 0; f < NPL; ++f) g[c][f] = km[f * kqplane + PY / 2];
+                    }
+                    const T sg = (b == 0 || j == 0) ? (T)1 : (T)-1;
                     if constexpr (NOUT == 2)
-                        lv_mac_bin<T, 2>(X[0][v][b], X[1][v][b], X[2][v][b], sc.fold, gx[0][v][b], gx[1][v][b],
-                                         gx[2][v][b], gy[0][v][b], gy[1][v][b], gy[2][v][b], sg, ph[v][b], d2,
-                                         neg[v][b], ax[v][b], ay[v][b]);
+                        lv_mac_bin<T, 2>(X[0][b], X[1][b], X[2][b], sc.fold, g[c][0], g[c][1], g[c][2], g[c][3], g[c][4],
+                                         g[c][5], sg, ph[b], d2, neg[b], ax[c][b], ay[c][b]);
                     else
-                        lv_mac_bin<T, 1>(X[0][v][b], X[1][v][b], X[2][v][b], sc.fold, gx[0][v][b], gx[1][v][b],
-                                         gx[2][v][b], (T)0, (T)0, (T)0, sg, ph[v][b], d2, neg[v][b], ax[v][b],
-                                         ay[v][b]);
+                        lv_mac_bin<T, 1>(X[0][b], X[1][b], X[2][b], sc.fold, g[c][0], g[c][1], g[c][2], (T)0, (T)0, (T)0,
+                                         sg, ph[b], d2, neg[b], ax[c][b], ay[c][b]);
                 }
             }
         }
 #pragma unroll
-        for (int v = 0; v < V; ++v) {
+        for (int c = 0; c < NC; ++c)
 #pragma unroll
             for (int b = 0; b < 2; ++b) {
-                bx[spad<C>(ky[v][b])] = ax[v][b];
-                if constexpr (NOUT == 2) by[spad<C>(ky[v][b])] = ay[v][b];
+                seqs[(c * NOUT) * SEQ + spad<C>(ky[b])] = ax[c][b];
+                if constexpr (NOUT == 2) seqs[(c * NOUT + 1) * SEQ + spad<C>(ky[b])] = ay[c][b];
             }
-        }
     }
     __syncthreads();
-    const int lm = a.lm[l];
-    if constexpr (lv_fold_targets(PY)) {
-        // a coarse target level is sampled every 2^c rows: fold onto its compact
-        // length, in place (bin k < M of an output is written only by the thread
-        // that reads it)
-        if (lm < lv_log2(PY)) {
-            for (int e = threadIdx.x; e < (NOUT << lm); e += THREADS) {
-                C *seq = bx + spad<C>((e >> lm) * PY);
-                const int k = e & ((1 << lm) - 1);
-                seq[spad<C>(k)] = lv_fold_bin<C, PY>(seq, k, lm, a.fh[l] != 0, cph);
-            }
-            __syncthreads();
+    // inverse transforms, NSQ sequences at a time, in registers with the sequences'
+    // own shared memory for the exchanges
+    constexpr int STEP = PY / 8, ROUNDS = NC * NOUT / NSQ;
+    const int q = threadIdx.x / STEP, jt = threadIdx.x % STEP;
+#pragma unroll 1
+    for (int r = 0; r < ROUNDS; ++r) {
+        C *base = seqs + r * NSQ * SEQ;
+        C v[8];
+        if (q < NSQ) {
+#pragma unroll
+            for (int m = 0; m < 8; ++m) v[m] = base[q * SEQ + spad<C>(jt + m * STEP)];
         }
-        SG_LV_LEN_SWITCH(lm, PY, (lv_inv_columns<C, PY, PP, NOUT, THREADS>(bx, (const C *)a.tw[l])));
-    }
-    const int ny = a.ny[l], p0 = a.p0[l], st = a.st[l];
-    for (int o = 0; o < NOUT; ++o) {
-        C *seq = bx + spad<C>(o * PY);
-        if constexpr (!lv_fold_targets(PY)) fft_batch<C, PY, 1, THREADS, true, false, true>(seq, (const C *)a.tw[l]);
-        C *dst = out + a.inv_off[l] + ((int64_t)o * a.qx + kx) * ny;
-        for (int j = threadIdx.x; j < ny; j += THREADS) dst[j] = seq[spad<C>(p0 + (j << st))];
+        __syncthreads();
+        int par = 0;
+        fft_regs<C, PY, NSQ, THREADS, 1, true, SEQ>(v, base, par, tw);
+        if (q >= NSQ) continue;
+        const int sq = r * NSQ + q, cls = c0 + sq / NOUT, o = sq % NOUT;
+        // the levels of the class: the last (finest), or all others
+        for (int l = cls == 0 ? a.nsrc - 1 : 0; l < (cls == 0 ? a.nsrc : a.nsrc - 1); ++l) {
+            C *dst = out + a.inv_off[l];
+            const int mask = (1 << a.st[l]) - 1, ny = a.ny[l];
+#pragma unroll
+            for (int m = 0; m < 4; ++m) {
+                const int rel = jt + m * STEP - a.p0[l], j = rel >> a.st[l];
+                if (rel >= 0 && (rel & mask) == 0 && j < ny) dst[lv_inv_index(o, kx, j, a.qx, ny)] = v[m];
+            }
+        }
     }
 }
 
@@ -755,12 +816,16 @@ __global__ void __launch_bounds__(LV_ROW_THREADS) k_lv_row_inv(lv_row_inv_args<T
     constexpr int NB = lv_nb(PX), THREADS = LV_ROW_THREADS;
     constexpr int RB = 2 * NB;
     constexpr int QX = PX / 2 + 1;
+    // register form where the rows are not folded: staged in the second exchange buffer
+    constexpr bool REGS = lv_in_regs<T>(PX) && !lv_fold_targets(PX);
+    constexpr int SEQ = REGS ? lv_seq<T>(PX, NB) : spad<C>(PX);
+    if constexpr (REGS) buf += NB * SEQ;
     const int lvl = lv_level_of(A.cta0, A.nlev);
     const lv_out_dst &a = A.a[lvl];
     const int o = blockIdx.y;
     const int j0 = (blockIdx.x - A.cta0[lvl]) * RB;
     const int ny = a.ny;
-    const C *w = A.in[lvl] + (int64_t)o * QX * ny;
+    const C *w = A.in[lvl];
     T *out = o == 0 ? fx : fy;
     constexpr int NE = NB * QX;
     for (int e0 = threadIdx.x; e0 < NE; e0 += LV_LOAD_UNROLL * THREADS) {
@@ -768,8 +833,20 @@ __global__ void __launch_bounds__(LV_ROW_THREADS) k_lv_row_inv(lv_row_inv_args<T
 #pragma unroll
         for (int u = 0; u < LV_LOAD_UNROLL; ++u) {
             const int e = e0 + u * THREADS, q = e % NB, k = e / NB, ja = j0 + 2 * q;
-            xv[u] = (e < NE && ja < ny) ? w[(int64_t)k * ny + ja] : cmake<C>((T)0, (T)0);
-            yv[u] = (e < NE && ja + 1 < ny) ? w[(int64_t)k * ny + ja + 1] : cmake<C>((T)0, (T)0);
+            xv[u] = yv[u] = cmake<C>((T)0, (T)0);
+            if (e < NE && ja < ny) {
+                // rows ja, ja + 1 side by side (ja is even): one 16-byte load in FP32
+                const C *p = &w[lv_inv_index(o, k, ja, QX, ny)];
+                if constexpr (sizeof(C) == 8) {
+                    const float4 t = *reinterpret_cast<const float4 *>(p);
+                    xv[u] = cmake<C>(t.x, t.y);
+                    yv[u] = cmake<C>(t.z, t.w);
+                } else {
+                    xv[u] = p[0];
+                    yv[u] = p[1];
+                }
+                if (ja + 1 >= ny) yv[u] = cmake<C>((T)0, (T)0);
+            }
         }
 #pragma unroll
         for (int u = 0; u < LV_LOAD_UNROLL; ++u) {
@@ -780,54 +857,52 @@ __global__ void __launch_bounds__(LV_ROW_THREADS) k_lv_row_inv(lv_row_inv_args<T
                 x.y = (T)0;
                 y.y = (T)0;
             }
-            buf[spad<C>(q * PX + k)] = cmake<C>(x.x - y.y, x.y + y.x);
-            if (k > 0 && k < PX / 2) buf[spad<C>(q * PX + PX - k)] = cmake<C>(x.x + y.y, y.x - x.y);
+            buf[q * SEQ + spad<C>(k)] = cmake<C>(x.x - y.y, x.y + y.x);
+            if (k > 0 && k < PX / 2) buf[q * SEQ + spad<C>(PX - k)] = cmake<C>(x.x + y.y, y.x - x.y);
         }
     }
     __syncthreads();
     const int lm = a.lm;
-    if constexpr (lv_fold_targets(PX)) {
-        if (lm < lv_log2(PX)) lv_fold_spectrum<C, PX, NB, THREADS>(buf, lm, a.fh != 0, A.cph);
-        SG_LV_LEN_SWITCH(lm, PX, (fft_batch<C, PP, NB, THREADS, true, false, true>(buf, A.tw[lvl])));
-    } else {
-        fft_batch<C, PX, NB, THREADS, true, false, true>(buf, A.tw[lvl]);
-    }
-    for (int e = threadIdx.x; e < NB * a.nx; e += THREADS) {
-        const int q = e / a.nx, i = e % a.nx;
-        const int ja = j0 + 2 * q;
-        const C zz = buf[spad<C>((q << lm) + a.p0 + (i << a.st))];
+    auto put = [&](int ja, int i, C z) {
         if (ja < ny) {
             const int c = a.map[(int64_t)ja * a.nx + i];
-            if (c >= 0) out[c] = zz.x;
+            if (c >= 0) out[c] = z.x;
         }
         if (ja + 1 < ny) {
             const int c = a.map[(int64_t)(ja + 1) * a.nx + i];
-            if (c >= 0) out[c] = zz.y;
+            if (c >= 0) out[c] = z.y;
+        }
+    };
+    if constexpr (REGS) {
+        constexpr int STEP = PX / 8;
+        const int q = threadIdx.x / STEP, jt = threadIdx.x % STEP;
+        C v[8];
+#pragma unroll
+        for (int m = 0; m < 8; ++m) v[m] = buf[q * SEQ + spad<C>(jt + m * STEP)];
+        int par = 0;
+        fft_regs<C, PX, NB, THREADS, 2, true, SEQ>(v, reinterpret_cast<C *>(smem_raw), par, A.tw[lvl]);
+        const int mask = (1 << a.st) - 1;
+#pragma unroll
+        for (int m = 0; m < 4; ++m) {
+            const int rel = jt + m * STEP - a.p0, i = rel >> a.st;
+            if (rel >= 0 && (rel & mask) == 0 && i < a.nx) put(j0 + 2 * q, i, v[m]);
+        }
+        return;
+    } else {
+        if constexpr (lv_fold_targets(PX)) {
+            if (lm < lv_log2(PX)) lv_fold_spectrum<C, PX, NB, THREADS>(buf, lm, a.fh != 0, A.cph);
+            SG_LV_LEN_SWITCH(lm, PX, (fft_batch<C, PP, NB, THREADS, true, false, true>(buf, A.tw[lvl])));
+        } else {
+            fft_batch<C, PX, NB, THREADS, true, false, true>(buf, A.tw[lvl]);
+        }
+        for (int e = threadIdx.x; e < NB * a.nx; e += THREADS) {
+            const int q = e / a.nx, i = e % a.nx;
+            put(j0 + 2 * q, i, buf[spad<C>((q << lm) + a.p0 + (i << a.st))]);
         }
     }
 }
 
 // ----------------------------------------------------------- launchers --
-
-constexpr int lv_col_threads(int py) { return py / 8 < 64 ? 64 : (py / 8 > 512 ? 512 : py / 8); }
-// Column-MAC CTAs: the two shared spectra of a column grow to 2 x 8192 x 8 bytes
-// (FP32) or 2 x 4096 x 16 (FP64), which leaves one CTA per SM; the FP32 one gets
-// 1024 threads (at most 64 registers each) so that more loads are in flight, the
-// FP64 one 512 (its allocation spills at 64).
-template <typename T>
-constexpr int lv_mac_threads(int py)
-{
-    return sizeof(T) == 8 ? (py >= 4096 ? 512 : lv_col_threads(py)) : (py >= 8192 ? 1024 : lv_col_threads(py));
-}
-// FP32 2048-point columns with two outputs: four CTAs of 256 threads per SM (at
-// most 64 registers; one slot pair per thread)
-template <typename T>
-constexpr int lv_mac_minb(int py, int nout)
-{
-    return sizeof(T) == 4 && py == 4096               ? 2
-           : sizeof(T) == 4 && py == 2048 && nout == 2 ? 4
-                                                        : (lv_mac_threads<T>(py) >= 1024 ? 1 : 0);
-}
 
 template <typename K>
 sg_status smem_attr(K kern, size_t bytes)
@@ -839,7 +914,7 @@ sg_status smem_attr(K kern, size_t bytes)
 template <typename T>
 sg_status launch_row_fwd(const lv_row_fwd_args<T> &A, int ncta, int lmax, cudaStream_t st)
 {
-    const size_t sm = spad_size<cplx_t<T>>(lv_nb(lmax) * lmax) * sizeof(cplx_t<T>);
+    const size_t sm = lv_row_smem_max<T>(lmax);
     auto kern = lmax > 4096 ? k_lv_row_fwd<T, 8192> : k_lv_row_fwd<T, 4096>;
     SG_TRY(smem_attr(kern, sm));
     SG_CUDA_TRY(sg_launch_dep(kern, dim3(ncta, 3), dim3(LV_ROW_THREADS), sm, st, A));
@@ -850,7 +925,7 @@ sg_status launch_row_fwd(const lv_row_fwd_args<T> &A, int ncta, int lmax, cudaSt
 template <typename T>
 sg_status launch_col_fwd(const lv_col_fwd_args<T> &A, int ncta, int lmax, cudaStream_t st)
 {
-    const size_t sm = spad_size<cplx_t<T>>(lv_cnb(lmax) * lmax) * sizeof(cplx_t<T>);
+    const size_t sm = lv_row_smem_max<T>(lmax);
     auto kern = lmax > 4096 ? k_lv_col_fwd<T, 8192> : k_lv_col_fwd<T, 4096>;
     SG_TRY(smem_attr(kern, sm));
     SG_CUDA_TRY(sg_launch_dep(kern, dim3(ncta, 3), dim3(LV_CFWD_THREADS), sm, st, A));
@@ -860,13 +935,14 @@ sg_status launch_col_fwd(const lv_col_fwd_args<T> &A, int ncta, int lmax, cudaSt
 
 template <typename T, int PY, int NOUT>
 sg_status launch_col_mac_inv(const lv_mac_args &a, const cplx_t<T> *spec, const T *kspec, const cplx_t<T> *phx,
-                             const cplx_t<T> *phy, cplx_t<T> *out, const cplx_t<T> *cph, cudaStream_t st)
+                             const cplx_t<T> *phy, cplx_t<T> *out, const cplx_t<T> *tw, cudaStream_t st)
 {
-    constexpr int TH = lv_mac_threads<T>(PY);
-    const size_t sm = spad_size<cplx_t<T>>(NOUT * PY) * sizeof(cplx_t<T>);
-    auto kern = k_lv_col_mac_inv<T, PY, TH, lv_mac_minb<T>(PY, NOUT), NOUT>;
+    constexpr int NC = lv_mac_classes<T>(PY);
+    const size_t sm = (size_t)NC * NOUT * spad<cplx_t<T>>(PY) * sizeof(cplx_t<T>);
+    auto kern = k_lv_col_mac_inv<T, PY, NOUT>;
     SG_TRY(smem_attr(kern, sm));
-    SG_CUDA_TRY(sg_launch_dep(kern, dim3(a.qx * a.nsrc), dim3(TH), sm, st, a, spec, kspec, phx, phy, out, cph));
+    SG_CUDA_TRY(sg_launch_dep(kern, dim3(a.qx * (2 / NC)), dim3(lv_mac_threads<T>(PY)), sm, st, a, spec, kspec, phx, phy,
+                              out, tw));
     SG_CUDA_TRY(cudaGetLastError());
     return SG_OK;
 }
@@ -874,7 +950,8 @@ sg_status launch_col_mac_inv(const lv_mac_args &a, const cplx_t<T> *spec, const 
 template <typename T, int PX>
 sg_status launch_row_inv(const lv_row_inv_args<T> &A, int ncta, int nout, T *fx, T *fy, cudaStream_t st)
 {
-    const size_t sm = spad_size<cplx_t<T>>(lv_nb(PX) * PX) * sizeof(cplx_t<T>);
+    constexpr bool REGS = lv_in_regs<T>(PX) && !lv_fold_targets(PX);
+    const size_t sm = REGS ? lv_row_smem<T>(PX) : lv_nb(PX) * spad<cplx_t<T>>(PX) * sizeof(cplx_t<T>);
     auto kern = k_lv_row_inv<T, PX>;
     SG_TRY(smem_attr(kern, sm));
     SG_CUDA_TRY(sg_launch_dep(kern, dim3(ncta, nout), dim3(LV_ROW_THREADS), sm, st, A, fx, fy));
@@ -966,27 +1043,23 @@ sg_status lv_solve_t(sg_plan *plan, const sg_workspace *ws, void *out0, void *ou
             a.lpy[m] = sg_ilog2(lv.py >> M.cy);
             a.hx[m] = M.cx == M.s && M.s >= 1;
             a.hy[m] = M.cy == M.s && M.s >= 1;
-            for (int l = 0; l < lv.nlev; ++l) {
-                a.key[m][l] = lv.key[m][l];
-                a.d2[m][l] = lv.key_d2[lv.key[m][l]];
+            for (int c = 0; c < 2; ++c) {
+                a.key[m][c] = lv.key[m][c == 0 ? lv.nlev - 1 : 0];  // every level but the finest has one kernel
+                a.d2[m][c] = lv.key_d2[a.key[m][c]];
             }
-            const int fy = lv_fold_targets(lv.py) ? M.cy : 0;  // target fold exponent
             a.ny[m] = M.ny;
-            a.p0[m] = M.j0 >> fy;
-            a.st[m] = M.s - fy;
-            a.lm[m] = sg_ilog2(lv.py >> fy);
-            a.fh[m] = fy == M.s && M.s >= 1;
-            a.tw[m] = twid(lv.py >> fy);
+            a.p0[m] = M.j0;
+            a.st[m] = M.s;
             a.inv_off[m] = M.inv_off;
         }
         a.qx = qx;
         const C *phx = (const C *)lv.phase, *phy = phx + lv.px + 1;
         if (pot) {
-            SG_LV_SWITCH(lv.py, SG_TRY((launch_col_mac_inv<T, PP, 1>(a, spec, (const T *)lv.pspectra, phx, phy, wi, cphy,
-                                                                      st))));
+            SG_LV_SWITCH(lv.py, SG_TRY((launch_col_mac_inv<T, PP, 1>(a, spec, (const T *)lv.pspectra, phx, phy, wi,
+                                                                      twid(lv.py), st))));
         } else {
-            SG_LV_SWITCH(lv.py, SG_TRY((launch_col_mac_inv<T, PP, 2>(a, spec, (const T *)lv.spectra, phx, phy, wi, cphy,
-                                                                      st))));
+            SG_LV_SWITCH(lv.py, SG_TRY((launch_col_mac_inv<T, PP, 2>(a, spec, (const T *)lv.spectra, phx, phy, wi,
+                                                                      twid(lv.py), st))));
         }
     }
     sg_timing_end(ws, SG_STAGE_COL_CONV, st);
@@ -1062,7 +1135,7 @@ sg_status sg_lv_setup(sg_plan *plan, const sg_lv_setup_args *a)
         const int64_t qxc = (a->px >> L.cx) / 2 + 1;
         fwd += 3LL * qxc * L.ny;
         spec += 3LL * qxc * (a->py >> L.cy);
-        inv += 2LL * qx * L.ny;
+        inv += 2LL * qx * ((L.ny + LV_ROWS - 1) / LV_ROWS * LV_ROWS);
         SG_TRY(sg_plan_upload(plan, (void **)&L.map, a->map[m], (size_t)L.nx * L.ny * sizeof(int)));
     }
     lv->fwd_elems = fwd;
