@@ -947,6 +947,15 @@ __host__ __device__ constexpr bool col_feasible_t()
     return CB >= 1 && CB * PY / 8 >= 32 && CB * PY / 8 <= 512 && col_smem_bytes<T, PY, CB, NPL>() <= 200 * 1024;
 }
 
+// Dynamic shared memory beyond the 48 KB every kernel may use without asking.
+template <typename K>
+inline sg_status smem_limit(K kern, size_t smem)
+{
+    if (smem > 48 * 1024)
+        SG_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    return SG_OK;
+}
+
 // Dispatchers (explicitly instantiated for float and double in their units).
 // A batch (one launch for `nmem` members of one padded length): `many` is a
 // device array of the members' arguments and `maxny` their largest row count;

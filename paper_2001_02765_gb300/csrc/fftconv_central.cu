@@ -13,7 +13,7 @@ sg_status launch_cols_central(const col_args<T> &one, const col_args<T> *many, b
     constexpr int THREADS = CB * PY / 8;
     const size_t smem = (size_t)col_smem_bytes<T, PY, CB, 6, col_central_nbuf<T, PY, CB, BATCH>()>();
     auto kern = k_col_conv_central<T, PY, CB, THREADS, BATCH>;
-    SG_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    SG_TRY(smem_limit(kern, smem));
     dim3 grid((qx + CB - 1) / CB, 1, BATCH ? bs.nmem : 1);
     if (dep) SG_CUDA_TRY(sg_launch_dep(kern, grid, dim3(THREADS), smem, st, one, many, qx, tw, err));
     else kern<<<grid, THREADS, smem, st>>>(one, many, qx, tw, err);
@@ -54,11 +54,11 @@ sg_status launch_edge_cols(const edge_args<T> &one, const edge_args<T> *many, ba
     // a dependent launch after the row pass (see k_edge_cols)
     if (many) {
         auto kern = k_edge_cols<T, PY, THREADS, true>;
-        SG_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        SG_TRY(smem_limit(kern, smem));
         SG_CUDA_TRY(sg_launch_dep(kern, dim3(1, 1, bs.nmem), dim3(THREADS), smem, st, one, many, tw));
     } else {
         auto kern = k_edge_cols<T, PY, THREADS, false>;
-        SG_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        SG_TRY(smem_limit(kern, smem));
         SG_CUDA_TRY(sg_launch_dep(kern, dim3(1), dim3(THREADS), smem, st, one, many, tw));
     }
     SG_CUDA_TRY(cudaGetLastError());

@@ -15,7 +15,7 @@ sg_status launch_cols(const col_args<T> &one, const col_args<T> *many, batch_sha
     constexpr int THREADS = CB * PY / 8;
     const size_t smem = (size_t)col_smem_bytes<T, PY, CB, NOUT == 3 ? 9 : (NOUT == 1 ? 3 : 6)>();
     auto kern = k_col_conv<T, PY, CB, THREADS, NOUT, BATCH>;
-    SG_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    SG_TRY(smem_limit(kern, smem));
     dim3 grid((qx + CB - 1) / CB, 1, BATCH ? bs.nmem : 1);
     if (dep) SG_CUDA_TRY(sg_launch_dep(kern, grid, dim3(THREADS), smem, st, one, many, qx, nf, tw, err));
     else kern<<<grid, THREADS, smem, st>>>(one, many, qx, nf, tw, err);

@@ -18,7 +18,7 @@ sg_status launch_rows_fwd(const row_fwd_args<T> &one, const row_fwd_args<T> *man
     constexpr int THREADS = row_threads(PX, NB);
     const size_t smem = (size_t)row_smem_bytes<T>(PX, NB, THREADS);
     auto kern = k_row_fwd<T, PX, NB, THREADS, BATCH, AFTER_EDGE>;
-    SG_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    SG_TRY(smem_limit(kern, smem));
     const int ny = BATCH ? bs.maxny : one.src.ny;
     dim3 grid((ny + 2 * NB - 1) / (2 * NB), nf, BATCH ? bs.nmem : 1);
     SG_CUDA_TRY(sg_launch_dep(kern, grid, dim3(THREADS), smem, st, one, many, tw));

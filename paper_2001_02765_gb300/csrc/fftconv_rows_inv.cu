@@ -13,7 +13,7 @@ sg_status launch_rows_inv(const row_inv_args<T> &one, const row_inv_args<T> *man
     constexpr int THREADS = row_threads(PX, NB);
     const size_t smem = (size_t)row_smem_bytes<T>(PX, NB, THREADS);
     auto kern = k_row_inv<T, PX, NB, THREADS, BATCH>;
-    SG_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    SG_TRY(smem_limit(kern, smem));
     const int ny = BATCH ? bs.maxny : one.ny;
     dim3 grid((ny + 2 * NB - 1) / (2 * NB), nout, BATCH ? bs.nmem : 1);
     SG_CUDA_TRY(sg_launch_dep(kern, grid, dim3(THREADS), smem, st, one, many, tw));

@@ -520,6 +520,23 @@ def sg_zones_links(zone_args):
 
 # ------------------------------------------------------------ convenience --
 
+_torch = None
+_raw_stream = None
+
+
+def _torch_mod():
+    """torch, imported at the first use of a Plan (the low-level names need none)."""
+    global _torch, _raw_stream
+    if _torch is None:
+        import torch
+        _torch = torch
+        # the current stream as a number, without building a Stream object (2.9 us of
+        # a call on a Grace core); absent in some builds
+        get, dev = getattr(torch._C, "_cuda_getCurrentRawStream", None), getattr(torch._C, "_cuda_getDevice", None)
+        _raw_stream = (lambda: get(dev())) if get and dev else (lambda: torch.cuda.current_stream().cuda_stream)
+    return _torch
+
+
 class Plan:
     """A plan for one geometry; fields are torch tensors on the current CUDA device.
 
@@ -562,8 +579,14 @@ class Plan:
         return sg_kernel_tables(self.handle, patch, w, p[1], p[2])
 
     def _torch_dtype(self):
-        import torch
+        torch = _torch_mod()
         return torch.float32 if self.precision == SG_FP32 else torch.float64
+
+    def _check_fields(self, n, *fields):
+        dt = self._torch_dtype()
+        for t in fields:
+            if t is not None and (t.dtype is not dt or not t.is_cuda or t.numel() != n or not t.is_contiguous()):
+                raise ValueError("fields must be contiguous %s CUDA tensors of %d elements" % (dt, n))
 
     def empty_fields(self, n=2):
         import torch
@@ -571,43 +594,34 @@ class Plan:
 
     def force(self, sigma, dx=None, dy=None, fx=None, fy=None, stream=None):
         """Enqueue a solve on `stream` (default: torch's current stream); returns (fx, fy)."""
-        import torch
-        dt = self._torch_dtype()
-        for t in (sigma, dx, dy, fx, fy):
-            if t is not None and (t.dtype != dt or not t.is_cuda or not t.is_contiguous() or t.numel() != self.ncells):
-                raise ValueError("fields must be contiguous %s CUDA tensors of %d elements" % (dt, self.ncells))
+        torch = _torch_mod()
+        self._check_fields(self.ncells, sigma, dx, dy, fx, fy)
         if fx is None:
             fx = torch.empty_like(sigma)
         if fy is None:
             fy = torch.empty_like(sigma)
-        st = (stream or torch.cuda.current_stream()).cuda_stream
+        st = stream.cuda_stream if stream else _raw_stream()
         sg_force(self.handle, sigma.data_ptr(), dx.data_ptr() if dx is not None else 0,
                  dy.data_ptr() if dy is not None else 0, fx.data_ptr(), fy.data_ptr(), st)
         return fx, fy
 
     def force3(self, sigma, dx=None, dy=None, stream=None):
         """Enqueue a solve with Fz (see sg_force3); returns (fx, fy, fz)."""
-        import torch
-        dt = self._torch_dtype()
-        for t in (sigma, dx, dy):
-            if t is not None and (t.dtype != dt or not t.is_cuda or not t.is_contiguous() or t.numel() != self.ncells):
-                raise ValueError("fields must be contiguous %s CUDA tensors of %d elements" % (dt, self.ncells))
+        torch = _torch_mod()
+        self._check_fields(self.ncells, sigma, dx, dy)
         fx, fy, fz = (torch.empty_like(sigma) for _ in range(3))
-        st = (stream or torch.cuda.current_stream()).cuda_stream
+        st = stream.cuda_stream if stream else _raw_stream()
         sg_force3(self.handle, sigma.data_ptr(), dx.data_ptr() if dx is not None else 0,
                   dy.data_ptr() if dy is not None else 0, fx.data_ptr(), fy.data_ptr(), fz.data_ptr(), st)
         return fx, fy, fz
 
     def potential(self, sigma, dx=None, dy=None, phi=None, stream=None):
         """Enqueue the mid-plane potential (see sg_potential); returns phi."""
-        import torch
-        dt = self._torch_dtype()
-        for t in (sigma, dx, dy, phi):
-            if t is not None and (t.dtype != dt or not t.is_cuda or not t.is_contiguous() or t.numel() != self.ncells):
-                raise ValueError("fields must be contiguous %s CUDA tensors of %d elements" % (dt, self.ncells))
+        torch = _torch_mod()
+        self._check_fields(self.ncells, sigma, dx, dy, phi)
         if phi is None:
             phi = torch.empty_like(sigma)
-        st = (stream or torch.cuda.current_stream()).cuda_stream
+        st = stream.cuda_stream if stream else _raw_stream()
         sg_potential(self.handle, sigma.data_ptr(), dx.data_ptr() if dx is not None else 0,
                      dy.data_ptr() if dy is not None else 0, phi.data_ptr(), st)
         return phi
@@ -684,30 +698,24 @@ class ZonePlan(Plan):
 
     def force_zones(self, sigma, dx=None, dy=None, fx=None, fy=None, stream=None):
         """Enqueue a solve on zone-ordered tensors; returns (fx, fy), 0 at non-leaf zones."""
-        import torch
-        dt = self._torch_dtype()
-        for t in (sigma, dx, dy, fx, fy):
-            if t is not None and (t.dtype != dt or not t.is_cuda or not t.is_contiguous() or t.numel() != self.nzones):
-                raise ValueError("fields must be contiguous %s CUDA tensors of %d elements" % (dt, self.nzones))
+        torch = _torch_mod()
+        self._check_fields(self.nzones, sigma, dx, dy, fx, fy)
         if fx is None:
             fx = torch.empty_like(sigma)
         if fy is None:
             fy = torch.empty_like(sigma)
-        st = (stream or torch.cuda.current_stream()).cuda_stream
+        st = stream.cuda_stream if stream else _raw_stream()
         sg_force_zones(self.handle, sigma.data_ptr(), dx.data_ptr() if dx is not None else 0,
                        dy.data_ptr() if dy is not None else 0, fx.data_ptr(), fy.data_ptr(), st)
         return fx, fy
 
     def potential_zones(self, sigma, dx=None, dy=None, phi=None, stream=None):
         """Enqueue the potential on zone-ordered tensors; returns phi, 0 at non-leaf zones."""
-        import torch
-        dt = self._torch_dtype()
-        for t in (sigma, dx, dy, phi):
-            if t is not None and (t.dtype != dt or not t.is_cuda or not t.is_contiguous() or t.numel() != self.nzones):
-                raise ValueError("fields must be contiguous %s CUDA tensors of %d elements" % (dt, self.nzones))
+        torch = _torch_mod()
+        self._check_fields(self.nzones, sigma, dx, dy, phi)
         if phi is None:
             phi = torch.empty_like(sigma)
-        st = (stream or torch.cuda.current_stream()).cuda_stream
+        st = stream.cuda_stream if stream else _raw_stream()
         sg_potential_zones(self.handle, sigma.data_ptr(), dx.data_ptr() if dx is not None else 0,
                            dy.data_ptr() if dy is not None else 0, phi.data_ptr(), st)
         return phi
