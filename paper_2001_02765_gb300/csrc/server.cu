@@ -143,8 +143,6 @@ void finalize(sg_server *s, sg_request *r)
     r->state.store(RQ_FINISHED);
 }
 
-// Start a queued request on a free slot (lock held). Returns false when its
-// workspace cannot be allocated now (it stays queued).
 // The request's workspace, stream-ordered from the server's pool on `st`, its
 // error word cleared; false (nothing held) when it cannot be allocated now.
 bool alloc_ws(sg_server *s, sg_request *r, cudaStream_t st)
@@ -174,18 +172,58 @@ bool alloc_ws(sg_server *s, sg_request *r, cudaStream_t st)
     return true;
 }
 
-bool start(sg_server *s, sg_request *r)
+// Take requests off the queue for a free slot (lock held): they count as running
+// from here on, so that the lock can be released while they are launched.
+void claim(sg_server *s, const std::vector<sg_request *> &mem, int slot)
+{
+    const double t = now_s();
+    for (sg_request *r : mem) {
+        s->queue.erase(std::find(s->queue.begin(), s->queue.end(), r));
+        r->slot = slot;
+        r->t_start = t;
+        r->state.store(RQ_RUNNING);
+        s->bytes_in_use += r->bytes;
+        s->running.push_back(r);
+    }
+    s->peak_bytes = std::max(s->peak_bytes, s->bytes_in_use);
+    s->err_host[slot] = 0;
+}
+
+// Undo claim (lock held): back to the head of the queue, in order.
+void unclaim(sg_server *s, const std::vector<sg_request *> &mem, int slot)
+{
+    for (size_t k = mem.size(); k-- > 0;) {
+        sg_request *r = mem[k];
+        s->running.erase(std::find(s->running.begin(), s->running.end(), r));
+        s->bytes_in_use -= r->bytes;
+        if (s->stop) {  // the server is being destroyed: as the queued ones
+            r->result = SG_ECANCELLED;
+            r->state.store(RQ_FINISHED);
+            s->cancelled++;
+        } else {
+            r->state.store(RQ_QUEUED);
+            s->queue.push_front(r);
+        }
+    }
+    s->free_slots.push_back(slot);
+}
+
+// Start a queued request on a free slot (lock held on entry and return, released
+// while the workspace is allocated and the solve launched, so that submissions do
+// not wait for that). Returns false when its workspace cannot be allocated now (it
+// is queued again).
+bool start(sg_server *s, sg_request *r, std::unique_lock<std::mutex> &lock)
 {
     const int slot = s->free_slots.back();
     cudaStream_t st = s->streams[slot];
-    if (!alloc_ws(s, r, st)) return false;
     s->free_slots.pop_back();
-    r->slot = slot;
-    s->bytes_in_use += r->bytes;
-    s->peak_bytes = std::max(s->peak_bytes, s->bytes_in_use);
-    r->t_start = now_s();
-    r->state.store(RQ_RUNNING);
-    s->err_host[slot] = 0;
+    claim(s, {r}, slot);
+    lock.unlock();
+    if (!alloc_ws(s, r, st)) {
+        lock.lock();
+        unclaim(s, {r}, slot);
+        return false;
+    }
     r->result = sg_force_ws(r->plan, &r->ws, r->sigma, r->dx, r->dy, r->fx, r->fy, st);
     if (r->result == SG_OK &&
         cudaMemcpyAsync(&s->err_host[slot], r->ws.err, sizeof(int), cudaMemcpyDeviceToHost, st) != cudaSuccess)
@@ -197,7 +235,7 @@ bool start(sg_server *s, sg_request *r)
         r->t_done = now_s();
         r->state.store(RQ_GPU_DONE);
     }
-    s->running.push_back(r);
+    lock.lock();
     return true;
 }
 
@@ -214,7 +252,7 @@ void CUDART_CB on_group_done(void *p)
 }
 
 // Pack the members' pass arguments into the slot's pinned staging, copy them
-// to a pool allocation and enqueue the grouped launches (lock held).
+// to a pool allocation and enqueue the grouped launches.
 template <typename T>
 sg_status group_launch(sg_server *s, sg_group_run *g, cudaStream_t st)
 {
@@ -259,36 +297,28 @@ sg_status group_launch(sg_server *s, sg_group_run *g, cudaStream_t st)
 }
 
 // Start the requests `mem` (same group key; the queue's head first) together on
-// a free slot (lock held). Returns false, holding nothing, when some member's
-// workspace cannot be allocated now.
-bool start_group(sg_server *s, const std::vector<sg_request *> &mem)
+// a free slot (lock as for start). Returns false, holding nothing, when some
+// member's workspace cannot be allocated now.
+bool start_group(sg_server *s, const std::vector<sg_request *> &mem, std::unique_lock<std::mutex> &lock)
 {
     const int slot = s->free_slots.back();
     cudaStream_t st = s->streams[slot];
+    s->free_slots.pop_back();
+    claim(s, mem, slot);
+    lock.unlock();
     for (size_t k = 0; k < mem.size(); ++k) {
         if (!alloc_ws(s, mem[k], st)) {
             for (size_t q = 0; q < k; ++q) sg_workspace_free(&mem[q]->ws, st, true);
+            lock.lock();
+            unclaim(s, mem, slot);
             return false;
         }
     }
-    s->free_slots.pop_back();
     sg_group_run *g = new sg_group_run();
     g->slot = slot;
     g->members = mem;
     g->pending = (int)mem.size();
-    const double t = now_s();
-    for (sg_request *r : mem) {
-        r->slot = slot;
-        r->group = g;
-        s->bytes_in_use += r->bytes;
-        r->t_start = t;
-        r->state.store(RQ_RUNNING);
-        s->running.push_back(r);
-    }
-    s->peak_bytes = std::max(s->peak_bytes, s->bytes_in_use);
-    s->err_host[slot] = 0;
-    s->groups_started++;
-    s->grouped_requests += mem.size();
+    for (sg_request *r : mem) r->group = g;
     sg_status res = mem[0]->plan->prec == SG_FP64 ? group_launch<double>(s, g, st) : group_launch<float>(s, g, st);
     if (res == SG_OK &&
         cudaMemcpyAsync(&s->err_host[slot], mem[0]->ws.err, sizeof(int), cudaMemcpyDeviceToHost, st) != cudaSuccess)
@@ -304,6 +334,9 @@ bool start_group(sg_server *s, const std::vector<sg_request *> &mem)
             r->state.store(RQ_GPU_DONE);
         }
     }
+    lock.lock();
+    s->groups_started++;
+    s->grouped_requests += mem.size();
     return true;
 }
 
@@ -352,12 +385,10 @@ void worker_main(sg_server *s)
             sg_request *r = s->queue.front();
             if (s->bytes_in_use + r->bytes > s->budget) break;
             const std::vector<sg_request *> grp = collect_group(s);
-            if (grp.size() > 1 && start_group(s, grp)) {
-                for (sg_request *q : grp) s->queue.erase(std::find(s->queue.begin(), s->queue.end(), q));
-                continue;
-            }
-            if (!start(s, r)) {
-                if (!s->running.empty()) break;  // memory frees up when a running request ends
+            if (grp.size() > 1 && start_group(s, grp, lock)) continue;
+            if (s->stop || s->queue.empty() || s->queue.front() != r) continue;  // changed while the lock was released
+            if (!start(s, r, lock)) {
+                if (!s->running.empty() || s->queue.empty() || s->queue.front() != r) break;  // memory frees up when a running request ends
                 // nothing running and still no memory: fail this request rather than wait forever
                 s->queue.pop_front();
                 r->result = SG_ENOMEM;
@@ -366,7 +397,6 @@ void worker_main(sg_server *s)
                 s->finished.notify_all();
                 continue;
             }
-            s->queue.pop_front();
         }
         if (s->stop && s->running.empty()) break;
         s->wake.wait_for(lock, std::chrono::milliseconds(1));
