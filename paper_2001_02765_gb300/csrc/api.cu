@@ -840,7 +840,7 @@ sg_status plan_build(const sg_geom *g, sg_precision prec, size_t budget, sg_plan
     {
         const bool central = g->slope_mode == SG_SLOPES_CENTRAL && g->z == 0.0 && !(gi.n > 1 || gi.masked);
         // level convolutions: one launch each for the row, column, column-MAC and inverse-row passes
-        int n = use_lv ? 4 : gi.n * (central ? 4 : 3);
+        int n = use_lv ? 4 : gi.n * (central && !sg_edge_inside(pdev[0].px, pdev[0].py) ? 4 : 3);
         if (plan->composite) {
             n += gi.lmax > 0 ? gi.lmax : 1;  // composite sources: covered cells of levels 1 .. lmax-1, then all S_l
             if (plan->amr_central) n += (gi.lmax > 1 ? gi.lmax - 1 : 0) + gi.lmax + 1;  // fills, then slopes per level

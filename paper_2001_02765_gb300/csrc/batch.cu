@@ -309,9 +309,9 @@ sg_status capture_layout(sg_batch *b, const batch_inputs &in, bool persistent, i
                                                  r64.tries, r64.smem, nsm, bs);
         }, 1);
     for (const sgk::group_passes<float> &g : g32)
-        run_branch([&](cudaStream_t bs) { return sgk::group_enqueue<float>(g, bs); }, g.u.central ? 4 : 3);
+        run_branch([&](cudaStream_t bs) { return sgk::group_enqueue<float>(g, bs); }, g.u.edge == sgk::EDGE_BEFORE ? 4 : 3);
     for (const sgk::group_passes<double> &g : g64)
-        run_branch([&](cudaStream_t bs) { return sgk::group_enqueue<double>(g, bs); }, g.u.central ? 4 : 3);
+        run_branch([&](cudaStream_t bs) { return sgk::group_enqueue<double>(g, bs); }, g.u.edge == sgk::EDGE_BEFORE ? 4 : 3);
     for (int i : rest)
         run_branch([&](cudaStream_t bs) {
             return sg_force_ws(in.plans[i], &b->ws[i], in.sigma[i], in.dx(i), in.dy(i), in.fx[i], in.fy[i], bs);

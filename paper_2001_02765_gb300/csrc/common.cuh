@@ -230,6 +230,10 @@ struct sg_far {
     sg_near_tab tab, ptab;  // force (or off-plane force); potential (built at its first call)
 };
 
+// Whether the row pass of a central-slope solve transforms the edge columns itself
+// (fftconv.cuh): plans count their launches by it.
+static inline __host__ __device__ constexpr bool sg_edge_inside(int px, int py) { return px == py && px <= 512; }
+
 struct sg_patch_plan {
     sg_patch geom;
     sg_patch_dev d;

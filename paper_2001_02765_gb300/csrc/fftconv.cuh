@@ -296,17 +296,6 @@ __device__ __forceinline__ void row_fwd_body(const row_fwd_args<T> &args, int bx
     if constexpr (WAIT_AT_END) sg_dep_wait();
 }
 
-template <typename T, int PX, int NB, int THREADS, bool BATCH = false, bool WAIT_AT_END = false>
-__global__ void __launch_bounds__(THREADS) k_row_fwd(row_fwd_args<T> one, const row_fwd_args<T> *__restrict__ many,
-                                                     const cplx_t<T> *__restrict__ tw)
-{
-    // the first kernel of a solve without an edge pass lets the next one start only
-    // once the stream's previous kernel has finished (see sg_dep_first)
-    if constexpr (WAIT_AT_END) sg_dep_trigger();
-    else sg_dep_first();
-    const row_fwd_args<T> args = pass_args<BATCH>(one, many);
-    row_fwd_body<T, PX, NB, THREADS, WAIT_AT_END>(args, blockIdx.x, blockIdx.y, tw);
-}
 
 // exp(2 pi i u / 8)
 template <typename T>
@@ -683,11 +672,40 @@ __device__ __forceinline__ void edge_body(const edge_args<T> &args, const cplx_t
     }
 }
 
+// What the row pass of a solve does about the edge columns: nothing (no central
+// slopes); run after a separate edge pass, which is launched first and overlaps the
+// end of the previous solve; or transform them itself, in CTA 0 of the grid, one
+// launch fewer: for Px == Py up to 512 points, where launches set the time (100^2
+// 12.4 -> 11.7 us, 250^2 13.2 -> 12.1). Longer columns make that CTA the last one of
+// the pass (500^2 19.3 -> 20.9 us, 1024^2 41.4 -> 44.8 that way).
+enum { EDGE_NONE = 0, EDGE_BEFORE = 1, EDGE_INSIDE = 2 };
+__host__ __device__ constexpr bool edge_inside(int px, int py) { return sg_edge_inside(px, py); }
+
+template <typename T, int PX, int NB, int THREADS, bool BATCH = false, int EDGE = EDGE_NONE>
+__global__ void __launch_bounds__(THREADS) k_row_fwd(row_fwd_args<T> one, const row_fwd_args<T> *__restrict__ many,
+                                                     edge_args<T> ed_one, const edge_args<T> *__restrict__ ed_many,
+                                                     const cplx_t<T> *__restrict__ tw)
+{
+    // the first kernel of a solve lets the next one start only once the stream's
+    // previous kernel has finished (see sg_dep_first)
+    if constexpr (EDGE == EDGE_BEFORE) sg_dep_trigger();
+    else sg_dep_first();
+    if constexpr (EDGE == EDGE_INSIDE) {
+        if (blockIdx.x == 0) {  // first in the grid: it is as long as a row CTA
+            edge_body<T, PX, THREADS>(pass_args<BATCH>(ed_one, ed_many), tw);
+            return;
+        }
+    }
+    const row_fwd_args<T> args = pass_args<BATCH>(one, many);
+    row_fwd_body<T, PX, NB, THREADS, EDGE == EDGE_BEFORE>(args, blockIdx.x - (EDGE == EDGE_INSIDE ? 1 : 0), blockIdx.y,
+                                                          tw);
+}
+
 template <typename T, int PY, int THREADS, bool BATCH = false>
 __global__ void __launch_bounds__(THREADS) k_edge_cols(edge_args<T> one, const edge_args<T> *__restrict__ many,
                                                        const cplx_t<T> *__restrict__ tw)
 {
-    // the first kernel of a central-slope solve: it waits for the previous
+    // the first kernel of a central-slope solve (see EDGE_BEFORE): it waits for the previous
     // kernel of the stream (its scratch is the solve's scratch), then lets the
     // row pass start beside it (k_row_fwd with WAIT_AT_END), whose completion
     // then implies this kernel's for the column pass after them
@@ -966,7 +984,8 @@ struct batch_shape {
 };
 template <typename T>
 sg_status rows_fwd(int px, int nb, const row_fwd_args<T> &one, int nf, const cplx_t<T> *tw, cudaStream_t st,
-                   const row_fwd_args<T> *many = nullptr, batch_shape bs = {0, 0}, bool after_edge = false);
+                   const row_fwd_args<T> *many = nullptr, batch_shape bs = {0, 0}, int edge = EDGE_NONE,
+                   const edge_args<T> *ed = nullptr, const edge_args<T> *ed_many = nullptr);
 // The column and inverse-row passes are launched as dependent launches
 // (sg_launch_dep) on the pass before them in the stream; dep = false launches a
 // column pass normally (when its stream waits on an event just before it).
@@ -997,6 +1016,7 @@ struct uniform_passes {
     int nf_cols;    // fields of the generic column pass
     int nout;       // outputs
     bool central;   // central slopes formed in the spectrum (edge columns, central column pass)
+    int edge;       // how its row pass treats the edge columns (EDGE_*)
     int px, py, qx;
     const cplx_t<T> *twx, *twy;
     int shx[SG_TUNE_KNOBS], shy[SG_TUNE_KNOBS];  // launch shapes of the x and y lengths (tuning table)
@@ -1038,6 +1058,7 @@ inline uniform_passes<T> uniform_setup(const sg_plan *plan, const sg_workspace *
     u.twx = (const C *)((const char *)plan->twiddles + twoff[sg_len_index(d.px)]);
     u.twy = (const C *)((const char *)plan->twiddles + twoff[sg_len_index(d.py)]);
     u.central = src.mode == SG_SLOPES_CENTRAL && pp.phase && !pot_spec;
+    u.edge = !u.central ? EDGE_NONE : (edge_inside(u.px, u.py) ? EDGE_INSIDE : EDGE_BEFORE);
     u.nf_rows = u.central ? 1 : nf;
     u.nf_cols = nf;
     u.nout = pot_spec ? 1 : (fz ? 3 : 2);
