@@ -965,11 +965,12 @@ __host__ __device__ constexpr bool col_feasible_t()
     return CB >= 1 && CB * PY / 8 >= 32 && CB * PY / 8 <= 512 && col_smem_bytes<T, PY, CB, NPL>() <= 200 * 1024;
 }
 
-// Dynamic shared memory beyond the 48 KB every kernel may use without asking.
+// Dynamic shared memory beyond the 48 KB every kernel may use without asking, of
+// which a pass's static arrays take at most 4 KB.
 template <typename K>
 inline sg_status smem_limit(K kern, size_t smem)
 {
-    if (smem > 48 * 1024)
+    if (smem > 44 * 1024)
         SG_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     return SG_OK;
 }
