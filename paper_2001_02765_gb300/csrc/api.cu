@@ -615,7 +615,6 @@ void plan_free(sg_plan *plan)
             cudaFree(plan->pp[k].phase);
             cudaFree(plan->pp[k].pspectra);
         }
-        cudaFree(plan->pot_fwd);
     }
     sg_lv_free(plan);
     cudaFree(plan->twiddles);
@@ -738,7 +737,7 @@ sg_status plan_build(const sg_geom *g, sg_precision prec, size_t budget, sg_plan
         pdev[k] = d;
         const int nplanes = g->z != 0.0 ? 9 : 6;
         if (!use_lv) st = dev_alloc(plan, &pp.spectra, nplanes * (size_t)(d.px / 2 + 1) * sg_spec_stride(d.py) * es);
-        if (st == SG_OK && g->slope_mode == SG_SLOPES_CENTRAL && g->z == 0.0 && !(gi.n > 1 || gi.masked))
+        if (st == SG_OK && g->slope_mode == SG_SLOPES_CENTRAL && !(gi.n > 1 || gi.masked))
             st = dev_alloc(plan, &pp.phase, (4 * (size_t)(d.px / 2 + 1) + 4 * (size_t)d.py) * es);
     }
     if (plan->composite) {
@@ -796,9 +795,9 @@ sg_status plan_build(const sg_geom *g, sg_precision prec, size_t budget, sg_plan
     int64_t wf = 0, wi = 0;
     for (int k = 0; k < gi.n; ++k) {
         const int64_t q = (int64_t)(pdev[k].px / 2 + 1) * pdev[k].ny * (int64_t)(2 * es);
-        // central slopes of a single unmasked patch (in the plane) transform sigma only, plus the
+        // central slopes of a single unmasked patch transform sigma only, plus the
         // two edge columns (2 x py complex); hierarchies transform three composite fields
-        const bool central = g->slope_mode == SG_SLOPES_CENTRAL && g->z == 0.0 && !(gi.n > 1 || gi.masked);
+        const bool central = g->slope_mode == SG_SLOPES_CENTRAL && !(gi.n > 1 || gi.masked);
         const int64_t f = central ? q + (2LL * pdev[k].py + 1) * (int64_t)(2 * es) : 3 * q;  // edge pairs, even start
         const int nout = g->z != 0.0 ? 3 : 2;
         if (f > wf) wf = f;
@@ -838,7 +837,7 @@ sg_status plan_build(const sg_geom *g, sg_precision prec, size_t budget, sg_plan
     if (st == SG_OK && use_lv) st = sg_lv_setup(plan, &lva);  // sets the transform scratch sizes
     plan->scratch_bytes = sg_workspace_bytes(plan);  // the plan's own workspace is allocated at its first sg_force
     {
-        const bool central = g->slope_mode == SG_SLOPES_CENTRAL && g->z == 0.0 && !(gi.n > 1 || gi.masked);
+        const bool central = g->slope_mode == SG_SLOPES_CENTRAL && !(gi.n > 1 || gi.masked);
         // level convolutions: one launch each for the row, column, column-MAC and inverse-row passes
         int n = use_lv ? 4 : gi.n * (central && !sg_edge_inside(pdev[0].px, pdev[0].py) ? 4 : 3);
         if (plan->composite) {
@@ -1134,24 +1133,14 @@ sg_status sg_potential(sg_plan *plan, const void *sigma, const void *deltax, con
         const char *S = (const char *)plan->ws->sfield;
         const size_t plane = (size_t)plan->ncells * es;
         for (int k = 0; k < plan->npatches; ++k)
-            SG_TRY(sg_uniform_potential(plan, plan->ws, k, plan->ws->work_fwd, S, S + plane, S + 2 * plane, phi, st));
+            SG_TRY(sg_uniform_potential(plan, plan->ws, k, S, S + plane, S + 2 * plane, phi, st));
         return sg_cross_potential(plan, plan->ws, S, S + plane, S + 2 * plane, phi, st);
     }
     SG_TRY(sg_potential_spectra_build(plan));
     SG_TRY(ensure_ws(plan));
-    const sg_patch_dev &d = plan->pp[0].d;
-    const int64_t need = 3LL * (d.px / 2 + 1) * d.ny * (int64_t)(2 * es);
-    void *wf = plan->ws->work_fwd;
-    if (plan->ws_fwd_bytes < need) {
-        if (!plan->pot_fwd) {
-            SG_TRY(dev_alloc(plan, &plan->pot_fwd, (size_t)need));
-            plan->pot_fwd_bytes = need;
-        }
-        wf = plan->pot_fwd;
-    }
     sg_timing_reset(plan->timing);
     plan->ws->timing = plan->timing;
-    return sg_uniform_potential(plan, plan->ws, 0, wf, sigma, caller ? deltax : nullptr, caller ? deltay : nullptr, phi,
+    return sg_uniform_potential(plan, plan->ws, 0, sigma, caller ? deltax : nullptr, caller ? deltay : nullptr, phi,
                                 (cudaStream_t)stream);
 }
 

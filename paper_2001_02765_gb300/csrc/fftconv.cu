@@ -8,16 +8,14 @@ namespace {
 
 template <typename T>
 sg_status uniform_solve_t(sg_plan *plan, const sg_workspace *ws, int p, const void *sigma, const void *dx,
-                          const void *dy, void *fx, void *fy, void *fz, cudaStream_t st, const T *pot_spec = nullptr,
-                          void *wf_pot = nullptr)
+                          const void *dy, void *fx, void *fy, void *fz, cudaStream_t st, const T *pot_spec = nullptr)
 {
-    const sgk::uniform_passes<T> u = sgk::uniform_setup<T>(plan, ws, p, sigma, dx, dy, fx, fy, fz, pot_spec, wf_pot);
+    const sgk::uniform_passes<T> u = sgk::uniform_setup<T>(plan, ws, p, sigma, dx, dy, fx, fy, fz, pot_spec);
     // the passes' scratch must hold what they write (checked before any launch)
     const int64_t q = (int64_t)u.qx * plan->pp[p].d.ny * (int64_t)sizeof(cplx_t<T>);
     const int64_t need_f = u.nf_rows * q + (u.central ? (2LL * u.py + 1) * (int64_t)sizeof(cplx_t<T>) : 0);
-    const int64_t have_f = pot_spec && wf_pot != ws->work_fwd ? plan->pot_fwd_bytes : plan->ws_fwd_bytes;
     const int64_t need_i = u.nout * (int64_t)u.qx * sgk::inv_rows(plan->pp[p].d.ny) * (int64_t)sizeof(cplx_t<T>);
-    if (need_f > have_f || need_i > plan->ws_inv_bytes) {
+    if (need_f > plan->ws_fwd_bytes || need_i > plan->ws_inv_bytes) {
         sg_set_last_error_message("internal: a transform pass needs more scratch than the plan sized");
         return SG_EINVAL;
     }
@@ -28,7 +26,7 @@ sg_status uniform_solve_t(sg_plan *plan, const sg_workspace *ws, int p, const vo
     SG_TRY(sgk::rows_fwd<T>(u.px, u.shx[0], u.rf, u.nf_rows, u.twx, st, nullptr, {0, 0}, u.edge, &u.ed));
     sg_timing_end(ws, SG_STAGE_ROW_FWD, st);
     sg_timing_begin(ws, SG_STAGE_COL_CONV, st);
-    if (u.central) SG_TRY(sgk::cols_central<T>(u.py, u.shy[3], u.col, u.qx, u.twy, ws->err, st));
+    if (u.central) SG_TRY(sgk::cols_central<T>(u.py, u.shy[3], u.nout, u.col, u.qx, u.twy, ws->err, st));
     else SG_TRY(sgk::cols<T>(u.py, u.shy[2], u.nout, u.col, u.qx, u.nf_cols, u.twy, ws->err, st));
     sg_timing_end(ws, SG_STAGE_COL_CONV, st);
     sg_timing_begin(ws, SG_STAGE_ROW_INV, st);
@@ -46,13 +44,13 @@ sg_status sg_uniform_solve(sg_plan *plan, const sg_workspace *ws, int patch, con
     return uniform_solve_t<float>(plan, ws, patch, sigma, dx, dy, fx, fy, fz, st);
 }
 
-sg_status sg_uniform_potential(sg_plan *plan, const sg_workspace *ws, int patch, void *wf, const void *sigma,
+sg_status sg_uniform_potential(sg_plan *plan, const sg_workspace *ws, int patch, const void *sigma,
                                const void *dx, const void *dy, void *phi, cudaStream_t st)
 {
     const sg_patch_plan &pp = plan->pp[patch];
     if (plan->prec == SG_FP64)
         return uniform_solve_t<double>(plan, ws, patch, sigma, dx, dy, phi, nullptr, nullptr, st,
-                                       (const double *)pp.pspectra, wf);
+                                       (const double *)pp.pspectra);
     return uniform_solve_t<float>(plan, ws, patch, sigma, dx, dy, phi, nullptr, nullptr, st,
-                                  (const float *)pp.pspectra, wf);
+                                  (const float *)pp.pspectra);
 }

@@ -346,10 +346,10 @@ __host__ __device__ constexpr int col_cb_default(int py)
 // per batch); single solves of the shorter lengths, bound by latency, are 3 % faster
 // at two CTAs without the spills (250^2 14.8 against 15.2 us). The caller-slope pass
 // spills 100 bytes at 64 registers and takes 80 (three CTAs).
-template <typename T, int PY, int CB, bool BATCH>
+template <typename T, int PY, int CB, int NOUT, bool BATCH>
 __host__ __device__ constexpr bool col_central_four()
 {
-    return sizeof(T) == 4 && sg_pow2(PY) && CB == col_cb_default(PY) && (BATCH || PY >= 2048);
+    return sizeof(T) == 4 && NOUT < 3 && sg_pow2(PY) && CB == col_cb_default(PY) && (BATCH || PY >= 2048);
 }
 // 768 and 1536 points likewise take 64 registers (both buffers fit): five CTAs of
 // 192 threads at 1536 points (a 700^2 solve 37.4 -> 35.6 us). At 1280 and 2560 the
@@ -357,8 +357,8 @@ __host__ __device__ constexpr bool col_central_four()
 // registers, 30.9 at 80).
 template <typename T, int PY, int CB>
 __host__ __device__ constexpr bool col_central_lean() { return sizeof(T) == 4 && (PY == 768 || PY == 1536); }
-template <typename T, int PY, int CB, bool BATCH>
-__host__ __device__ constexpr int col_central_nbuf() { return col_central_four<T, PY, CB, BATCH>() ? 1 : col_nbuf<T, PY>(); }
+template <typename T, int PY, int CB, int NOUT, bool BATCH>
+__host__ __device__ constexpr int col_central_nbuf() { return col_central_four<T, PY, CB, NOUT, BATCH>() ? 1 : col_nbuf<T, PY>(); }
 template <typename T, int PY, int CB, int NB = col_nbuf<T, PY>()>
 __host__ __device__ constexpr int col_buf_bytes() { return NB * ((spad_size<cplx_t<T>>(CB * PY) * (int)sizeof(cplx_t<T>) + 15) & ~15); }
 template <typename T, int PY, int CB, int NPL = 6, int NB = col_nbuf<T, PY>()>
@@ -417,10 +417,11 @@ constexpr int col_min_blocks()
     constexpr int d = col_min_blocks_def<T, PY, NOUT>();
     return d * def_threads / THREADS >= 1 ? d * def_threads / THREADS : 1;
 }
-template <typename T, int PY, int CB, int THREADS, bool BATCH>
+template <typename T, int PY, int CB, int THREADS, int NOUT, bool BATCH>
 constexpr int col_central_blocks()
 {
-    if (col_central_four<T, PY, CB, BATCH>()) return 65536 / (64 * THREADS);
+    if (NOUT == 3) return col_min_blocks<T, PY, THREADS, 3>();
+    if (col_central_four<T, PY, CB, NOUT, BATCH>()) return 65536 / (64 * THREADS);
     if (col_central_lean<T, PY, CB>()) return 65536 / (64 * THREADS);
     if (sizeof(T) == 4 && sg_pow2(PY) && PY < 2048) return 512 / THREADS >= 1 ? 512 / THREADS : 1;
     return col_min_blocks<T, PY, THREADS>();
@@ -823,11 +824,17 @@ __device__ __forceinline__ void col_central_body(const col_args<T> &args, int bx
 // inlined body it ran 19% slower (32.8 against 27.6 us at 2048 x 2048, FP32;
 // same registers, more time waiting on global loads). The batch tests check that
 // the persistent kernel (which runs the body) and this kernel agree bit for bit.
-template <typename T, int PY, int CB, int THREADS, bool BATCH = false>
-__global__ void __launch_bounds__(THREADS, (col_central_blocks<T, PY, CB, THREADS, BATCH>())) k_col_conv_central(
+// NOUT = 1 is the potential (3 spectrum planes), NOUT = 3 the off-plane force (9):
+// they too read the transform of sigma alone. With three fields transformed for them,
+// a potential solve of 1024 x 1024 took 55.2 us, of which the forward rows 18.5 and the
+// columns 28; with one, 33.6 (rows 8, columns 16), at the same error (1.7e-7 of 64 bits).
+template <typename T, int PY, int CB, int THREADS, int NOUT = 2, bool BATCH = false>
+__global__ void __launch_bounds__(THREADS, (col_central_blocks<T, PY, CB, THREADS, NOUT, BATCH>())) k_col_conv_central(
     col_args<T> one, const col_args<T> *__restrict__ many, int qx, const cplx_t<T> *__restrict__ tw, int *err)
 {
     using C = cplx_t<T>;
+    constexpr int NBUF = col_central_nbuf<T, PY, CB, NOUT, BATCH>();
+    constexpr int NPL = NOUT == 3 ? 9 : (NOUT == 1 ? 3 : 6);
     sg_dep_trigger();
     const col_args<T> args = pass_args<BATCH>(one, many);
     const cplx_t<T> *__restrict__ work_fwd = args.wf;
@@ -838,7 +845,7 @@ __global__ void __launch_bounds__(THREADS, (col_central_blocks<T, PY, CB, THREAD
     const int ny = args.ny;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     C *bufs = reinterpret_cast<C *>(smem_raw);
-    T *ssp = reinterpret_cast<T *>(smem_raw + col_buf_bytes<T, PY, CB, col_central_nbuf<T, PY, CB, BATCH>()>());
+    T *ssp = reinterpret_cast<T *>(smem_raw + col_buf_bytes<T, PY, CB, NBUF>());
     __shared__ uint64_t bar;
     __shared__ C rows[CB][2];  // R0, R1 of each column
     static_assert(CB * PY / THREADS == 8, "eight elements per thread");
@@ -849,7 +856,7 @@ __global__ void __launch_bounds__(THREADS, (col_central_blocks<T, PY, CB, THREAD
     const int kx = kx0 + c;
     if (threadIdx.x == 0) mbar_init(&bar, 1);
     __syncthreads();
-    if (threadIdx.x == 0) fetch_spectra<T, PY, CB>(ssp, spec, kx0, qx, &bar);
+    if (threadIdx.x == 0) fetch_spectra<T, PY, CB, NPL>(ssp, spec, kx0, qx, &bar);
     sg_dep_wait();  // the row pass's output (the kernel spectra are the plan's own)
     const C *cpair = reinterpret_cast<const C *>(phase), *rpair = cpair + 2 * qx;  // (e1, e2) per kx, per ky
 
@@ -866,7 +873,7 @@ __global__ void __launch_bounds__(THREADS, (col_central_blocks<T, PY, CB, THREAD
     for (int m = 0; m < 4; ++m)
         if (jt + m * STEP == ny - 1) rows[c][1] = v[m];
     int par = 0;
-    fft_regs<C, PY, CB, THREADS, col_central_nbuf<T, PY, CB, BATCH>(), false>(v, bufs, par, tw);
+    fft_regs<C, PY, CB, THREADS, NBUF, false>(v, bufs, par, tw);
     if (!spectra_ready(&bar, err, args.tries)) return;
 
     // the slope factors of the column, and of the bins jt + q PY/8: those of bin jt
@@ -877,11 +884,13 @@ __global__ void __launch_bounds__(THREADS, (col_central_blocks<T, PY, CB, THREAD
     C r0 = rows[c < CB ? c : 0][0], r1 = rows[c < CB ? c : 0][1];
     r0 = cmul_rn(f1, r0);
     r1 = cmul_rn(f2, r1);
-    C accx[8], accy[8];
+    C accx[8], accy[NOUT > 1 ? 8 : 1], accz[NOUT > 2 ? 8 : 1];
 #pragma unroll
     for (int q = 0; q < 8; ++q) {
         const int ky = jt + q * STEP;
-        accx[q] = accy[q] = cmake<C>((T)0, (T)0);
+        accx[q] = cmake<C>((T)0, (T)0);
+        if constexpr (NOUT > 1) accy[q] = accx[q];
+        if constexpr (NOUT > 2) accz[q] = accx[q];
         if (kx >= qx) continue;
         const bool lower = ky <= PY / 2;
         const int kq = lower ? ky : PY - ky;
@@ -897,29 +906,39 @@ __global__ void __launch_bounds__(THREADS, (col_central_blocks<T, PY, CB, THREAD
         const C q2 = cmul_rn(turn8<T>(-ny * q), r1), q1 = rot8(r0, q);
         const C X = cmake<C>(add_rn(add_rn(-mul_rn(cs, S.y), p2.x), -p1.x), add_rn(add_rn(mul_rn(cs, S.x), p2.y), -p1.y));
         const C Y = cmake<C>(add_rn(add_rn(-mul_rn(rs, S.y), q2.x), -q1.x), add_rn(add_rn(mul_rn(rs, S.x), q2.y), -q1.y));
-        const T a = sp[0 * CB * QS];
-        const T b = sp[1 * CB * QS];
-        const T cc = sg * sp[2 * CB * QS];
-        const T d = sg * sp[3 * CB * QS];
-        const T ee = sp[4 * CB * QS];
-        const T ff = sg * sp[5 * CB * QS];
-        accx[q] = cmake<C>(fma(cc, Y.x, fma(b, X.x, -mul_rn(a, S.y))), fma(cc, Y.y, fma(b, X.y, mul_rn(a, S.x))));
-        accy[q] = cmake<C>(fma(ff, X.x, fma(ee, Y.x, -mul_rn(d, S.y))), fma(ff, X.y, fma(ee, Y.y, mul_rn(d, S.x))));
+        if constexpr (NOUT == 1) {
+            // the potential: p S + i (a X + b Y), the planes of k_col_conv
+            const T p = sp[0], a = sp[1 * CB * QS], b = sg * sp[2 * CB * QS];
+            accx[q] = cmake<C>(fma(-b, Y.y, fma(-a, X.y, mul_rn(p, S.x))), fma(b, Y.x, fma(a, X.x, mul_rn(p, S.y))));
+        } else {
+            const T a = sp[0 * CB * QS];
+            const T b = sp[1 * CB * QS];
+            const T cc = sg * sp[2 * CB * QS];
+            const T d = sg * sp[3 * CB * QS];
+            const T ee = sp[4 * CB * QS];
+            const T ff = sg * sp[5 * CB * QS];
+            accx[q] = cmake<C>(fma(cc, Y.x, fma(b, X.x, -mul_rn(a, S.y))), fma(cc, Y.y, fma(b, X.y, mul_rn(a, S.x))));
+            accy[q] = cmake<C>(fma(ff, X.x, fma(ee, Y.x, -mul_rn(d, S.y))), fma(ff, X.y, fma(ee, Y.y, mul_rn(d, S.x))));
+            if constexpr (NOUT == 3) {
+                // Fz: g S + i (hh X + kk Y)
+                const T g = sp[6 * CB * QS], hh = sp[7 * CB * QS], kk = sg * sp[8 * CB * QS];
+                accz[q] = cmake<C>(fma(-kk, Y.y, fma(-hh, X.y, mul_rn(g, S.x))), fma(kk, Y.x, fma(hh, X.x, mul_rn(g, S.y))));
+            }
+        }
     }
 
     // inverse transforms: the products are already in the transform's input pattern
-    if (col_central_nbuf<T, PY, CB, BATCH>() == 1) __syncthreads();
-    fft_regs<C, PY, CB, THREADS, col_central_nbuf<T, PY, CB, BATCH>(), true>(accx, bufs, par, tw);
-    int at = inv_index(0, kx, jt, qx, ny);  // STEP is a whole number of row blocks
+    auto finish = [&](C(&acc)[8], int o) {
+        if (NBUF == 1) __syncthreads();
+        fft_regs<C, PY, CB, THREADS, NBUF, true>(acc, bufs, par, tw);
+        const int at = inv_index(o, kx, jt, qx, ny);  // STEP is a whole number of row blocks
 #pragma unroll
-    for (int m = 0; m < 4; ++m)
-        if (jt + m * STEP < ny && kx < qx) work_inv[at + m * (STEP * qx)] = accx[m];
-    if (col_central_nbuf<T, PY, CB, BATCH>() == 1) __syncthreads();
-    fft_regs<C, PY, CB, THREADS, col_central_nbuf<T, PY, CB, BATCH>(), true>(accy, bufs, par, tw);
-    at = inv_index(1, kx, jt, qx, ny);
-#pragma unroll
-    for (int m = 0; m < 4; ++m)
-        if (jt + m * STEP < ny && kx < qx) work_inv[at + m * (STEP * qx)] = accy[m];
+        for (int m = 0; m < 4; ++m)
+            if (jt + m * STEP < ny && kx < qx) work_inv[at + m * (STEP * qx)] = acc[m];
+    };
+    finish(accx, 0);
+    if constexpr (NOUT > 1) finish(accy, 1);
+    if constexpr (NOUT > 2) finish(accz, 2);
 }
 
 // ------------------------------------------------------------ launch shapes --
@@ -997,7 +1016,7 @@ template <typename T>
 sg_status cols(int py, int cb, int nout, const col_args<T> &one, int qx, int nf, const cplx_t<T> *tw, int *err,
                cudaStream_t st, const col_args<T> *many = nullptr, batch_shape bs = {0, 0}, bool dep = true);
 template <typename T>
-sg_status cols_central(int py, int cb, const col_args<T> &one, int qx, const cplx_t<T> *tw, int *err, cudaStream_t st,
+sg_status cols_central(int py, int cb, int nout, const col_args<T> &one, int qx, const cplx_t<T> *tw, int *err, cudaStream_t st,
                        const col_args<T> *many = nullptr, batch_shape bs = {0, 0}, bool dep = true);
 template <typename T>
 sg_status edge_cols(int py, const edge_args<T> &one, const cplx_t<T> *tw, cudaStream_t st,
@@ -1005,8 +1024,7 @@ sg_status edge_cols(int py, const edge_args<T> &one, const cplx_t<T> *tw, cudaSt
 
 // The arguments of every pass of one patch's solve (fftconv.cu), shared by the
 // single solve and by batches (batch.cu). pot_spec != NULL: the potential (one
-// output, three spectrum planes) with the forward scratch wf_pot, slopes formed
-// in the row pass.
+// output, three spectrum planes).
 template <typename T>
 struct uniform_passes {
     row_fwd_args<T> rf;
@@ -1026,7 +1044,7 @@ struct uniform_passes {
 template <typename T>
 inline uniform_passes<T> uniform_setup(const sg_plan *plan, const sg_workspace *ws, int p, const void *sigma,
                                        const void *dx, const void *dy, void *fx, void *fy, void *fz,
-                                       const T *pot_spec = nullptr, void *wf_pot = nullptr)
+                                       const T *pot_spec = nullptr)
 {
     using C = cplx_t<T>;
     uniform_passes<T> u;
@@ -1053,12 +1071,12 @@ inline uniform_passes<T> uniform_setup(const sg_plan *plan, const sg_workspace *
     u.px = d.px;
     u.py = d.py;
     u.qx = d.px / 2 + 1;
-    C *wf = pot_spec ? (C *)wf_pot : (C *)ws->work_fwd;
+    C *wf = (C *)ws->work_fwd;
     C *wi = (C *)ws->work_inv;
     const int64_t *twoff = sizeof(T) == 8 ? plan->tw64_off : plan->tw32_off;
     u.twx = (const C *)((const char *)plan->twiddles + twoff[sg_len_index(d.px)]);
     u.twy = (const C *)((const char *)plan->twiddles + twoff[sg_len_index(d.py)]);
-    u.central = src.mode == SG_SLOPES_CENTRAL && pp.phase && !pot_spec;
+    u.central = src.mode == SG_SLOPES_CENTRAL && pp.phase;
     u.edge = !u.central ? EDGE_NONE : (edge_inside(u.px, u.py) ? EDGE_INSIDE : EDGE_BEFORE);
     u.nf_rows = u.central ? 1 : nf;
     u.nf_cols = nf;

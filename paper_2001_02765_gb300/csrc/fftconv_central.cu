@@ -6,13 +6,13 @@
 namespace sgk {
 namespace {
 
-template <typename T, int PY, int CB, bool BATCH>
+template <typename T, int PY, int CB, int NOUT, bool BATCH>
 sg_status launch_cols_central(const col_args<T> &one, const col_args<T> *many, batch_shape bs, int qx,
                               const cplx_t<T> *tw, int *err, cudaStream_t st, bool dep)
 {
-    constexpr int THREADS = CB * PY / 8;
-    const size_t smem = (size_t)col_smem_bytes<T, PY, CB, 6, col_central_nbuf<T, PY, CB, BATCH>()>();
-    auto kern = k_col_conv_central<T, PY, CB, THREADS, BATCH>;
+    constexpr int THREADS = CB * PY / 8, NPL = NOUT == 3 ? 9 : (NOUT == 1 ? 3 : 6);
+    const size_t smem = (size_t)col_smem_bytes<T, PY, CB, NPL, col_central_nbuf<T, PY, CB, NOUT, BATCH>()>();
+    auto kern = k_col_conv_central<T, PY, CB, THREADS, NOUT, BATCH>;
     SG_TRY(smem_limit(kern, smem));
     dim3 grid((qx + CB - 1) / CB, 1, BATCH ? bs.nmem : 1);
     if (dep) SG_CUDA_TRY(sg_launch_dep(kern, grid, dim3(THREADS), smem, st, one, many, qx, tw, err));
@@ -25,16 +25,22 @@ template <typename T, int PY, int CB>
 sg_status launch_cols_central_any(const col_args<T> &one, const col_args<T> *many, batch_shape bs, int qx,
                                   const cplx_t<T> *tw, int *err, cudaStream_t st, bool dep)
 {
-    if (many) return launch_cols_central<T, PY, CB, true>(one, many, bs, qx, tw, err, st, dep);
-    return launch_cols_central<T, PY, CB, false>(one, many, bs, qx, tw, err, st, dep);
+    if (many) return launch_cols_central<T, PY, CB, 2, true>(one, many, bs, qx, tw, err, st, dep);
+    return launch_cols_central<T, PY, CB, 2, false>(one, many, bs, qx, tw, err, st, dep);
 }
 
+// the potential and off-plane passes (one and three outputs) have the default shape only
 template <typename T, int PY>
-sg_status cols_central_py(int cb, const col_args<T> &one, const col_args<T> *many, batch_shape bs, int qx,
+sg_status cols_central_py(int cb, int nout, const col_args<T> &one, const col_args<T> *many, batch_shape bs, int qx,
                           const cplx_t<T> *tw, int *err, cudaStream_t st, bool dep)
 {
     constexpr int D = col_cb_default(PY);
     constexpr int A = shape_candidate(D, 0), C = shape_candidate(D, 2);
+    if (nout != 2) {
+        if (many) return SG_EINVAL;
+        if (nout == 1) return launch_cols_central<T, PY, D, 1, false>(one, many, bs, qx, tw, err, st, dep);
+        return launch_cols_central<T, PY, D, 3, false>(one, many, bs, qx, tw, err, st, dep);
+    }
     if (cb == D) return launch_cols_central_any<T, PY, D>(one, many, bs, qx, tw, err, st, dep);
     if constexpr (sg_pow2(PY) && col_feasible_t<T, PY, A, 6>()) {
         if (cb == A) return launch_cols_central_any<T, PY, A>(one, many, bs, qx, tw, err, st, dep);
@@ -68,10 +74,10 @@ sg_status launch_edge_cols(const edge_args<T> &one, const edge_args<T> *many, ba
 }  // namespace
 
 template <typename T>
-sg_status cols_central(int py, int cb, const col_args<T> &one, int qx, const cplx_t<T> *tw, int *err, cudaStream_t st,
+sg_status cols_central(int py, int cb, int nout, const col_args<T> &one, int qx, const cplx_t<T> *tw, int *err, cudaStream_t st,
                        const col_args<T> *many, batch_shape bs, bool dep)
 {
-    SG_PAD_SWITCH(py, return (cols_central_py<T, PP>(cb, one, many, bs, qx, tw, err, st, dep)));
+    SG_PAD_SWITCH(py, return (cols_central_py<T, PP>(cb, nout, one, many, bs, qx, tw, err, st, dep)));
     return SG_EINVAL;
 }
 
@@ -83,9 +89,9 @@ sg_status edge_cols(int py, const edge_args<T> &one, const cplx_t<T> *tw, cudaSt
     return SG_EINVAL;
 }
 
-template sg_status cols_central<float>(int, int, const col_args<float> &, int, const float2 *, int *, cudaStream_t,
+template sg_status cols_central<float>(int, int, int, const col_args<float> &, int, const float2 *, int *, cudaStream_t,
                                        const col_args<float> *, batch_shape, bool);
-template sg_status cols_central<double>(int, int, const col_args<double> &, int, const double2 *, int *, cudaStream_t,
+template sg_status cols_central<double>(int, int, int, const col_args<double> &, int, const double2 *, int *, cudaStream_t,
                                         const col_args<double> *, batch_shape, bool);
 template sg_status edge_cols<float>(int, const edge_args<float> &, const float2 *, cudaStream_t,
                                     const edge_args<float> *, batch_shape);
