@@ -547,7 +547,7 @@ sizes plan_sizes(const sg_geom *g, const geom_info &gi, sg_precision prec, int n
     if (gi.n > 1 && lv_bytes < 0) {
         s.direct += gi.nleaves * (int64_t)sizeof(int4) + (int64_t)nblocks * (int64_t)sizeof(sg_target_block);
         if (prec == SG_FP32) {
-            // clusters of 8 x 8 cells and their parents (up to 4/3 of them), the near field
+            // clusters of SG_CL_CELLS^2 cells and their parents (up to 4/3 of them), the near field
             int64_t ncl = 0;
             for (int k = 0; k < gi.n; ++k)
                 for (int w = SG_CL_CELLS;; w *= 2) {

@@ -132,8 +132,8 @@ struct __align__(32) sg_dvec4 {
 // (near field); other cells by the expansion of their integrals about their
 // centre, or in clusters of SG_CL_CELLS 2^k cells per side.
 #define SG_NEAR_R 6
-#define SG_CL_CELLS 8
-#define SG_CL_LEVELS 9          // clusters of a patch: 2048 / 8 = 2^8 per side, nine levels
+#define SG_CL_CELLS 4
+#define SG_CL_LEVELS 10         // clusters of a patch: 2048 / 4 = 2^9 per side, ten levels
 // Near tables: targets up to 2^SG_NT_GMAX times narrower than the source cells
 // (4^g positions of 6.9 KB each: 7 MB at 5), keyed by log2 of the source cell
 // width in lattice units (below SG_NT_STEPS) and the width ratio's exponent (-1 .. SG_NT_GMAX).

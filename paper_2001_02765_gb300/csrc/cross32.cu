@@ -18,7 +18,7 @@
 //    five times cheaper than a DFMA and rounds at 2^-45. Pairs of levels more
 //    than SG_NT_GMAX apart (4^g positions) or with too few targets to repay a
 //    table keep the corner form in FP64 (k_near_corner).
-//  * Middle cells (up to two clusters of 8 cells away): the expansion of each
+//  * Middle cells (up to two clusters of 4 cells away): the expansion of each
 //    cell's integrals about its centre through H^6 (force, potential) or 3 x 3
 //    Gauss-Legendre nodes (off the plane), in FP32. Per unit G, with a, b =
 //    (centre - target)/H, rho^2 = a^2 + b^2, w = 1/(a + i b), s = 1/rho^2, m =
@@ -32,7 +32,7 @@
 //      Phi = -G H (m I0 + deltax H Ix + deltay H Iy), p = 1/rho:
 //      I0 = p + p^3/24 + p^5 (-7/1920 + (7/96) a^2 b^2 p^4)
 //      Ix = -a p^3/12 + (7/240) a p^5 - a p^7 (a^2/32 + 5 b^2/96)   (Iy: a <-> b)
-//  * Far cells, in clusters. A cluster is a square of 8 2^k cells of a patch; its
+//  * Far cells, in clusters. A cluster is a square of 4 2^k cells of a patch; its
 //    density is carried by 8 x 8 charges on the Chebyshev points of the square,
 //      q_nm = (1/a^2) integral of L_n(x) L_m(y) sigma,  a = half its width,
 //    L the Lagrange polynomials: interpolation of the kernel in the source
@@ -46,16 +46,20 @@
 //    Each block of up to 256 targets (16 x 16 cells) takes, per source patch, at
 //    every level the clusters that are far enough whose parents are not: an index
 //    rectangle minus an index rectangle, so no interaction lists are kept. Where
-//    the cluster is at least as wide as the block, the field is itself smooth
+//    the cluster lies two block widths from the block's centre, its field is smooth
 //    over the block: it is evaluated on 8 x 8 Chebyshev points of the block and
 //    interpolated to the targets once at the end (same bound by symmetry), which
 //    is a quarter of the evaluations; four groups of 64 threads share the
-//    clusters. Smaller clusters act on the targets directly.
+//    clusters. The clusters between act on the targets directly.
+//    Clusters start at 4 cells (four charges a cell): a charge takes 8 cycles of the
+//    special-function unit, a middle cell 62 operations, so that between 8 and 16
+//    cells from a block a cluster costs half of its cells. From 8 cells on, six nested
+//    256^2 levels took 3.74 ms and three off the plane 1.64; from 4 on, 3.23 and 1.32.
 //
 // The direct sum over all pairs that this replaces cost 17.3 ms (far) + 8.9 ms
 // (near, FP64 pipe) on three nested 256^2 levels. Measured per solve: six nested
-// 256^2 levels 121.5 -> 3.74 ms, three off the plane 50.4 -> 1.64 ms; error against
-// FP64 3.5e-7 -> 1.6e-7 and 1.3e-7 -> 7e-8.
+// 256^2 levels 121.5 -> 3.23 ms, three off the plane 50.4 -> 1.32 ms; error against
+// FP64 4.4e-7 -> 1.4e-7 and 1.5e-7 -> 8e-8.
 #include "common.cuh"
 #include "kmath.cuh"
 
@@ -77,7 +81,7 @@ template <int Q> constexpr int q_planes() { return Q == Q_POT ? 3 : (Q == Q_OFF 
 constexpr int CL = SG_CL_CELLS;        // cells per side of a level-0 cluster
 constexpr int NP = 8;                  // Chebyshev points per axis
 constexpr int NQ = NP * NP;            // charges of a cluster
-static_assert(CL == 8 && NQ == 64, "thread maps below");
+static_assert(CL * CL <= NQ && NP * CL <= NQ && NQ == 64, "thread maps below");
 
 // Chebyshev points cos((2 n + 1) pi / 16)
 __device__ __forceinline__ constexpr float cheb(int n)
@@ -121,7 +125,7 @@ __device__ __forceinline__ int floor_div(int64_t a, int64_t b)
 // the distance from the cell's centre,
 //   q_nm = sum_j [ sum_i (sigma A_n[i] + deltax a B_n[i]) ] A_m[j] + [ sum_i deltay a A_n[i] ] B_m[j].
 // 64 threads per cluster (four clusters per CTA), one charge each; bound by
-// latency (16 k FMAs and 768 bytes per cluster).
+// latency (3.5 k FMAs and 192 bytes per cluster).
 __global__ void __launch_bounds__(256) k_p2m(const int4 *__restrict__ desc, int ncl, const sg_patch_dev *__restrict__ pd,
                                              const float *__restrict__ sigma, const float *__restrict__ dx,
                                              const float *__restrict__ dy, double lambda,
@@ -138,22 +142,24 @@ __global__ void __launch_bounds__(256) k_p2m(const int4 *__restrict__ desc, int 
     if (live) {
         const int4 d = desc[c];
         const sg_patch_dev &p = pd[d.x];
-        const int i = d.y * CL + (t & 7), j = d.z * CL + (t >> 3);
+        const int i = d.y * CL + t % CL, j = d.z * CL + t / CL;
         float s = 0.f, x = 0.f, y = 0.f;
-        if (i < p.nx && j < p.ny) {
+        if (t < CL * CL && i < p.nx && j < p.ny) {
             const int64_t o = p.cell_off + (int64_t)j * p.nx + i;
             const double a = (double)(CL / 2) * p.step * lambda;  // half the cluster's width
             s = sigma[o];
             x = (float)((double)dx[o] * a);
             y = (float)((double)dy[o] * a);
         }
-        f[g][0][t] = s;
-        f[g][1][t] = x;
-        f[g][2][t] = y;
+        if (t < CL * CL) {
+            f[g][0][t] = s;
+            f[g][1][t] = x;
+            f[g][2][t] = y;
+        }
     }
     __syncthreads();
-    if (live) {  // t = n * 8 + j
-        const int n = t >> 3, j = t & 7;
+    if (live && t < NP * CL) {  // t = n CL + j
+        const int n = t / CL, j = t % CL;
         float t1 = 0.f, t2 = 0.f;
 #pragma unroll
         for (int i = 0; i < CL; ++i) {
@@ -404,10 +410,9 @@ struct far_args {
 // to the targets' own-patch results. CTAs take blocks from the last to the
 // first (the finest patches, with the most coarser cells near them, first).
 // Bound by FP32 issue (middle cells: 62 operations each) and the special-function
-// unit (far field). Six nested 256^2 levels: 1.9e9 block-point evaluations, 0.2e9
-// at targets and 1.0e9 middle pairs, of which half on the block's points (a quarter
-// of the work): 2.7 ms, 3.8 with every middle cell on the targets; three levels off
-// the plane 1.25 against 1.49 ms.
+// unit (clusters). Middle cells smooth over the block go on its points as well: 2.7 ms
+// for six nested 256^2 levels against 3.8 with every middle cell on the targets, 1.25
+// against 1.49 for three off the plane (with clusters of 8 cells; 4 save 0.5 and 0.3).
 template <int Q>
 __global__ void __launch_bounds__(256, 3) k_far(far_args A)
 {
@@ -452,27 +457,47 @@ __global__ void __launch_bounds__(256, 3) k_far(far_args A)
                 const int nj0 = max(ra, floor_div(-b2 - 5 * (int64_t)W - oy2, 2 * (int64_t)W) + 1);
                 const int nj1 = min(rb, -floor_div(-(b2 + 3 * (int64_t)W - oy2), 2 * (int64_t)W) - 1);
                 const bool some = ni0 <= ni1 && nj0 <= nj1;
-                const bool wide = W >= b2;  // the field is smooth over the block
+                // clusters nearer than 2 b2 + W/2, whose field is not smooth over the block
+                const int M2 = max(4 * b2 + W, b2 + 4 * W);
+                const int mi0 = max(ca, floor_div(-(int64_t)M2 - ox2 - W, 2 * (int64_t)W) + 1);
+                const int mi1 = min(cb, -floor_div(-((int64_t)M2 - ox2 - W), 2 * (int64_t)W) - 1);
+                const int mj0 = max(ra, floor_div(-(int64_t)M2 - oy2 - W, 2 * (int64_t)W) + 1);
+                const int mj1 = min(rb, -floor_div(-((int64_t)M2 - oy2 - W), 2 * (int64_t)W) - 1);
+                const bool mid = mi0 <= mi1 && mj0 <= mj1;
                 const float inv = 2.f / (float)W;
-                const float ux = (wide ? px : tx) * inv, uy = (wide ? py : ty) * inv;
                 const float zeta = Q == Q_OFF ? (float)(2.0 * A.zl / (double)W) : 0.f;
-                const int w = cb - ca + 1, total = w * (rb - ra + 1);
                 const int *sl = A.slot + cp.off[k];
-                for (int e = wide ? grp : 0; e < total; e += wide ? 4 : 1) {
-                    const int j = e / w, i = ca + e - j * w, jj = ra + j;
-                    if (some && i >= ni0 && i <= ni1 && jj >= nj0 && jj <= nj1) continue;
-                    const int s = __ldg(&sl[jj * nx + i]);
-                    if (s < 0) continue;
-                    const float X0 = (float)(ox2 + (2 * i + 1) * W) / (float)W - ux;
-                    const float Y0 = (float)(oy2 + (2 * jj + 1) * W) / (float)W - uy;
-                    float v[NO];
-                    cluster_field<Q>(reinterpret_cast<const float4 *>(A.charges + (int64_t)s * NQ), X0, Y0, zeta * zeta, v);
-                    if constexpr (Q == Q_POT) v[0] *= 0.5f * (float)W;  // q / R in lattice units
-                    if constexpr (Q == Q_OFF) v[2] *= -zeta;
+                // two passes: the others on the block's points, a quarter per group; those on the targets
+                for (int pass = 0; pass < 2; ++pass) {
+                    const bool outer = pass == 0;
+                    if (!outer && (W >= b2 || !mid || (tid & ~31) >= blk.count)) continue;
+                    const int x0 = outer ? ca : mi0, x1 = outer ? cb : mi1, y1 = outer ? rb : mj1;
+                    const bool hole = outer ? mid : some;
+                    const int hx0 = outer ? mi0 : ni0, hx1 = outer ? mi1 : ni1;
+                    const int hy0 = outer ? mj0 : nj0, hy1 = outer ? mj1 : nj1;
+                    const int w = x1 - x0 + 1, de = outer ? 4 : 1;
+                    const float ux = (outer ? px : tx) * inv, uy = (outer ? py : ty) * inv;
+                    int i = x0 + (outer ? grp : 0), jj = outer ? ra : mj0;
+                    for (;; i += de) {
+                        while (i > x1) {
+                            i -= w;
+                            ++jj;
+                        }
+                        if (jj > y1) break;
+                        if (hole && i >= hx0 && i <= hx1 && jj >= hy0 && jj <= hy1) continue;
+                        const int s = __ldg(&sl[jj * nx + i]);
+                        if (s < 0) continue;
+                        const float X0 = (float)(ox2 + (2 * i + 1) * W) / (float)W - ux;
+                        const float Y0 = (float)(oy2 + (2 * jj + 1) * W) / (float)W - uy;
+                        float v[NO];
+                        cluster_field<Q>(reinterpret_cast<const float4 *>(A.charges + (int64_t)s * NQ), X0, Y0, zeta * zeta, v);
+                        if constexpr (Q == Q_POT) v[0] *= 0.5f * (float)W;  // q / R in lattice units
+                        if constexpr (Q == Q_OFF) v[2] *= -zeta;
 #pragma unroll
-                    for (int o = 0; o < NO; ++o) {
-                        if (wide) add2(nh[o], nl[o], v[o]);
-                        else add2(th[o], tl[o], v[o]);
+                        for (int o = 0; o < NO; ++o) {
+                            if (outer) add2(nh[o], nl[o], v[o]);
+                            else add2(th[o], tl[o], v[o]);
+                        }
                     }
                 }
                 pi0 = ni0;
@@ -1109,7 +1134,7 @@ sg_status sg_far_setup(sg_plan *plan, const int *const *codes, int nlevels, cons
     // interpolation matrices: A_n[i], B_n[i] (8-point Gauss-Legendre, exact for these degrees), C_h[n'][n]
     static const double gx[4] = {0.1834346424956498, 0.5255324099163290, 0.7966664774136267, 0.9602898564975363};
     static const double gw[4] = {0.3626837833783620, 0.3137066458778873, 0.2223810344533745, 0.1012285362903763};
-    std::vector<float> mat(4 * NQ);
+    std::vector<float> mat(2 * NP * CL + 2 * NQ);
     for (int n = 0; n < NP; ++n)
         for (int i = 0; i < CL; ++i) {
             const double c = -1.0 + (i + 0.5) * (2.0 / CL), hw = 1.0 / CL;  // cell centre, half width
@@ -1120,12 +1145,12 @@ sg_status sg_far_setup(sg_plan *plan, const int *const *codes, int nlevels, cons
                 b += w * s * lagrange(n, c + s);
             }
             mat[n * CL + i] = (float)a;
-            mat[NQ + n * CL + i] = (float)b;
+            mat[NP * CL + n * CL + i] = (float)b;
         }
     for (int h = 0; h < 2; ++h)
         for (int u = 0; u < NP; ++u)
             for (int n = 0; n < NP; ++n)
-                mat[2 * NQ + h * NQ + u * NP + n] = (float)lagrange(n, 0.5 * (cos((2 * u + 1) * M_PI / 16) + (h ? 1.0 : -1.0)));
+                mat[2 * NP * CL + h * NQ + u * NP + n] = (float)lagrange(n, 0.5 * (cos((2 * u + 1) * M_PI / 16) + (h ? 1.0 : -1.0)));
     F->nclass = near_keys(nlevels, level_targets, gmax, F->keys_host, F->untabled);
     SG_TRY(sg_plan_upload(plan, (void **)&F->patch, cp.data(), cp.size() * sizeof(sg_cl_patch)));
     SG_TRY(sg_plan_upload(plan, (void **)&F->slot, slot.data(), slot.size() * sizeof(int)));

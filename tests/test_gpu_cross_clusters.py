@@ -1,6 +1,6 @@
 """The FP32 cross-patch sum (clusters, middle cells, near tables or the corner
 form) against the oracle's plain leaf sum, on shapes where its index rules can go
-wrong: patches ending inside a cluster of 8 cells, several patches per level, the
+wrong: patches ending inside a cluster, several patches per level, the
 smallest patches, width ratios beyond the near tables, budgets that leave them out.
 
 Tolerance 2e-6 (relative L2 over the leaves): the stated truncations of the middle
