@@ -868,7 +868,7 @@ def run_gpu(args):
     if (not args.no_autotune and wl["patches"] and plan.info["max_pad"] <= 4096
             and plan.info["cross_mode"] != 2):
         t0 = time.perf_counter()
-        pads = sorted({_pad(p[1]) for p in wl["patches"]} | {_pad(p[2]) for p in wl["patches"]})
+        pads = sorted({sg_pad(p[1]) for p in wl["patches"]} | {sg_pad(p[2]) for p in wl["patches"]})
         res = sg.sg_autotune(sg.SG_FP32, pads[0], pads[-1], reps=15)
         tuned = {"seconds": time.perf_counter() - t0, "shapes": {str(p): res[p][0] for p in pads}}
     # the cross-patch direct sum's split and far-field grid (skipped where one
@@ -1199,10 +1199,10 @@ TRAFFIC = {("spiral1024", "col_conv"): 33.810e6 + 0.014e6,
 
 
 def _pad(n):
-    p = 64
-    while p < 2 * n - 1:
-        p *= 2
-    return p
+    """Padded length of a uniform patch's axis: the least 2^k from 64, 5/4 2^k and
+    3/2 2^k from 256, at or above 2 n - 1."""
+    p = sg_pad(n)
+    return next((q for q in (p // 8 * 5, p // 4 * 3) if p >= 512 and q >= 2 * n - 1), p)
 
 
 def _lv_cexp(s, p):
@@ -1239,15 +1239,15 @@ def lv_geometry(wl):
             imgs.append((gx1 - gx0, gy1 - gy0, lmax - m))
         wx = max(round((p[3] - X0) / h0) + p[1] for p in pats if p[0] == 0) << lmax
         wy = max(round((p[4] - Y0) / h0) + p[2] for p in pats if p[0] == 0) << lmax
-    return _pad(wx), _pad(wy), imgs
+    return sg_pad(wx), sg_pad(wy), imgs
 
 
 def algorithmic_flops(wl, info, stage, nout=2):
     """Conventional flop counts: 5 L log2 L per complex FFT of length L, plus
     the spectral multiply-adds (8 flops per field per bin; about 60 per bin for
     the central-slope spectrum; 10 per field and target for level convolutions);
-    the direct sum counts 28 FP32 operations per target-corner pair (FMA = 2).
-    nout = 1: the potential (one output; slopes formed in the row pass)."""
+    the cross-patch sum by its own rule.
+    nout = 1: the potential (one output)."""
     import math
     total = 0.0
     if info.get("cross_mode") == 2:
@@ -1274,7 +1274,7 @@ def algorithmic_flops(wl, info, stage, nout=2):
         qx = px // 2 + 1
         fft_x = 5.0 * px * math.log2(px)
         fft_y = 5.0 * py * math.log2(py)
-        central = wl["slope_mode"] == 1 and nout == 2
+        central = wl["slope_mode"] == 1 and not info.get("cross_mode")
         nfwd = 1 if wl["slope_mode"] == 0 or central else 3
         if stage == "row_fwd":
             total += nfwd * (ny / 2) * fft_x + (fft_y if central else 0)
@@ -1283,15 +1283,13 @@ def algorithmic_flops(wl, info, stage, nout=2):
         elif stage == "row_inv":
             total += nout * (ny / 2) * fft_x  # two rows per transform
     if stage == "cross_direct":
-        # FP32 plans: 30 flops per target-cell pair for the force (the far-field
-        # expansion through H^4, FMA = 2), 16 for the potential (its moments
-        # through p^3); FP64 plans: 28 per target-corner pair
-        fp32 = wl.get("precision", "fp32") == "fp32"
-        total = (30.0 if nout == 2 else 16.0) if fp32 else 28.0
-        if wl.get("z"):
-            # off the plane: FP32 plans 2 x 2 Gauss nodes per far pair at 16 flops each
-            # (3 x 3 within SG_FAR_R4 cells); FP64 plans the corner form, 36 per target-corner pair
-            total = 64.0 if fp32 else 36.0
+        # FP64 plans: 28 operations per target-corner pair (36 off the plane). FP32 plans sum
+        # clusters, whose evaluations depend on the geometry; counted are the near field's
+        # products alone, 144 cells x 3 fields x outputs in two-part arithmetic (10 operations)
+        # per target: a lower count
+        if wl.get("precision", "fp32") == "fp32":
+            return wl["targets"] * 144 * 3 * (3 if wl.get("z") else nout) * 10.0
+        total = 36.0 if wl.get("z") else 28.0
         total *= info["cross_pairs"]
     return total
 
@@ -1326,9 +1324,8 @@ def algorithmic_bytes(wl, info, stage, nout=2):
             keys = {(sm, (sm >= 1) - (sl >= 1)) for _, _, sm in imgs for _, _, sl in imgs}
             total += len(keys) * 3 * nout * qx * qy * es
         return total
-    # central slopes are formed from sigma's transforms: one field is transformed
-    # (the potential forms them in the row pass: three fields)
-    nf = 1 if wl["slope_mode"] == 0 or (wl["slope_mode"] == 1 and nout == 2) else 3
+    # central slopes of a single patch are formed from sigma's transforms: one field is transformed
+    nf = 1 if wl["slope_mode"] == 0 or (wl["slope_mode"] == 1 and not info.get("cross_mode")) else 3
     for p in wl["patches"]:
         nx, ny = p[1], p[2]
         px, py = _pad(nx), _pad(ny)
