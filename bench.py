@@ -1192,10 +1192,10 @@ def oracle_fft_route(wl, reps=3):
 # DRAM bytes (read + write) per launch of a stage's kernel from the ncu capture
 # of the current kernel build (see profiles/); None when not captured for it.
 # amr3 col_conv: the stage's column-transform and column-MAC launches, one each
-# per solve (profiles/k_lv_col_fwd_amr3.md, k_lv_col_mac_inv_amr3.md).
+# per solve (profiles/amr3_levels_launches.md).
 TRAFFIC = {("spiral1024", "col_conv"): 33.810e6 + 0.014e6,
-           ("amr3", "col_conv"): (11.152e6 + 7.286e6) + (226.808e6 + 11.011e6),
-           ("amr3", "cross_direct"): 5.882e6 + 3.741e6}
+           ("amr3", "col_conv"): (11.131e6 + 3.899e6) + (226.635e6 + 6.682e6),
+           ("amr3", "cross_direct"): 3.907e6 + 11.629e6}
 
 
 def _pad(n):

@@ -844,8 +844,8 @@ sg_status plan_build(const sg_geom *g, sg_precision prec, size_t budget, sg_plan
             n += gi.lmax > 0 ? gi.lmax : 1;  // composite sources: covered cells of levels 1 .. lmax-1, then all S_l
             if (plan->amr_central) n += (gi.lmax > 1 ? gi.lmax - 1 : 0) + gi.lmax + 1;  // fills, then slopes per level
             // direct sum: corner weights, pair sum (+ split reduction) in FP64; the charges of
-            // every cluster level, near field (tables, and the corner form where there is none)
-            // and far field in FP32
+            // every cluster level, near and far field (and the corner form where there is no
+            // table) and their addition to the own-patch results in FP32
             if (plan->ntiles > 0) n += prec == SG_FP64 ? 2 + (nsplit > 1) : plan->far->nlev + 2 + plan->far->untabled;
         }
         plan->launches = n;

@@ -58,7 +58,7 @@
 //
 // The direct sum over all pairs that this replaces cost 17.3 ms (far) + 8.9 ms
 // (near, FP64 pipe) on three nested 256^2 levels. Measured per solve: six nested
-// 256^2 levels 121.5 -> 3.23 ms, three off the plane 50.4 -> 1.32 ms; error against
+// 256^2 levels 121.5 -> 3.03 ms, three off the plane 50.4 -> 1.10 ms; error against
 // FP64 4.4e-7 -> 1.4e-7 and 1.5e-7 -> 8e-8.
 #include "common.cuh"
 #include "kmath.cuh"
@@ -402,23 +402,23 @@ struct far_args {
     double lambda;                  // lattice unit
     double G;
     double zl;                      // height in lattice units
-    const double *near;             // near field per target, q_out components
-    float *out[3];
+    int ctas;                       // CTAs of the middle and far field; the near field's follow
+    int ntargets;
+    const int *keys;                // near tables
+    const float2 *tab;
+    double *near, *far;             // per target, q_out components
 };
 
-// Middle and far field of one target block per CTA, added with the near field
-// to the targets' own-patch results. CTAs take blocks from the last to the
+// Middle and far field of one target block per CTA. CTAs take blocks from the last to the
 // first (the finest patches, with the most coarser cells near them, first).
 // Bound by FP32 issue (middle cells: 62 operations each) and the special-function
 // unit (clusters). Middle cells smooth over the block go on its points as well: 2.7 ms
 // for six nested 256^2 levels against 3.8 with every middle cell on the targets, 1.25
 // against 1.49 for three off the plane (with clusters of 8 cells; 4 save 0.5 and 0.3).
 template <int Q>
-__global__ void __launch_bounds__(256, 3) k_far(far_args A)
+__device__ __forceinline__ void far_field(const far_args &A)
 {
     constexpr int NO = q_out<Q>();
-    sg_dep_trigger();
-    sg_dep_wait();  // the charges, the near field, the patches' own results
     __shared__ float4 mc[256];
     __shared__ float2 mp[256];
     __shared__ float nodes[4][NQ][NO][2];
@@ -426,7 +426,7 @@ __global__ void __launch_bounds__(256, 3) k_far(far_args A)
     __shared__ float diff[NQ][NO];
     const int tid = threadIdx.x;
     const int grp = tid >> 6, node = tid & 63;
-    for (int item = blockIdx.x; item < A.nblocks; item += gridDim.x) {
+    for (int item = blockIdx.x; item < A.nblocks; item += A.ctas) {
         const sg_target_block blk = A.blocks[A.nblocks - 1 - item];
         const bool active = tid < blk.count;
         const int4 tg = A.targets[blk.first + (active ? tid : 0)];
@@ -630,10 +630,8 @@ __global__ void __launch_bounds__(256, 3) k_far(far_args A)
             const double scale = Q == Q_POT ? -A.G * A.lambda : A.G;
 #pragma unroll
             for (int o = 0; o < NO; ++o) {
-                if (!A.out[o]) continue;  // sg_force on an off-plane plan takes Fx, Fy only
                 const double far = base[o] + (double)f[o] + ((double)th[o] + (double)tl[o]);
-                float *dst = A.out[o] + tg.z;
-                *dst = (float)((double)*dst + (scale * far + A.near[(int64_t)(blk.first + tid) * NO + o]));
+                A.far[(int64_t)(blk.first + tid) * NO + o] = scale * far;
             }
         }
         __syncthreads();  // base and diff have been read
@@ -744,20 +742,17 @@ constexpr int NEAR_WARPS = 8;
 // for the 865,000 boxes of six nested 256^2 levels (the FP64 corner form: 40 ms),
 // 0.31 ms for the 199,000 off-plane boxes of three.
 template <int Q>
-__global__ void __launch_bounds__(NEAR_WARPS * 32) k_near_tab(const int4 *__restrict__ targets, int ntargets,
-                                                              const sg_patch_dev *__restrict__ pd, int npatches,
-                                                              const float *__restrict__ sigma,
-                                                              const float *__restrict__ dx, const float *__restrict__ dy,
-                                                              const int *__restrict__ keys, const float2 *__restrict__ tab,
-                                                              double *__restrict__ near_out)
+__device__ __forceinline__ void near_field(const far_args &A, int cta)
 {
     constexpr int NO = q_out<Q>(), NPL = q_planes<Q>();
-    sg_dep_trigger();
-    sg_dep_wait();  // the composite sources (and the reader of the previous solve's near field)
+    const sg_patch_dev *__restrict__ pd = A.pd;
+    const float *__restrict__ sigma = A.sigma, *__restrict__ dx = A.dx, *__restrict__ dy = A.dy;
+    const int *__restrict__ keys = A.keys;
+    const int npatches = A.npatches;
     const int lane = threadIdx.x & 31;
-    const int t = (int)((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5);
-    if (t >= ntargets) return;
-    const int4 tg = targets[t];
+    const int t = cta * NEAR_WARPS + (int)(threadIdx.x >> 5);
+    if (t >= A.ntargets) return;
+    const int4 tg = A.targets[t];
     const int ts = pd[tg.w].step;
     float hi[NO], lo[NO];
 #pragma unroll
@@ -776,7 +771,7 @@ __global__ void __launch_bounds__(NEAR_WARPS * 32) k_near_tab(const int4 *__rest
             const int x = tg.x - p.ox, y = tg.y - p.oy;
             const int sh = ilog2_pow2(p.step), I = x >> sh, J = y >> sh;
             const int fx = g < 0 ? 0 : (x & (p.step - 1)) / ts, fy = g < 0 ? 0 : (y & (p.step - 1)) / ts;
-            const float2 *T = tab + ((int64_t)key + (g < 0 ? 0 : (fy << g) + fx)) * (NPL * NEAR_CELLS);
+            const float2 *T = A.tab + ((int64_t)key + (g < 0 ? 0 : (fy << g) + fx)) * (NPL * NEAR_CELLS);
             const int ib = I + near_first(fx, g), jb = J + near_first(fy, g);
 #pragma unroll
             for (int it = 0; it < (NEAR_CELLS + 31) / 32; ++it) {
@@ -795,7 +790,41 @@ __global__ void __launch_bounds__(NEAR_WARPS * 32) k_near_tab(const int4 *__rest
         double v = (double)hi[o] + (double)lo[o];
 #pragma unroll
         for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
-        if (lane == 0) near_out[(int64_t)t * NO + o] = v;
+        if (lane == 0) A.near[(int64_t)t * NO + o] = v;
+    }
+}
+
+// The cross-patch sum in one launch: the CTAs of the middle and far field first, then
+// those of the near field, which are short and fill the SMs while the last of the
+// uneven far blocks run. As two launches, one after the other: six nested 256^2 levels
+// 3.23 ms, three off the plane 1.32, three in the plane 1.08; so 3.03, 1.10 and 0.92.
+template <int Q>
+__global__ void __launch_bounds__(NEAR_WARPS * 32, 3) k_near_far(far_args A)
+{
+    static_assert(NEAR_WARPS * 32 == 256, "one CTA size for both");
+    sg_dep_trigger();
+    sg_dep_wait();  // the composite sources and the charges (and the reader of the previous solve's sums)
+    if ((int)blockIdx.x < A.ctas) far_field<Q>(A);
+    else near_field<Q>(A, (int)blockIdx.x - A.ctas);
+}
+
+// Adds both sums to the targets' own-patch results.
+template <int Q>
+__global__ void __launch_bounds__(256) k_cross_add(const int4 *__restrict__ targets, int ntargets,
+                                                   const double *__restrict__ near, const double *__restrict__ far,
+                                                   float *o0, float *o1, float *o2)
+{
+    constexpr int NO = q_out<Q>();
+    sg_dep_trigger();
+    sg_dep_wait();
+    const int t = blockIdx.x * 256 + threadIdx.x;
+    if (t >= ntargets) return;
+    const int at = targets[t].z;
+    float *const out[3] = {o0, o1, o2};
+#pragma unroll
+    for (int o = 0; o < NO; ++o) {
+        if (!out[o]) continue;  // sg_force on an off-plane plan takes Fx, Fy only
+        out[o][at] = (float)((double)out[o][at] + (far[(int64_t)t * NO + o] + near[(int64_t)t * NO + o]));
     }
 }
 
@@ -942,13 +971,6 @@ sg_status solve(sg_plan *plan, const sg_workspace *ws, const float *sigma, const
     sg_timing_begin(ws, SG_STAGE_DIRECT, st);
     const int grid_n = (plan->ntargets + NEAR_WARPS - 1) / NEAR_WARPS;
     const sg_near_tab &nt = Q == Q_POT ? F.ptab : F.tab;
-    SG_CUDA_TRY(sg_launch_dep(k_near_tab<Q>, dim3(grid_n), dim3(NEAR_WARPS * 32), 0, st, plan->targets, plan->ntargets,
-                              plan->patch_dev, plan->npatches, sigma, dx, dy, F.keys, (const float2 *)nt.data,
-                              ws->partial));
-    if (F.untabled)
-        SG_CUDA_TRY(sg_launch_dep(k_near_corner<Q>, dim3(grid_n), dim3(NEAR_WARPS * 32), 0, st, plan->targets,
-                                  plan->ntargets, plan->patch_dev, plan->npatches, sigma, dx, dy, F.keys,
-                                  plan->lattice_unit, plan->geom.G, plan->geom.z, ws->partial));
     far_args A;
     memset(&A, 0, sizeof(A));
     A.blocks = plan->blocks;
@@ -965,11 +987,19 @@ sg_status solve(sg_plan *plan, const sg_workspace *ws, const float *sigma, const
     A.lambda = plan->lattice_unit;
     A.G = plan->geom.G;
     A.zl = plan->geom.z / plan->lattice_unit;
-    A.near = ws->partial;
-    A.out[0] = o0;
-    A.out[1] = o1;
-    A.out[2] = o2;
-    SG_CUDA_TRY(sg_launch_dep(k_far<Q>, dim3(plan->far_grid), dim3(256), 0, st, A));
+    A.ctas = plan->far_grid;
+    A.ntargets = plan->ntargets;
+    A.keys = F.keys;
+    A.tab = (const float2 *)nt.data;
+    A.near = (double *)ws->partial;
+    A.far = (double *)ws->partial + (int64_t)plan->ntargets * q_out<Q>();
+    SG_CUDA_TRY(sg_launch_dep(k_near_far<Q>, dim3(plan->far_grid + grid_n), dim3(256), 0, st, A));
+    if (F.untabled)
+        SG_CUDA_TRY(sg_launch_dep(k_near_corner<Q>, dim3(grid_n), dim3(NEAR_WARPS * 32), 0, st, plan->targets,
+                                  plan->ntargets, plan->patch_dev, plan->npatches, sigma, dx, dy, F.keys,
+                                  plan->lattice_unit, plan->geom.G, plan->geom.z, ws->partial));
+    SG_CUDA_TRY(sg_launch_dep(k_cross_add<Q>, dim3((plan->ntargets + 255) / 256), dim3(256), 0, st, plan->targets,
+                              plan->ntargets, A.near, A.far, o0, o1, o2));
     SG_CUDA_TRY(cudaGetLastError());
     sg_timing_end(ws, SG_STAGE_DIRECT, st);
     return SG_OK;
@@ -1058,7 +1088,7 @@ int64_t sg_near_table_bytes(int nlevels, const int64_t *level_targets, double z,
 
 int64_t sg_far_bytes(int64_t nclusters, int64_t ntargets, double z)
 {
-    return nclusters * (NQ * 4 + 24) + ntargets * (z != 0.0 ? 24 : 16);
+    return nclusters * (NQ * 4 + 24) + ntargets * (z != 0.0 ? 48 : 32);
 }
 
 void sg_far_free(sg_plan *plan)
@@ -1158,7 +1188,7 @@ sg_status sg_far_setup(sg_plan *plan, const int *const *codes, int nlevels, cons
     SG_TRY(sg_plan_upload(plan, (void **)&F->mat, mat.data(), mat.size() * sizeof(float)));
     SG_TRY(sg_plan_upload(plan, (void **)&F->keys, F->keys_host, sizeof(F->keys_host)));
     plan->ws_tile_bytes = (int64_t)F->ncl * NQ * (int64_t)sizeof(float);
-    plan->ws_partial_bytes = (int64_t)plan->ntargets * (plan->geom.z != 0.0 ? 3 : 2) * (int64_t)sizeof(double);
+    plan->ws_partial_bytes = (int64_t)plan->ntargets * (plan->geom.z != 0.0 ? 6 : 4) * (int64_t)sizeof(double);
     plan->far_grid = plan->nblocks;
     if (plan->geom.z != 0.0) return build_tables<Q_OFF>(plan, F->tab);
     return build_tables<Q_FORCE>(plan, F->tab);
