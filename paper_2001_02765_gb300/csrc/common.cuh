@@ -337,7 +337,7 @@ struct sg_workspace {
     void *tile_w;           // AMR corner weights (FP64 plans: ntiles x SG_TILE_N x 4) or cluster
                             // charges (FP32 plans: 64 per charged cluster)
     double *partial;        // AMR direct-sum partial sums: nsplit x ntargets x 2 (FP64 plans, nsplit > 1);
-                            // the near and the far field, each ntargets x 2 or 3 (FP32 plans)
+                            // near plus far field, ntargets x 2 or 3 (FP32 plans)
     void *zone_buf;         // zone plans: inputs (3 planes) and outputs (2 planes) in patch layout
     int *err;               // device word: err[0] nonzero after a bounded wait in a kernel ran out
     struct sg_timing *timing;  // stage timers, or NULL

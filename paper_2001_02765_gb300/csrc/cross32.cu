@@ -125,14 +125,16 @@ __device__ __forceinline__ int floor_div(int64_t a, int64_t b)
 // the distance from the cell's centre,
 //   q_nm = sum_j [ sum_i (sigma A_n[i] + deltax a B_n[i]) ] A_m[j] + [ sum_i deltay a A_n[i] ] B_m[j].
 // 64 threads per cluster (four clusters per CTA), one charge each; bound by
-// latency (3.5 k FMAs and 192 bytes per cluster).
+// latency (3.5 k FMAs and 192 bytes per cluster). Clears the targets' sums as well.
 __global__ void __launch_bounds__(256) k_p2m(const int4 *__restrict__ desc, int ncl, const sg_patch_dev *__restrict__ pd,
                                              const float *__restrict__ sigma, const float *__restrict__ dx,
                                              const float *__restrict__ dy, double lambda,
-                                             const float *__restrict__ mat, float *__restrict__ charges)
+                                             const float *__restrict__ mat, float *__restrict__ charges,
+                                             double *__restrict__ sums, int nsums)
 {
     sg_dep_trigger();
-    sg_dep_wait();  // the composite sources
+    sg_dep_wait();  // the composite sources (and the reader of the previous solve's sums)
+    for (int64_t e = blockIdx.x * 256LL + threadIdx.x; e < nsums; e += gridDim.x * 256LL) sums[e] = 0.0;
     __shared__ float f[4][3][CL * CL];
     __shared__ float T[4][2][NP * CL];
     const int g = threadIdx.x >> 6, t = threadIdx.x & 63;
@@ -406,7 +408,7 @@ struct far_args {
     int ntargets;
     const int *keys;                // near tables
     const float2 *tab;
-    double *near, *far;             // per target, q_out components
+    double *sums;                   // near + far per target, q_out components, cleared by k_p2m
 };
 
 // Middle and far field of one target block per CTA. CTAs take blocks from the last to the
@@ -631,7 +633,7 @@ __device__ __forceinline__ void far_field(const far_args &A)
 #pragma unroll
             for (int o = 0; o < NO; ++o) {
                 const double far = base[o] + (double)f[o] + ((double)th[o] + (double)tl[o]);
-                A.far[(int64_t)(blk.first + tid) * NO + o] = scale * far;
+                atomicAdd(&A.sums[(int64_t)(blk.first + tid) * NO + o], scale * far);
             }
         }
         __syncthreads();  // base and diff have been read
@@ -790,29 +792,29 @@ __device__ __forceinline__ void near_field(const far_args &A, int cta)
         double v = (double)hi[o] + (double)lo[o];
 #pragma unroll
         for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
-        if (lane == 0) A.near[(int64_t)t * NO + o] = v;
+        if (lane == 0) atomicAdd(&A.sums[(int64_t)t * NO + o], v);
     }
 }
 
 // The cross-patch sum in one launch: the CTAs of the middle and far field first, then
 // those of the near field, which are short and fill the SMs while the last of the
-// uneven far blocks run. As two launches, one after the other: six nested 256^2 levels
+// uneven far blocks run. Each target receives one addend from either, added to zero
+// in either order (the same result). As two launches, one after the other: six nested 256^2 levels
 // 3.23 ms, three off the plane 1.32, three in the plane 1.08; so 3.03, 1.10 and 0.92.
 template <int Q>
 __global__ void __launch_bounds__(NEAR_WARPS * 32, 3) k_near_far(far_args A)
 {
     static_assert(NEAR_WARPS * 32 == 256, "one CTA size for both");
     sg_dep_trigger();
-    sg_dep_wait();  // the composite sources and the charges (and the reader of the previous solve's sums)
+    sg_dep_wait();  // the composite sources, the charges, the cleared sums
     if ((int)blockIdx.x < A.ctas) far_field<Q>(A);
     else near_field<Q>(A, (int)blockIdx.x - A.ctas);
 }
 
-// Adds both sums to the targets' own-patch results.
+// Adds the sums to the targets' own-patch results.
 template <int Q>
 __global__ void __launch_bounds__(256) k_cross_add(const int4 *__restrict__ targets, int ntargets,
-                                                   const double *__restrict__ near, const double *__restrict__ far,
-                                                   float *o0, float *o1, float *o2)
+                                                   const double *__restrict__ sums, float *o0, float *o1, float *o2)
 {
     constexpr int NO = q_out<Q>();
     sg_dep_trigger();
@@ -824,7 +826,7 @@ __global__ void __launch_bounds__(256) k_cross_add(const int4 *__restrict__ targ
 #pragma unroll
     for (int o = 0; o < NO; ++o) {
         if (!out[o]) continue;  // sg_force on an off-plane plan takes Fx, Fy only
-        out[o][at] = (float)((double)out[o][at] + (far[(int64_t)t * NO + o] + near[(int64_t)t * NO + o]));
+        out[o][at] = (float)((double)out[o][at] + sums[(int64_t)t * NO + o]);
     }
 }
 
@@ -961,7 +963,8 @@ sg_status solve(sg_plan *plan, const sg_workspace *ws, const float *sigma, const
     float *charges = (float *)ws->tile_w;
     sg_timing_begin(ws, SG_STAGE_WEIGHTS, st);
     SG_CUDA_TRY(sg_launch_dep(k_p2m, dim3((F.first[1] + 3) / 4), dim3(256), 0, st, F.desc, F.first[1], plan->patch_dev,
-                              sigma, dx, dy, plan->lattice_unit, F.mat, charges));
+                              sigma, dx, dy, plan->lattice_unit, F.mat, charges, ws->partial,
+                              plan->ntargets * q_out<Q>()));
     for (int k = 1; k < F.nlev; ++k) {
         const int n = F.first[k + 1] - F.first[k];
         SG_CUDA_TRY(sg_launch_dep(k_m2m, dim3((n + 3) / 4), dim3(256), 0, st, F.desc, F.first[k], n, F.patch, F.slot,
@@ -991,15 +994,14 @@ sg_status solve(sg_plan *plan, const sg_workspace *ws, const float *sigma, const
     A.ntargets = plan->ntargets;
     A.keys = F.keys;
     A.tab = (const float2 *)nt.data;
-    A.near = (double *)ws->partial;
-    A.far = (double *)ws->partial + (int64_t)plan->ntargets * q_out<Q>();
+    A.sums = ws->partial;
     SG_CUDA_TRY(sg_launch_dep(k_near_far<Q>, dim3(plan->far_grid + grid_n), dim3(256), 0, st, A));
     if (F.untabled)
         SG_CUDA_TRY(sg_launch_dep(k_near_corner<Q>, dim3(grid_n), dim3(NEAR_WARPS * 32), 0, st, plan->targets,
                                   plan->ntargets, plan->patch_dev, plan->npatches, sigma, dx, dy, F.keys,
                                   plan->lattice_unit, plan->geom.G, plan->geom.z, ws->partial));
     SG_CUDA_TRY(sg_launch_dep(k_cross_add<Q>, dim3((plan->ntargets + 255) / 256), dim3(256), 0, st, plan->targets,
-                              plan->ntargets, A.near, A.far, o0, o1, o2));
+                              plan->ntargets, A.sums, o0, o1, o2));
     SG_CUDA_TRY(cudaGetLastError());
     sg_timing_end(ws, SG_STAGE_DIRECT, st);
     return SG_OK;
@@ -1088,7 +1090,7 @@ int64_t sg_near_table_bytes(int nlevels, const int64_t *level_targets, double z,
 
 int64_t sg_far_bytes(int64_t nclusters, int64_t ntargets, double z)
 {
-    return nclusters * (NQ * 4 + 24) + ntargets * (z != 0.0 ? 48 : 32);
+    return nclusters * (NQ * 4 + 24) + ntargets * (z != 0.0 ? 24 : 16);
 }
 
 void sg_far_free(sg_plan *plan)
@@ -1188,7 +1190,7 @@ sg_status sg_far_setup(sg_plan *plan, const int *const *codes, int nlevels, cons
     SG_TRY(sg_plan_upload(plan, (void **)&F->mat, mat.data(), mat.size() * sizeof(float)));
     SG_TRY(sg_plan_upload(plan, (void **)&F->keys, F->keys_host, sizeof(F->keys_host)));
     plan->ws_tile_bytes = (int64_t)F->ncl * NQ * (int64_t)sizeof(float);
-    plan->ws_partial_bytes = (int64_t)plan->ntargets * (plan->geom.z != 0.0 ? 6 : 4) * (int64_t)sizeof(double);
+    plan->ws_partial_bytes = (int64_t)plan->ntargets * (plan->geom.z != 0.0 ? 3 : 2) * (int64_t)sizeof(double);
     plan->far_grid = plan->nblocks;
     if (plan->geom.z != 0.0) return build_tables<Q_OFF>(plan, F->tab);
     return build_tables<Q_FORCE>(plan, F->tab);
