@@ -140,7 +140,8 @@ typedef struct sg_plan sg_plan;
  * overlap; a patch of level l+1 has h = h_l / 2, lies inside one level-l patch,
  * starts on that patch's cell lattice and covers whole parent cells (even nx,
  * ny); patches of one level do not overlap; at most 12 levels; the lattice of
- * the finest level's half-cells spans at most 2^23 units per axis; a single
+ * the finest level's half-cells spans at most 2^23 units per axis; the patches
+ * have at most 2^31 - 256 cells together (indexes are 32-bit); a single
  * patch has at most 2048 cells per side. slope_mode SG_SLOPES_CENTRAL needs a
  * single patch. Masks, where given, follow the rules stated at sg_geom.masks.
  * Returns SG_OK or SG_EINVAL.

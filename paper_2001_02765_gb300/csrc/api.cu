@@ -124,7 +124,9 @@ sg_status analyse(const sg_geom *g, geom_info &gi)
         if (P[k].level < 0 || P[k].level >= SG_MAX_LEVELS) return fail("patch level out of range");
         if (k > 0 && P[k].level < P[k - 1].level) return fail("patches are not sorted by level");
         if (P[k].level > gi.lmax) gi.lmax = P[k].level;
+        gi.ncells += (int64_t)P[k].nx * P[k].ny;
     }
+    if (gi.ncells > SG_MAX_CELLS) return fail("geometry has more than 2^31 - 256 cells");
     gi.h0 = P[0].h;
     gi.X0 = P[0].x0;
     gi.Y0 = P[0].y0;

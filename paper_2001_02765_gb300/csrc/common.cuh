@@ -119,6 +119,9 @@ struct __align__(32) sg_dvec4 {
 #define SG_LEN_SLOTS 48
 #define SG_MAX_PATCH_SIDE 2048
 #define SG_MAX_LEVELS 12
+// Cells of a geometry: cell indexes and target counts are 32-bit, and kernels round
+// target counts up to whole CTAs of at most 256.
+#define SG_MAX_CELLS ((1LL << 31) - 256)
 
 // Source tiles of the cross-patch direct sum of FP64 plans (corner form):
 // TILE_X x TILE_Y corners.

@@ -130,7 +130,7 @@ __global__ void __launch_bounds__(256) k_p2m(const int4 *__restrict__ desc, int 
                                              const float *__restrict__ sigma, const float *__restrict__ dx,
                                              const float *__restrict__ dy, double lambda,
                                              const float *__restrict__ mat, float *__restrict__ charges,
-                                             double *__restrict__ sums, int nsums)
+                                             double *__restrict__ sums, int64_t nsums)
 {
     sg_dep_trigger();
     sg_dep_wait();  // the composite sources (and the reader of the previous solve's sums)
@@ -964,7 +964,7 @@ sg_status solve(sg_plan *plan, const sg_workspace *ws, const float *sigma, const
     sg_timing_begin(ws, SG_STAGE_WEIGHTS, st);
     SG_CUDA_TRY(sg_launch_dep(k_p2m, dim3((F.first[1] + 3) / 4), dim3(256), 0, st, F.desc, F.first[1], plan->patch_dev,
                               sigma, dx, dy, plan->lattice_unit, F.mat, charges, ws->partial,
-                              plan->ntargets * q_out<Q>()));
+                              (int64_t)plan->ntargets * q_out<Q>()));
     for (int k = 1; k < F.nlev; ++k) {
         const int n = F.first[k + 1] - F.first[k];
         SG_CUDA_TRY(sg_launch_dep(k_m2m, dim3((n + 3) / 4), dim3(256), 0, st, F.desc, F.first[k], n, F.patch, F.slot,

@@ -1,0 +1,123 @@
+// Host side of the FP32 cross-patch sum (cross32.cu) on a CPU: the CUDA runtime
+// calls it makes are replaced by the fakes below, which record every launch.
+// Usage: cross_host SCENARIO; exits 0 when the scenario holds.
+#include "../paper_2001_02765_gb300/csrc/cross32.cu"
+
+#include <stdio.h>
+#include <stdlib.h>
+
+#include <tuple>
+
+struct launch {
+    const void *kern;
+    unsigned grid;
+    void **args;
+};
+static std::vector<launch> g_launches;
+static int64_t g_sums = -1;  // how many target sums the level-0 charge kernel was told to clear
+
+// the last argument of a kernel, whatever its integer type
+template <typename... A>
+static int64_t last_arg(void (*)(A...), void **args)
+{
+    using last = std::tuple_element_t<sizeof...(A) - 1, std::tuple<A...>>;
+    return (int64_t)*(const last *)args[sizeof...(A) - 1];
+}
+
+#ifndef __CUDA_ARCH__
+extern "C" {
+cudaError_t cudaMalloc(void **p, size_t n) { return (*p = calloc(n, 1)) ? cudaSuccess : cudaErrorMemoryAllocation; }
+cudaError_t cudaFree(void *p)
+{
+    free(p);
+    return cudaSuccess;
+}
+cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t *c, const void *kern, void **args)
+{
+    g_launches.push_back({kern, c->gridDim.x, args});
+    if (kern == (const void *)k_p2m) g_sums = last_arg(k_p2m, args);
+    return c->gridDim.x >= 1 ? cudaSuccess : cudaErrorInvalidConfiguration;
+}
+cudaError_t cudaLaunchKernel(const void *kern, dim3 grid, dim3, void **args, size_t, cudaStream_t)
+{
+    g_launches.push_back({kern, grid.x, args});
+    return cudaSuccess;
+}
+cudaError_t cudaGetLastError() { return cudaSuccess; }
+cudaError_t cudaDeviceSynchronize() { return cudaSuccess; }
+}
+#endif
+
+// what cross32.cu takes from the rest of the library
+void sg_set_last_cuda_error(cudaError_t, const char *) {}
+void sg_set_last_error_message(const char *) {}
+void sg_timing_begin(const sg_workspace *, int, cudaStream_t) {}
+void sg_timing_end(const sg_workspace *, int, cudaStream_t) {}
+sg_status sg_plan_upload(sg_plan *plan, void **dst, const void *src, size_t n)
+{
+    *dst = malloc(n ? n : 1);
+    if (n) memcpy(*dst, src, n);
+    plan->device_bytes += (int64_t)n;
+    return SG_OK;
+}
+
+// A plan of the given patches (nx, ny, existing cells or none), all on one level.
+struct shape {
+    int nx, ny;
+    bool any;
+};
+static sg_status make_plan(sg_plan *plan, sg_workspace *ws, const std::vector<shape> &patches, double z)
+{
+    memset(plan, 0, sizeof(*plan));
+    memset(ws, 0, sizeof(*ws));
+    plan->npatches = (int)patches.size();
+    plan->pp = new sg_patch_plan[patches.size()]();
+    plan->geom.z = z;
+    plan->lattice_unit = 1.0;
+    std::vector<std::vector<int>> code;
+    std::vector<const int *> codes;
+    int64_t leaves = 0;
+    for (size_t p = 0; p < patches.size(); ++p) {
+        plan->pp[p].d.nx = patches[p].nx;
+        plan->pp[p].d.ny = patches[p].ny;
+        plan->pp[p].d.step = 2;
+        code.emplace_back((size_t)patches[p].nx * patches[p].ny, patches[p].any ? SG_CELL_LEAF : SG_CELL_ABSENT);
+        if (patches[p].any) leaves += (int64_t)patches[p].nx * patches[p].ny;
+    }
+    for (const auto &c : code) codes.push_back(c.data());
+    plan->ntargets = (int)leaves;
+    plan->nblocks = 1;
+    return sg_far_setup(plan, codes.data(), 1, &leaves, SG_NT_GMAX);
+}
+
+#define CHECK(x)                                                              \
+    do {                                                                      \
+        if (!(x)) {                                                           \
+            fprintf(stderr, "%s:%d: %s does not hold\n", __FILE__, __LINE__, #x); \
+            return 1;                                                         \
+        }                                                                     \
+    } while (0)
+
+// every target's sums are cleared, also where their number exceeds 32 bits
+static int clears_every_sum()
+{
+    for (double z : {0.0, 0.5}) {
+        sg_plan plan;
+        sg_workspace ws;
+        CHECK(make_plan(&plan, &ws, {{8, 8, true}, {8, 8, true}}, z) == SG_OK);
+        for (int64_t n : {(int64_t)128, (int64_t)1 << 30, ((int64_t)1 << 31) - 256}) {
+            plan.ntargets = (int)n;
+            CHECK(sg_far_solve(&plan, &ws, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, 0) == SG_OK);
+            CHECK(g_sums == n * (z != 0.0 ? 3 : 2));
+        }
+    }
+    return 0;
+}
+
+int main(int argc, char **argv)
+{
+    const char *s = argc > 1 ? argv[1] : "";
+    if (!strcmp(s, "clears_every_sum")) return clears_every_sum();
+    fprintf(stderr, "unknown scenario '%s'\n", s);
+    return 2;
+}
