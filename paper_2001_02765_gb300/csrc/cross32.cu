@@ -1161,6 +1161,8 @@ sg_status sg_far_setup(sg_plan *plan, const int *const *codes, int nlevels, cons
         }
     }
     for (int k = nlev; k <= SG_CL_LEVELS; ++k) F->first[k] = (int)desc.size();
+    // (the levels of a patch without an existing cell hold no cluster; a launch over none is an error)
+    while (nlev > 1 && F->first[nlev] == F->first[nlev - 1]) --nlev;
     F->nlev = nlev;
     F->ncl = (int)desc.size();
     // interpolation matrices: A_n[i], B_n[i] (8-point Gauss-Legendre, exact for these degrees), C_h[n'][n]

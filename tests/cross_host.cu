@@ -114,10 +114,34 @@ static int clears_every_sum()
     return 0;
 }
 
+// a patch without an existing cell adds no launch (its levels hold no cluster)
+static int empty_patch_adds_no_launch()
+{
+    for (const shape &empty : {shape{256, 256, false}, shape{4, 4, false}}) {
+        size_t n[2];
+        int nlev[2];
+        for (int k = 0; k < 2; ++k) {
+            sg_plan plan;
+            sg_workspace ws;
+            std::vector<shape> patches = {{16, 16, true}, {12, 16, true}};
+            if (k == 1) patches.push_back(empty);
+            CHECK(make_plan(&plan, &ws, patches, 0.0) == SG_OK);
+            g_launches.clear();
+            CHECK(sg_far_solve(&plan, &ws, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, 0) == SG_OK);
+            for (const launch &l : g_launches) CHECK(l.grid >= 1);
+            n[k] = g_launches.size();
+            nlev[k] = plan.far->nlev;
+        }
+        CHECK(n[0] == n[1] && nlev[0] == nlev[1] && nlev[0] == 3);
+    }
+    return 0;
+}
+
 int main(int argc, char **argv)
 {
     const char *s = argc > 1 ? argv[1] : "";
     if (!strcmp(s, "clears_every_sum")) return clears_every_sum();
+    if (!strcmp(s, "empty_patch_adds_no_launch")) return empty_patch_adds_no_launch();
     fprintf(stderr, "unknown scenario '%s'\n", s);
     return 2;
 }

@@ -18,8 +18,9 @@ def host(tmp_path_factory):
     return lambda scenario: subprocess.run([exe, scenario], capture_output=True, text=True, timeout=120)
 
 
-def test_clears_every_sum(host):
-    r = host("clears_every_sum")
+@pytest.mark.parametrize("scenario", ["clears_every_sum", "empty_patch_adds_no_launch"])
+def test_host_side(host, scenario):
+    r = host(scenario)
     assert r.returncode == 0, r.stderr
 
 

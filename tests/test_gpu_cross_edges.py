@@ -1,0 +1,38 @@
+"""Edges of the FP32 cross-patch sum: patches that a mask leaves without a cell."""
+import numpy as np
+import pytest
+
+from tests._lib import concat_dev, ensure_built
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def sg():
+    import torch
+    assert torch.cuda.is_available()
+    ensure_built()
+    from paper_2001_02765_gb300 import sg as mod
+    return mod
+
+
+@pytest.mark.parametrize("kind", ["force", "potential", "force3"])
+def test_patch_without_a_cell_changes_nothing(sg, kind):
+    """The empty patch is wider than the others (more cluster levels): the solve runs
+    and every other patch's result is that of the plan without it, bit for bit."""
+    import torch
+    h = 1.0 / 32
+    patches = [(0, 16, 16, 0.0, 0.0, h), (0, 12, 20, 16 * h, 0.0, h), (0, 256, 256, 28 * h, 0.0, h)]
+    masks = [None, None, np.zeros((256, 256), np.uint8)]
+    rng = np.random.Generator(np.random.PCG64(5))
+    f = [[rng.uniform(-1, 1, (p[2], p[1])) for p in patches] for _ in range(3)]
+    out = []
+    for n in (2, 3):
+        plan = sg.Plan(patches[:n], z=0.5 * h if kind == "force3" else 0.0, cross_mode=sg.SG_CROSS_DIRECT,
+                       masks=masks[:n] if n == 3 else None)
+        r = getattr(plan, kind)(*[concat_dev(a[:n], np.float32) for a in f])
+        torch.cuda.synchronize()
+        m = 16 * 16 + 12 * 20
+        out.append([t[:m].clone() for t in (r if isinstance(r, tuple) else (r,))])
+        plan.close()
+    assert all(torch.equal(a, b) for a, b in zip(*out))
