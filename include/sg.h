@@ -472,8 +472,8 @@ sg_status sg_autotune(int precision, int min_pad, int max_pad, int reps, double 
  * ranges per target block of FP64 plans (the plan's value, a half or a quarter
  * of it; 1 in FP32 plans) and, for FP32 plans, the CTAs of the far-field launch
  * (one per target block, or 1, 2, 3, 4, 6 or 8 per SM that share the blocks),
- * each timed as the median of `reps` solves on zero fields with the plan's own
- * workspace; the fastest pair stays in the plan. The split only regroups the FP64
+ * each timed as the median of `reps` solves with density in every cell on the
+ * plan's own workspace; the fastest pair stays in the plan. The split only regroups the FP64
  * partial sums (results agree to FP64 rounding; the far-field grid changes nothing). Synchronous; call with no
  * solve of the plan in flight and before capturing the plan into a batch.
  * sg_plan_direct_shape reads the pair. best_ms may be NULL. Errors: SG_EINVAL,

@@ -66,6 +66,15 @@ bool knob_feasible(int knob, int pad, int v, bool fp64)
     return col_smem(pad, v, knob == 2 ? 9 : 6, fp64) <= 200 * 1024 && col_smem(pad, v, 3, fp64) <= 200 * 1024;
 }
 
+// Values in [1/2, 3/2), different from cell to cell: the cross-patch sum leaves out
+// cells without density, so zero fields would time only part of a solve.
+template <typename T>
+__global__ void k_tune_fill(T *__restrict__ f, int64_t n)
+{
+    for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < n; k += (int64_t)gridDim.x * blockDim.x)
+        f[k] = (T)0.5 + (T)((uint32_t)k * 2654435761u >> 8) * (T)(1.0 / (1 << 24));
+}
+
 std::vector<int> knob_candidates(int knob, int pad, bool fp64)
 {
     std::vector<int> c;
@@ -201,11 +210,11 @@ sg_status sg_autotune(int precision, int min_pad, int max_pad, int reps, double 
     return st;
 }
 
-// The cross-patch direct sum of one plan: source-tile ranges per target block
+// The cross-patch sum of one plan: source-tile ranges per target block of FP64 plans
 // (the plan's value, a half and a quarter of it: the partial-sum buffers were
-// sized for the plan's value) and, for FP32 plans, the CTAs of the persistent
-// far-field launch (1, 2, 3, 4, 6 or 8 per SM), timed on the plan's own
-// workspace with zero fields, the fastest kept.
+// sized for the plan's value) or, for FP32 plans, the CTAs of the middle and far
+// field (one per target block, or 1, 2, 3, 4, 6 or 8 per SM), timed on the plan's
+// own workspace with density in every cell, the fastest kept.
 sg_status sg_plan_autotune(sg_plan *plan, int reps, double *best_ms)
 {
     if (!plan || reps < 1) {
@@ -224,7 +233,9 @@ sg_status sg_plan_autotune(sg_plan *plan, int reps, double *best_ms)
     char *buf = nullptr;
     SG_CUDA_TRY(cudaMalloc(&buf, (size_t)(6 * n * es)));
     cudaEvent_t e0 = nullptr, e1 = nullptr;
-    sg_status st = cudaMemset(buf, 0, (size_t)(6 * n * es)) == cudaSuccess ? SG_OK : SG_ECUDA;
+    if (es == 8) k_tune_fill<<<1024, 256>>>((double *)buf, 3 * n);
+    else k_tune_fill<<<1024, 256>>>((float *)buf, 3 * n);
+    sg_status st = cudaGetLastError() == cudaSuccess ? SG_OK : SG_ECUDA;
     if (st == SG_OK && (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess)) st = SG_ECUDA;
     auto solve = [&]() -> sg_status {
         if (plan->geom.z != 0.0) return sg_force3(plan, buf, buf + n * es, buf + 2 * n * es, buf + 3 * n * es,
