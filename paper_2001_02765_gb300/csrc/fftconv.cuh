@@ -318,6 +318,17 @@ __device__ __forceinline__ C rot8(C a, int q)
     return a;
 }
 
+// sin(t + 2 pi q / 8), q = 0 .. 7, from a = (cos t, sin t) and b = (cos u, sin u) with
+// u = pi/4 - t: every one is an entry of either, so as good as the table's. (Turned
+// like the edge rows' factors, the sines near u = 0 come out of a cancellation, with
+// a relative error of the rounding over sin u.)
+template <typename C>
+__host__ __device__ __forceinline__ auto eighth_sine(C a, C b, int q)
+{
+    const auto s = (q & 1) ? ((q & 2) ? b.y : b.x) : ((q & 2) ? a.x : a.y);
+    return (q & 4) ? -s : s;
+}
+
 // Shared-memory layout of the column kernels: the padded FFT buffer, then the
 // kernel spectra of the CTA's columns, [planes][CB][sg_spec_stride(PY)] of T,
 // which one thread fetches with one 1-D bulk copy (TMA) per plane at kernel
@@ -765,11 +776,13 @@ __device__ __forceinline__ void col_central_body(const col_args<T> &args, int bx
     if (!spectra_ready(&bar, err, args.tries)) return;
     if (CO && threadIdx.x == 0) mbar_inval(&bar);  // every thread has passed its wait; the body runs again
 
-    // the slope factors of the column, and of the bins jt + q PY/8: those of bin jt
-    // turned by q (and -ny q) eighths, so one load instead of eight
+    // the slope factors of the column, and of the bins jt + q PY/8: the edge rows' from
+    // those of bin jt, turned by q (and -ny q) eighths, and the sines from those of jt
+    // and of its mirror PY/8 - jt (see eighth_sine): two loads instead of eight
     C e1, e2, f1, f2;
     ld_pair<false>(cpair, kx < qx ? kx : 0, e1, e2);
     ld_pair<false>(rpair, jt, f1, f2);
+    const C g1 = rpair[2 * (STEP - jt)];
     C r0 = rows[c < CB ? c : 0][0], r1 = rows[c < CB ? c : 0][1];
     r0 = cmul_rn(f1, r0);
     r1 = cmul_rn(f2, r1);
@@ -785,7 +798,7 @@ __device__ __forceinline__ void col_central_body(const col_args<T> &args, int bx
         const T *sp = ssp + c * QS + kq;  // plane p at sp[p * CB * QS]
         const C S = v[q];
         // slope spectra
-        const T cs = (T)2 * e1.y, rs = (T)2 * rot8(f1, q).y;  // sin(2 pi k / P) / h
+        const T cs = (T)2 * e1.y, rs = (T)2 * eighth_sine(f1, g1, q);  // sin(2 pi k / P) / h, exactly
         C c0, c1;
         ld_pair<CO>(edge, ky, c0, c1);
         // every operation explicitly rounded (see mul_rn): the result must not depend on the launch shape
@@ -876,11 +889,13 @@ __global__ void __launch_bounds__(THREADS, (col_central_blocks<T, PY, CB, THREAD
     fft_regs<C, PY, CB, THREADS, NBUF, false>(v, bufs, par, tw);
     if (!spectra_ready(&bar, err, args.tries)) return;
 
-    // the slope factors of the column, and of the bins jt + q PY/8: those of bin jt
-    // turned by q (and -ny q) eighths, so one load instead of eight
+    // the slope factors of the column, and of the bins jt + q PY/8: the edge rows' from
+    // those of bin jt, turned by q (and -ny q) eighths, and the sines from those of jt
+    // and of its mirror PY/8 - jt (see eighth_sine): two loads instead of eight
     C e1, e2, f1, f2;
     ld_pair<false>(cpair, kx < qx ? kx : 0, e1, e2);
     ld_pair<false>(rpair, jt, f1, f2);
+    const C g1 = rpair[2 * (STEP - jt)];
     C r0 = rows[c < CB ? c : 0][0], r1 = rows[c < CB ? c : 0][1];
     r0 = cmul_rn(f1, r0);
     r1 = cmul_rn(f2, r1);
@@ -898,7 +913,7 @@ __global__ void __launch_bounds__(THREADS, (col_central_blocks<T, PY, CB, THREAD
         const T *sp = ssp + c * QS + kq;  // plane p at sp[p * CB * QS]
         const C S = v[q];
         // slope spectra
-        const T cs = (T)2 * e1.y, rs = (T)2 * rot8(f1, q).y;  // sin(2 pi k / P) / h
+        const T cs = (T)2 * e1.y, rs = (T)2 * eighth_sine(f1, g1, q);  // sin(2 pi k / P) / h, exactly
         C c0, c1;
         ld_pair<false>(edge, ky, c0, c1);
         // every operation explicitly rounded (see mul_rn): the result must not depend on the launch shape
