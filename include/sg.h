@@ -226,8 +226,7 @@ sg_status sg_force3(sg_plan *plan, const void *sigma, const void *deltax, const 
  * Mid-plane potential (Section 2: Phi(x, y, 0) = -G times the integral of
  * K(xbar - x, ybar - y, 0) sigma with K = 1/r, the singular kernel integral
  * whose gradient gives the force) at every cell centre of a plan in the plane
- * (z == 0): one unmasked patch, with the plan's slope mode (central slopes are
- * formed in the row transform here), or a hierarchy (patches, masks) on either
+ * (z == 0): one unmasked patch, with the plan's slope mode, or a hierarchy (patches, masks) on either
  * path of its plan (level convolutions, or each patch's own convolution plus
  * the cross-patch sum: the corner form in FP64 plans, tabulated near cells, a
  * moment expansion and clusters of far cells in FP32 plans), summed over the leaf
@@ -236,8 +235,10 @@ sg_status sg_force3(sg_plan *plan, const void *sigma, const void *deltax, const 
  *   P^0, P^x, P^y = integrals over cell i of 1/r, (xbar - xc_i)/r, (ybar - yc_i)/r,
  * from the antiderivatives u ln(v + r) + v ln(u + r) and (v r + u^2 ln(v + r))/2
  * (finite everywhere, the own cell included). The first call on a plan builds
- * its three FP64-built potential spectra synchronously (legacy default
- * stream); later calls only enqueue on `stream`.
+ * its three FP64-built potential spectra and, in FP32 plans on the direct path,
+ * the near tables of the potential synchronously (legacy default stream; both
+ * come on top of the plan's hbm_budget and sg_plan_bytes, and a call that could
+ * not build them leaves none); later calls only enqueue on `stream`.
  *   sigma, deltax, deltay  as for sg_force;  phi  device pointer, ncells elements
  * Errors: SG_EINVAL (off the plane, null or misaligned pointer, missing caller
  * slopes), SG_ENOMEM, SG_ECUDA.

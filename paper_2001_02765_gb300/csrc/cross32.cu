@@ -1007,13 +1007,28 @@ sg_status solve(sg_plan *plan, const sg_workspace *ws, const float *sigma, const
     return SG_OK;
 }
 
+template <int Q>
+size_t table_bytes(const sg_far &F)
+{
+    return (size_t)std::max(1, F.nclass) * q_planes<Q>() * NEAR_CELLS * sizeof(float2);
+}
+
+// Give back tables whose build failed (nt.data set means built).
+template <int Q>
+void drop_tables(sg_plan *plan, sg_near_tab &nt)
+{
+    if (!nt.data) return;
+    cudaFree(nt.data);
+    nt.data = nullptr;
+    plan->device_bytes -= (int64_t)table_bytes<Q>(*plan->far);
+}
+
 // Build the near tables of quantity Q (asynchronous on the legacy default stream).
 template <int Q>
 sg_status build_tables(sg_plan *plan, sg_near_tab &nt)
 {
     sg_far &F = *plan->far;
-    const size_t cls = (size_t)q_planes<Q>() * NEAR_CELLS * sizeof(float2);
-    const size_t bytes = std::max<size_t>(1, F.nclass) * cls;
+    const size_t bytes = table_bytes<Q>(F);
     cudaError_t e = cudaMalloc(&nt.data, bytes);
     if (e != cudaSuccess) {
         cudaGetLastError();
@@ -1039,7 +1054,12 @@ sg_status build_tables(sg_plan *plan, sg_near_tab &nt)
     if (F.nclass == 0) return SG_OK;
     const int grid = (int)std::min<int64_t>(((int64_t)F.nclass * NEAR_CELLS + 127) / 128, 1 << 16);
     k_near_table<Q><<<grid, 128>>>((float2 *)nt.data, L, plan->geom.G, plan->geom.z);
-    SG_CUDA_TRY(cudaGetLastError());
+    e = cudaGetLastError();
+    if (e != cudaSuccess) {
+        drop_tables<Q>(plan, nt);
+        sg_set_last_cuda_error(e, "k_near_table");
+        return SG_ECUDA;
+    }
     return SG_OK;
 }
 
@@ -1204,6 +1224,7 @@ sg_status sg_far_potential_tables(sg_plan *plan)
     sg_status s = build_tables<Q_POT>(plan, plan->far->ptab);
     cudaError_t e = cudaDeviceSynchronize();
     if (s == SG_OK && e != cudaSuccess) {
+        drop_tables<Q_POT>(plan, plan->far->ptab);
         sg_set_last_cuda_error(e, "near tables of the potential");
         s = SG_ECUDA;
     }

@@ -14,6 +14,8 @@ struct launch {
     void **args;
 };
 static std::vector<launch> g_launches;
+static cudaError_t g_launch_error = cudaSuccess, g_sync_error = cudaSuccess;  // what the fakes report
+static int64_t g_live = 0;   // device allocations not yet freed
 static int64_t g_sums = -1;  // how many target sums the level-0 charge kernel was told to clear
 
 // the last argument of a kernel, whatever its integer type
@@ -26,9 +28,14 @@ static int64_t last_arg(void (*)(A...), void **args)
 
 #ifndef __CUDA_ARCH__
 extern "C" {
-cudaError_t cudaMalloc(void **p, size_t n) { return (*p = calloc(n, 1)) ? cudaSuccess : cudaErrorMemoryAllocation; }
+cudaError_t cudaMalloc(void **p, size_t n)
+{
+    ++g_live;
+    return (*p = calloc(n, 1)) ? cudaSuccess : cudaErrorMemoryAllocation;
+}
 cudaError_t cudaFree(void *p)
 {
+    if (p) --g_live;
     free(p);
     return cudaSuccess;
 }
@@ -38,13 +45,14 @@ cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t *c, const void *kern, v
     if (kern == (const void *)k_p2m) g_sums = last_arg(k_p2m, args);
     return c->gridDim.x >= 1 ? cudaSuccess : cudaErrorInvalidConfiguration;
 }
-cudaError_t cudaLaunchKernel(const void *kern, dim3 grid, dim3, void **args, size_t, cudaStream_t)
+// (a launch by <<<>>>)
+cudaError_t __cudaLaunchKernel(cudaKernel_t kern, dim3 grid, dim3, void **args, size_t, cudaStream_t)
 {
-    g_launches.push_back({kern, grid.x, args});
+    g_launches.push_back({(const void *)kern, grid.x, args});
     return cudaSuccess;
 }
-cudaError_t cudaGetLastError() { return cudaSuccess; }
-cudaError_t cudaDeviceSynchronize() { return cudaSuccess; }
+cudaError_t cudaGetLastError() { return g_launch_error; }
+cudaError_t cudaDeviceSynchronize() { return g_sync_error; }
 }
 #endif
 
@@ -137,11 +145,32 @@ static int empty_patch_adds_no_launch()
     return 0;
 }
 
+// tables of the potential that could not be built are not taken for built by the next call
+static int unbuilt_tables_are_dropped()
+{
+    sg_plan plan;
+    sg_workspace ws;
+    CHECK(make_plan(&plan, &ws, {{16, 16, true}, {12, 16, true}}, 0.0) == SG_OK);
+    const int64_t bytes = plan.device_bytes, live = g_live;
+    for (int k = 0; k < 2; ++k) {
+        (k == 0 ? g_launch_error : g_sync_error) = cudaErrorLaunchFailure;
+        CHECK(sg_far_potential_tables(&plan) == SG_ECUDA);
+        g_launch_error = g_sync_error = cudaSuccess;
+        CHECK(!plan.far->ptab.data && plan.device_bytes == bytes && g_live == live);
+    }
+    g_launches.clear();
+    CHECK(sg_far_potential_tables(&plan) == SG_OK);
+    CHECK(g_launches.size() == 1 && plan.far->ptab.data && plan.device_bytes > bytes);
+    CHECK(sg_far_potential_tables(&plan) == SG_OK && g_launches.size() == 1);
+    return 0;
+}
+
 int main(int argc, char **argv)
 {
     const char *s = argc > 1 ? argv[1] : "";
     if (!strcmp(s, "clears_every_sum")) return clears_every_sum();
     if (!strcmp(s, "empty_patch_adds_no_launch")) return empty_patch_adds_no_launch();
+    if (!strcmp(s, "unbuilt_tables_are_dropped")) return unbuilt_tables_are_dropped();
     fprintf(stderr, "unknown scenario '%s'\n", s);
     return 2;
 }

@@ -18,7 +18,7 @@ def host(tmp_path_factory):
     return lambda scenario: subprocess.run([exe, scenario], capture_output=True, text=True, timeout=120)
 
 
-@pytest.mark.parametrize("scenario", ["clears_every_sum", "empty_patch_adds_no_launch"])
+@pytest.mark.parametrize("scenario", ["clears_every_sum", "empty_patch_adds_no_launch", "unbuilt_tables_are_dropped"])
 def test_host_side(host, scenario):
     r = host(scenario)
     assert r.returncode == 0, r.stderr
