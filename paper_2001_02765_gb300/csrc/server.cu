@@ -185,15 +185,14 @@ void claim(sg_server *s, const std::vector<sg_request *> &mem, int slot)
         s->bytes_in_use += r->bytes;
         s->running.push_back(r);
     }
-    s->peak_bytes = std::max(s->peak_bytes, s->bytes_in_use);
     s->err_host[slot] = 0;
 }
 
-// Undo claim (lock held): back to the head of the queue, in order.
+// Undo claim (lock held): back into the queue in arrival order (a group's members
+// may have had other requests between them).
 void unclaim(sg_server *s, const std::vector<sg_request *> &mem, int slot)
 {
-    for (size_t k = mem.size(); k-- > 0;) {
-        sg_request *r = mem[k];
+    for (sg_request *r : mem) {
         s->running.erase(std::find(s->running.begin(), s->running.end(), r));
         s->bytes_in_use -= r->bytes;
         if (s->stop) {  // the server is being destroyed: as the queued ones
@@ -202,7 +201,9 @@ void unclaim(sg_server *s, const std::vector<sg_request *> &mem, int slot)
             s->cancelled++;
         } else {
             r->state.store(RQ_QUEUED);
-            s->queue.push_front(r);
+            s->queue.insert(std::lower_bound(s->queue.begin(), s->queue.end(), r,
+                                             [](sg_request *a, sg_request *b) { return a->ticket < b->ticket; }),
+                            r);
         }
     }
     s->free_slots.push_back(slot);
@@ -236,6 +237,7 @@ bool start(sg_server *s, sg_request *r, std::unique_lock<std::mutex> &lock)
         r->state.store(RQ_GPU_DONE);
     }
     lock.lock();
+    s->peak_bytes = std::max(s->peak_bytes, s->bytes_in_use);
     return true;
 }
 
@@ -335,6 +337,7 @@ bool start_group(sg_server *s, const std::vector<sg_request *> &mem, std::unique
         }
     }
     lock.lock();
+    s->peak_bytes = std::max(s->peak_bytes, s->bytes_in_use);
     s->groups_started++;
     s->grouped_requests += mem.size();
     return true;
