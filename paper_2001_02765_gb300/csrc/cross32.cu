@@ -38,9 +38,10 @@
 //    L the Lagrange polynomials: interpolation of the kernel in the source
 //    coordinate (a black-box fast multipole method; barycentric Lagrange
 //    treecode of Wang, Krasny & Tlupova 2020). It serves every kernel: a charge
-//    acts as a point mass. With the target at least 4 a from the centre (maximum
-//    norm) the interpolation error is below 2e-7 of the cluster's own field
-//    (5e-8 rms; measured over random densities) and falls as 8^-8 with distance.
+//    acts as a point mass. With the target 4 a from the centre (maximum norm) the
+//    interpolation errs by at most 3.3e-6 of a charge's own field (5.2e-7 rms over the
+//    square; the potential 4.0e-7 and 4.6e-8), with the sign changing from charge to
+//    charge; it falls as the eighth power of the distance (7e-9 at 8 a).
 //    Charges of level 0 come from the cells (k_p2m), those of level k + 1 from
 //    level k by the same interpolation (k_m2m).
 //    Each block of up to 256 targets (16 x 16 cells) takes, per source patch, at
