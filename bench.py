@@ -265,13 +265,13 @@ def run_batch(args):
     torch.cuda.set_device(local)
     ns, a, amp = W.batch_sizes(count=args.batch_size, lo=64, hi=512, seed=4 + rank)
     # launch shapes picked by the library's autotuner for the padded lengths of the batch
-    pads = sorted({sg_pad(int(n)) for n in ns})
+    pads = sorted({_pad(int(n)) for n in ns})
     tuned, tune_s = None, 0.0
     if not args.no_autotune:
         t0 = time.perf_counter()
-        res = sg.sg_autotune(sg.SG_FP32, pads[0], pads[-1], reps=15)
+        sg.sg_autotune(sg.SG_FP32, pads[0], pads[-1], reps=15)
         tune_s = time.perf_counter() - t0
-        tuned = {str(p): res[p][0] for p in pads}
+        tuned = {str(p): sg.sg_tune_get(sg.SG_FP32, p) for p in pads}
 
     def build(precision):
         # the members' fields are views of one input and one output allocation, so
@@ -868,9 +868,10 @@ def run_gpu(args):
     if (not args.no_autotune and wl["patches"] and plan.info["max_pad"] <= 4096
             and plan.info["cross_mode"] != 2):
         t0 = time.perf_counter()
-        pads = sorted({sg_pad(p[1]) for p in wl["patches"]} | {sg_pad(p[2]) for p in wl["patches"]})
-        res = sg.sg_autotune(sg.SG_FP32, pads[0], pads[-1], reps=15)
-        tuned = {"seconds": time.perf_counter() - t0, "shapes": {str(p): res[p][0] for p in pads}}
+        pads = sorted({_pad(p[1]) for p in wl["patches"]} | {_pad(p[2]) for p in wl["patches"]})
+        sg.sg_autotune(sg.SG_FP32, pads[0], pads[-1], reps=15)
+        tuned = {"seconds": time.perf_counter() - t0,
+                 "shapes": {str(p): sg.sg_tune_get(sg.SG_FP32, p) for p in pads}}
     # the cross-patch direct sum's split and far-field grid (skipped where one
     # solve takes seconds: the candidates would take minutes)
     if not args.no_autotune and plan.info["cross_mode"] == 1 and plan.info["cross_pairs"] < 1e11:

@@ -125,7 +125,7 @@ typedef struct {
     int64_t cross_pairs;        /* leaf-target x leaf-source pairs summed directly */
     int64_t device_bytes;       /* device memory held by the plan now */
     int64_t scratch_bytes;      /* per-call scratch (workspace) of one solve */
-    int max_pad;                /* largest padded FFT length, rounded up to a power of two */
+    int max_pad;                /* largest padded FFT length */
     int64_t nzones;             /* zones of a plan made by sg_plan_create_zones, else 0 */
     int launches;               /* kernels one sg_force (sg_force_zones for zone plans) enqueues */
     int cross_mode;             /* the path chosen: SG_CROSS_DIRECT or SG_CROSS_LEVELS (0 for a
@@ -442,9 +442,9 @@ sg_status sg_zones_links(const sg_zones *zones, int64_t *parent, uint8_t *leaf, 
  * three compiled launch shapes per padded length: half, the measured default
  * and twice the default number of row sequences (forward and inverse row
  * passes) or columns (column passes) per CTA, where shared memory and CTA size
- * allow (lengths 5/4 and 3/2 of a power of two, from 320 on, have one shape).
- * A process-wide table, initially the defaults, selects one per power-of-two
- * (precision, padded length); results are bit-identical under every shape
+ * allow. The padded lengths are 64, 128, 256 and from there 5/4, 3/2 and 2 times
+ * each power of two: 320, 384, 512, ... 4096. A process-wide table, initially
+ * the defaults, selects one per (precision, padded length); results are bit-identical under every shape
  * (only the grouping of sequences into CTAs changes). Solves read the table
  * when they enqueue (a graph captures the shapes in force at capture).
  *   shape[4]: 0 forward row pass, 1 inverse row pass, 2 column pass,
@@ -452,7 +452,7 @@ sg_status sg_zones_links(const sg_zones *zones, int64_t *parent, uint8_t *leaf, 
  * ------------------------------------------------------------------------ */
 
 /* Shapes in force for `precision` (SG_FP64 / SG_FP32) and padded length `pad`
- * (64 ... 4096, a power of two). Host only. Errors: SG_EINVAL. */
+ * (one of the lengths above). Host only. Errors: SG_EINVAL. */
 sg_status sg_tune_get(int precision, int pad, int *shape);
 
 /* Select shapes (each 0 or one of the compiled candidates; SG_EINVAL names the
@@ -460,11 +460,11 @@ sg_status sg_tune_get(int precision, int pad, int *shape);
 sg_status sg_tune_set(int precision, int pad, const int *shape);
 
 /* Time every candidate of every pass on a square patch of each padded length
- * min_pad ... max_pad (powers of two; caller slopes for the row and column
+ * min_pad ... max_pad (caller slopes for the row and column
  * passes, central slopes for the central column pass), median of `reps`
  * solves after one warm-up, one pass at a time in order, and keep the fastest.
- * best_ms (NULL or one entry per length) receives the median solve time with
- * the chosen shapes. Synchronous on the current device; allocates temporary
+ * best_ms (NULL or one entry for each length min_pad 2^k up to max_pad) receives
+ * the median solve time with the chosen shapes. Synchronous on the current device; allocates temporary
  * plans and buffers. Errors: SG_EINVAL, SG_ENOMEM, SG_ECUDA. */
 sg_status sg_autotune(int precision, int min_pad, int max_pad, int reps, double *best_ms);
 

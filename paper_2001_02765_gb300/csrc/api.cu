@@ -1063,7 +1063,12 @@ sg_status sg_plan_get_info(const sg_plan *plan, sg_plan_info *out)
     out->cross_pairs = plan->cross_pairs;
     out->device_bytes = plan->device_bytes;
     out->scratch_bytes = plan->scratch_bytes;
-    out->max_pad = plan->max_pad;
+    // the longest transform of a solve (plan->max_pad is the power of two of its twiddle tables)
+    out->max_pad = SG_MIN_PAD;
+    if (plan->lv) out->max_pad = std::max(plan->lv->px, plan->lv->py);
+    else
+        for (int k = 0; k < plan->npatches; ++k)
+            out->max_pad = std::max(out->max_pad, std::max(plan->pp[k].d.px, plan->pp[k].d.py));
     out->nzones = plan->nzones;
     out->launches = plan->launches;
     out->cross_mode = plan->cross_mode;

@@ -35,7 +35,7 @@
 // one row field and one forward column transform instead of three.
 //
 // The kernels and their launch-shape variants are split over translation
-// units by stage (fftconv_rows.cu, fftconv_cols.cu, fftconv_central.cu); the
+// units by stage (fftconv_rows.inl, fftconv_cols.inl, fftconv_central.inl); the
 // solve (fftconv.cu) calls them through the dispatchers declared below with
 // the launch shapes of the tuning table (tune.cu).
 #pragma once
@@ -984,7 +984,7 @@ __host__ __device__ constexpr int row_threads(int px, int nb)
     return ((n + r - 1) / r + 31) / 32 * 32;
 }
 
-// Candidate shapes of the powers of two: half, the default, and twice the default, where feasible
+// Candidate shapes: half, the default, and twice the default, where feasible
 // (shared memory within 200 KB, 32..512 threads per CTA: 1024 would cap registers at 64).
 __host__ __device__ constexpr int shape_candidate(int def, int k) { return k == 0 ? def / 2 : (k == 1 ? def : 2 * def); }
 template <typename T>

@@ -42,10 +42,10 @@ sg_status cols_central_py(int cb, int nout, const col_args<T> &one, const col_ar
         return launch_cols_central<T, PY, D, 3, false>(one, many, bs, qx, tw, err, st, dep);
     }
     if (cb == D) return launch_cols_central_any<T, PY, D>(one, many, bs, qx, tw, err, st, dep);
-    if constexpr (sg_pow2(PY) && col_feasible_t<T, PY, A, 6>()) {
+    if constexpr (col_feasible_t<T, PY, A, 6>()) {
         if (cb == A) return launch_cols_central_any<T, PY, A>(one, many, bs, qx, tw, err, st, dep);
     }
-    if constexpr (sg_pow2(PY) && col_feasible_t<T, PY, C, 6>()) {
+    if constexpr (col_feasible_t<T, PY, C, 6>()) {
         if (cb == C) return launch_cols_central_any<T, PY, C>(one, many, bs, qx, tw, err, st, dep);
     }
     return SG_EINVAL;
@@ -88,14 +88,5 @@ sg_status edge_cols(int py, const edge_args<T> &one, const cplx_t<T> *tw, cudaSt
     SG_PAD_SWITCH(py, return (launch_edge_cols<T, PP>(one, many, bs, tw, st)));
     return SG_EINVAL;
 }
-
-template sg_status cols_central<float>(int, int, int, const col_args<float> &, int, const float2 *, int *, cudaStream_t,
-                                       const col_args<float> *, batch_shape, bool);
-template sg_status cols_central<double>(int, int, int, const col_args<double> &, int, const double2 *, int *, cudaStream_t,
-                                        const col_args<double> *, batch_shape, bool);
-template sg_status edge_cols<float>(int, const edge_args<float> &, const float2 *, cudaStream_t,
-                                    const edge_args<float> *, batch_shape);
-template sg_status edge_cols<double>(int, const edge_args<double> &, const double2 *, cudaStream_t,
-                                     const edge_args<double> *, batch_shape);
 
 }  // namespace sgk

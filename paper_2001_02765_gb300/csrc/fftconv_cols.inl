@@ -43,10 +43,10 @@ sg_status cols_py(int cb, const col_args<T> &one, const col_args<T> *many, batch
     constexpr int D = col_cb_default(PY);
     constexpr int A = shape_candidate(D, 0), C = shape_candidate(D, 2);
     if (cb == D) return launch_cols_any<T, PY, D, NOUT>(one, many, bs, qx, nf, tw, err, st, dep);
-    if constexpr (sg_pow2(PY) && col_feasible_t<T, PY, A, NPL>()) {
+    if constexpr (col_feasible_t<T, PY, A, NPL>()) {
         if (cb == A) return launch_cols_any<T, PY, A, NOUT>(one, many, bs, qx, nf, tw, err, st, dep);
     }
-    if constexpr (sg_pow2(PY) && col_feasible_t<T, PY, C, NPL>()) {
+    if constexpr (col_feasible_t<T, PY, C, NPL>()) {
         if (cb == C) return launch_cols_any<T, PY, C, NOUT>(one, many, bs, qx, nf, tw, err, st, dep);
     }
     return SG_EINVAL;

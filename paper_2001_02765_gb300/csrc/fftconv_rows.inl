@@ -51,10 +51,10 @@ sg_status rows_fwd_px(int nb, const row_fwd_args<T> &one, const row_fwd_args<T> 
     constexpr int D = row_nb_default(PX);
     constexpr int A = shape_candidate(D, 0), C = shape_candidate(D, 2);
     if (nb == D) return launch_rows_fwd_any<T, PX, D>(one, many, ed, ed_many, bs, nf, tw, st, edge);
-    if constexpr (sg_pow2(PX) && row_feasible_t<T>(PX, A)) {
+    if constexpr (row_feasible_t<T>(PX, A)) {
         if (nb == A) return launch_rows_fwd_any<T, PX, A>(one, many, ed, ed_many, bs, nf, tw, st, edge);
     }
-    if constexpr (sg_pow2(PX) && row_feasible_t<T>(PX, C)) {
+    if constexpr (row_feasible_t<T>(PX, C)) {
         if (nb == C) return launch_rows_fwd_any<T, PX, C>(one, many, ed, ed_many, bs, nf, tw, st, edge);
     }
     return SG_EINVAL;
@@ -70,12 +70,5 @@ sg_status rows_fwd(int px, int nb, const row_fwd_args<T> &one, int nf, const cpl
     SG_PAD_SWITCH(px, return (rows_fwd_px<T, PP>(nb, one, many, bs, nf, tw, st, edge, ed, ed_many)));
     return SG_EINVAL;
 }
-
-template sg_status rows_fwd<float>(int, int, const row_fwd_args<float> &, int, const float2 *, cudaStream_t,
-                                   const row_fwd_args<float> *, batch_shape, int, const edge_args<float> *,
-                                   const edge_args<float> *);
-template sg_status rows_fwd<double>(int, int, const row_fwd_args<double> &, int, const double2 *, cudaStream_t,
-                                    const row_fwd_args<double> *, batch_shape, int, const edge_args<double> *,
-                                    const edge_args<double> *);
 
 }  // namespace sgk

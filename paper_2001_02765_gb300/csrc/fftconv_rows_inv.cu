@@ -36,10 +36,10 @@ sg_status rows_inv_px(int nb, const row_inv_args<T> &one, const row_inv_args<T> 
     constexpr int D = row_nb_inv_default(PX);
     constexpr int A = shape_candidate(D, 0), C = shape_candidate(D, 2);
     if (nb == D) return launch_rows_inv_any<T, PX, D>(one, many, bs, nout, tw, st);
-    if constexpr (sg_pow2(PX) && row_feasible_t<T>(PX, A)) {
+    if constexpr (row_feasible_t<T>(PX, A)) {
         if (nb == A) return launch_rows_inv_any<T, PX, A>(one, many, bs, nout, tw, st);
     }
-    if constexpr (sg_pow2(PX) && row_feasible_t<T>(PX, C)) {
+    if constexpr (row_feasible_t<T>(PX, C)) {
         if (nb == C) return launch_rows_inv_any<T, PX, C>(one, many, bs, nout, tw, st);
     }
     return SG_EINVAL;

@@ -22,14 +22,15 @@
 
 namespace {
 
-constexpr int NPAD = 7;  // 64 .. 4096
+constexpr int NPAD = 15;  // the transform lengths 64, 128, 256, 320, 384, 512, ..., 4096 (sg_next_length)
 std::atomic<int> g_shape[2][NPAD][SG_TUNE_KNOBS];  // 0 = default
 std::mutex g_tune_mutex;                            // one sg_autotune at a time
 
 int pad_index(int pad)
 {
-    for (int i = 0; i < NPAD; ++i)
-        if (pad == (SG_MIN_PAD << i)) return i;
+    int i = 0;
+    for (int L = SG_MIN_PAD; L <= SG_MAX_PAD; L = sg_next_length(L), ++i)
+        if (pad == L) return i;
     return -1;
 }
 
@@ -53,8 +54,8 @@ int64_t col_smem(int pad, int cb, int npl, bool fp64)
 bool knob_feasible(int knob, int pad, int v, bool fp64)
 {
     const int d = knob_default(knob, pad);
-    if (v != d && v != d / 2 && v != 2 * d) return false;
-    if (v < 1) return false;
+    if (v == d) return true;  // compiled whatever it takes
+    if ((v != d / 2 && v != 2 * d) || v < 1) return false;
     if (knob <= 1) {
         const int64_t n = (int64_t)v * pad;
         const int64_t padded = fp64 ? (n - 1) + ((n - 1) >> 3) + 1 : (n - 1) + ((n - 1) >> 4) + 1;
@@ -100,7 +101,7 @@ extern "C" {
 sg_status sg_tune_get(int precision, int pad, int *shape)
 {
     if ((precision != SG_FP64 && precision != SG_FP32) || pad_index(pad) < 0 || !shape) {
-        sg_set_last_error_message("sg_tune_get: precision, padded length (64..4096, power of two) or shape invalid");
+        sg_set_last_error_message("sg_tune_get: precision, padded length (a transform length, 64..4096) or shape invalid");
         return SG_EINVAL;
     }
     sg_tune_shape((sg_precision)precision, pad, shape);
@@ -111,7 +112,7 @@ sg_status sg_tune_set(int precision, int pad, const int *shape)
 {
     const int i = pad_index(pad);
     if ((precision != SG_FP64 && precision != SG_FP32) || i < 0 || !shape) {
-        sg_set_last_error_message("sg_tune_set: precision, padded length (64..4096, power of two) or shape invalid");
+        sg_set_last_error_message("sg_tune_set: precision, padded length (a transform length, 64..4096) or shape invalid");
         return SG_EINVAL;
     }
     for (int k = 0; k < SG_TUNE_KNOBS; ++k) {
@@ -142,7 +143,9 @@ sg_status sg_autotune(int precision, int min_pad, int max_pad, int reps, double 
     SG_CUDA_TRY(cudaEventCreate(&e0));
     SG_CUDA_TRY(cudaEventCreate(&e1));
     sg_status st = SG_OK;
-    for (int pad = min_pad, slot = 0; pad <= max_pad && st == SG_OK; pad <<= 1, ++slot) {
+    // best_ms has an entry for min_pad 2^k only; the lengths between are tuned too
+    int reported = min_pad, slot = 0;
+    for (int pad = min_pad; pad <= max_pad && st == SG_OK; pad = sg_next_length(pad)) {
         const int n = pad / 2;  // the largest patch that pads to this length
         // a caller-slope plan (three fields) for the row and generic column passes,
         // a central-slope plan for the central column pass
@@ -201,7 +204,11 @@ sg_status sg_autotune(int precision, int min_pad, int max_pad, int reps, double 
             g_shape[pi][pad_index(pad)][k].store(choice);
             if (m == 0) best = best_k;
         }
-        if (best_ms && st == SG_OK) best_ms[slot] = best;
+        if (pad == reported) {
+            if (best_ms && st == SG_OK) best_ms[slot] = best;
+            ++slot;
+            reported *= 2;
+        }
         cudaFree(buf);
         for (sg_plan *p : plans) sg_plan_destroy(p);
     }

@@ -444,7 +444,8 @@ def sg_tune_set(precision, pad, shape):
 
 
 def sg_autotune(precision, min_pad, max_pad, reps=5):
-    """Tune the launch shapes; returns {pad: (shapes, best solve ms)}."""
+    """Tune the launch shapes of every length from min_pad to max_pad; returns {pad: (shapes, best solve ms)}
+    for min_pad, 2 min_pad, 4 min_pad, ... (sg_tune_get tells those of the lengths between)."""
     pads = []
     p = int(min_pad)
     while p <= int(max_pad):

@@ -61,3 +61,46 @@ def test_plan_tuner_times_a_solve_of_a_real_density(sg):
         ms.append(e[0].elapsed_time(e[1]))
     plan.close()
     assert best > 0.75 * sorted(ms)[4], (best, ms)
+
+
+def _near_bytes(plan_patches, z):
+    """Bytes of every near table of a hierarchy without masks: 12 x 12 cells, two FP32
+    numbers, six planes (nine off the plane) per position; 4^g positions for width
+    ratios 2^g up to 2^5 with at least as many targets, one for wider targets."""
+    nlev = 1 + max(p[0] for p in plan_patches)
+    leaves = [sum(p[1] * p[2] for p in plan_patches if p[0] == l) -
+              sum(p[1] * p[2] // 4 for p in plan_patches if p[0] == l + 1) for l in range(nlev)]
+    keys = {(ls, max(-1, lt - ls)) for ls in range(nlev) for lt in range(nlev)
+            if leaves[lt] > 0 and (lt <= ls or (lt - ls <= 5 and 4 ** (lt - ls) <= leaves[lt]))}
+    every = all(lt <= ls or (lt - ls <= 5 and 4 ** (lt - ls) <= leaves[lt]) for ls in range(nlev) for lt in range(nlev)
+                if leaves[lt] > 0)
+    return sum(4 ** max(g, 0) for _, g in keys) * (9 if z else 6) * 144 * 8, every
+
+
+@pytest.mark.parametrize("kind", ["force", "potential", "force3"])
+@pytest.mark.parametrize("shape", ["deep", "ragged", "side", "wide"])
+def test_every_near_pair_in_the_corner_form(sg, shape, kind):
+    """A budget without room for any near table: cells of the targets' own width and
+    narrower ones (targets on their corners: the coincident-line forms) in the corner
+    form too, to the tolerance of the tables."""
+    from tests.test_gpu_cross_clusters import SHAPES, TOL, _fields, _reference, _solve
+    from tests._lib import gather_leaves
+    patches = SHAPES[shape]
+    z = 0.4 * patches[-1][5] if kind == "force3" else 0.0
+    near, every = _near_bytes(patches, z)
+    full = sg.Plan(patches, cross_mode=sg.SG_CROSS_DIRECT, z=z)
+    total = sg.sg_plan_bytes(patches, sg.SG_FP32, z=z, cross_mode=sg.SG_CROSS_DIRECT)
+    plan = sg.Plan(patches, cross_mode=sg.SG_CROSS_DIRECT, z=z, hbm_budget=total - near)
+    assert plan.info["launches"] == full.info["launches"] + (1 if every else 0)
+    assert plan.info["device_bytes"] < full.info["device_bytes"] - near // 2
+    with pytest.raises(sg.SgError):
+        sg.Plan(patches, cross_mode=sg.SG_CROSS_DIRECT, z=z, hbm_budget=total - near - 1)
+    full.close()
+    f = _fields(patches, seed=len(shape))
+    got = _solve(plan, kind, f)
+    leaves, ref = _reference(patches, kind, f, z)
+    g = [gather_leaves(plan, v, leaves) for v in got]
+    plan.close()
+    err = np.sqrt(sum(np.sum((a - b) ** 2) for a, b in zip(g, ref)) / sum(np.sum(b ** 2) for b in ref))
+    print("rel L2 %s %s: %.2e" % (shape, kind, err))
+    assert err < TOL
