@@ -37,7 +37,11 @@ __device__ __forceinline__ void sg_dep_trigger() { asm volatile("griddepcontrol.
 // The start of a solve's first kernel: the next kernel may start only when the
 // previous solve has finished. Without such a stop in the chain the kernels of
 // several solves wait on the SMs at once, which costs more than it hides (250^2
-// caller-slope solves back to back: 25 us each, 15 with the stop).
+// caller-slope solves back to back: 25 us each, 15 with the stop). A dependent
+// first launch is safe whatever comes before it: the wait comes before any access
+// and returns only when the kernel before it in the stream has finished and its
+// writes are visible, and a launch that follows an event wait, a copy or another
+// branch's work in a captured graph starts only after those, as any launch does.
 __device__ __forceinline__ void sg_dep_first()
 {
     sg_dep_wait();

@@ -1021,18 +1021,16 @@ template <typename T>
 sg_status rows_fwd(int px, int nb, const row_fwd_args<T> &one, int nf, const cplx_t<T> *tw, cudaStream_t st,
                    const row_fwd_args<T> *many = nullptr, batch_shape bs = {0, 0}, int edge = EDGE_NONE,
                    const edge_args<T> *ed = nullptr, const edge_args<T> *ed_many = nullptr);
-// The column and inverse-row passes are launched as dependent launches
-// (sg_launch_dep) on the pass before them in the stream; dep = false launches a
-// column pass normally (when its stream waits on an event just before it).
+// Every pass is a dependent launch (sg_launch_dep) on the kernel before it in the stream.
 template <typename T>
 sg_status rows_inv(int px, int nb, const row_inv_args<T> &one, int nout, const cplx_t<T> *tw, cudaStream_t st,
                    const row_inv_args<T> *many = nullptr, batch_shape bs = {0, 0});
 template <typename T>
 sg_status cols(int py, int cb, int nout, const col_args<T> &one, int qx, int nf, const cplx_t<T> *tw, int *err,
-               cudaStream_t st, const col_args<T> *many = nullptr, batch_shape bs = {0, 0}, bool dep = true);
+               cudaStream_t st, const col_args<T> *many = nullptr, batch_shape bs = {0, 0});
 template <typename T>
 sg_status cols_central(int py, int cb, int nout, const col_args<T> &one, int qx, const cplx_t<T> *tw, int *err, cudaStream_t st,
-                       const col_args<T> *many = nullptr, batch_shape bs = {0, 0}, bool dep = true);
+                       const col_args<T> *many = nullptr, batch_shape bs = {0, 0});
 template <typename T>
 sg_status edge_cols(int py, const edge_args<T> &one, const cplx_t<T> *tw, cudaStream_t st,
                     const edge_args<T> *many = nullptr, batch_shape bs = {0, 0});

@@ -3,7 +3,7 @@
 
 namespace sgk {
 template sg_status cols_central<float>(int, int, int, const col_args<float> &, int, const float2 *, int *, cudaStream_t,
-                                       const col_args<float> *, batch_shape, bool);
+                                       const col_args<float> *, batch_shape);
 template sg_status edge_cols<float>(int, const edge_args<float> &, const float2 *, cudaStream_t,
                                     const edge_args<float> *, batch_shape);
 }  // namespace sgk

@@ -87,13 +87,13 @@ sg_status edge_cols(int, const edge_args<T> &, const cplx_t<T> *, cudaStream_t, 
 }
 template <typename T>
 sg_status cols(int, int, int, const col_args<T> &, int, int, const cplx_t<T> *, int *, cudaStream_t, const col_args<T> *,
-               batch_shape, bool)
+               batch_shape)
 {
     return SG_OK;
 }
 template <typename T>
 sg_status cols_central(int, int, int, const col_args<T> &, int, const cplx_t<T> *, int *, cudaStream_t,
-                       const col_args<T> *, batch_shape, bool)
+                       const col_args<T> *, batch_shape)
 {
     return SG_OK;
 }
