@@ -403,7 +403,7 @@ struct far_args {
     int npatches;
     const float *sigma, *dx, *dy;   // composite sources
     double lambda;                  // lattice unit
-    double G;
+    double G;                       // over 2^sum_exponent
     double zl;                      // height in lattice units
     int ctas;                       // CTAs of the middle and far field; the near field's follow
     int ntargets;
@@ -670,7 +670,7 @@ struct near_list {
 // the integral diverges (a target on a corner or inside an edge of a cell: never a
 // leaf target with a cell that carries density).
 template <int Q>
-__global__ void k_near_table(float2 *__restrict__ out, near_list L, double G, double z)
+__global__ void k_near_table(float2 *__restrict__ out, near_list L, double G, double z)  // G: over 2^sum_exponent
 {
     const int64_t total = (int64_t)L.first[L.n] * NEAR_CELLS;
     for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
@@ -812,10 +812,11 @@ __global__ void __launch_bounds__(NEAR_WARPS * 32, 3) k_near_far(far_args A)
     else near_field<Q>(A, (int)blockIdx.x - A.ctas);
 }
 
-// Adds the sums to the targets' own-patch results.
+// Adds the sums, times scale (2^sum_exponent), to the targets' own-patch results.
 template <int Q>
 __global__ void __launch_bounds__(256) k_cross_add(const int4 *__restrict__ targets, int ntargets,
-                                                   const double *__restrict__ sums, float *o0, float *o1, float *o2)
+                                                   const double *__restrict__ sums, double scale, float *o0, float *o1,
+                                                   float *o2)
 {
     constexpr int NO = q_out<Q>();
     sg_dep_trigger();
@@ -827,7 +828,7 @@ __global__ void __launch_bounds__(256) k_cross_add(const int4 *__restrict__ targ
 #pragma unroll
     for (int o = 0; o < NO; ++o) {
         if (!out[o]) continue;  // sg_force on an off-plane plan takes Fx, Fy only
-        out[o][at] = (float)((double)out[o][at] + sums[(int64_t)t * NO + o]);
+        out[o][at] = (float)((double)out[o][at] + scale * sums[(int64_t)t * NO + o]);
     }
 }
 
@@ -954,6 +955,21 @@ __global__ void __launch_bounds__(NEAR_WARPS * 32) k_near_corner(const int4 *__r
     }
 }
 
+// The near tables and the targets' sums hold G times the integrals over 2^e, and
+// k_cross_add multiplies by 2^e: G, or G H in the potential, and half of H's exponent
+// are taken out, so that the tables' planes of sigma (as 1 / sqrt(H)) and of the slopes
+// (as sqrt(H)) are of FP32's middle range whatever the units. Powers of two: no bit of
+// an ordinary result changes. (Without it the potential's tables overflowed from
+// G H^2 = 3e38 on, where the FP32 spectra of the patches' own convolutions, over Px Py,
+// still fit. In k_cross_add and not in near_field: one FP64 multiplication more per
+// component and warp there cost 6 % of a solve of 2048^2 cells in four patches.)
+template <int Q>
+int sum_exponent(const sg_plan *plan)
+{
+    const int h = ilogb(plan->lattice_unit), g = plan->geom.G != 0.0 ? ilogb(plan->geom.G) : 0;
+    return g + (Q == Q_POT ? h : 0) + h / 2;
+}
+
 // ---------------------------------------------------------------- solve --
 
 template <int Q>
@@ -975,6 +991,7 @@ sg_status solve(sg_plan *plan, const sg_workspace *ws, const float *sigma, const
     sg_timing_begin(ws, SG_STAGE_DIRECT, st);
     const int grid_n = (plan->ntargets + NEAR_WARPS - 1) / NEAR_WARPS;
     const sg_near_tab &nt = Q == Q_POT ? F.ptab : F.tab;
+    const double Gs = ldexp(plan->geom.G, -sum_exponent<Q>(plan));
     far_args A;
     memset(&A, 0, sizeof(A));
     A.blocks = plan->blocks;
@@ -989,7 +1006,7 @@ sg_status solve(sg_plan *plan, const sg_workspace *ws, const float *sigma, const
     A.dx = dx;
     A.dy = dy;
     A.lambda = plan->lattice_unit;
-    A.G = plan->geom.G;
+    A.G = Gs;
     A.zl = plan->geom.z / plan->lattice_unit;
     A.ctas = plan->far_grid;
     A.ntargets = plan->ntargets;
@@ -1000,9 +1017,9 @@ sg_status solve(sg_plan *plan, const sg_workspace *ws, const float *sigma, const
     if (F.untabled)
         SG_CUDA_TRY(sg_launch_dep(k_near_corner<Q>, dim3(grid_n), dim3(NEAR_WARPS * 32), 0, st, plan->targets,
                                   plan->ntargets, plan->patch_dev, plan->npatches, sigma, dx, dy, F.keys,
-                                  plan->lattice_unit, plan->geom.G, plan->geom.z, ws->partial));
+                                  plan->lattice_unit, Gs, plan->geom.z, ws->partial));
     SG_CUDA_TRY(sg_launch_dep(k_cross_add<Q>, dim3((plan->ntargets + 255) / 256), dim3(256), 0, st, plan->targets,
-                              plan->ntargets, A.sums, o0, o1, o2));
+                              plan->ntargets, A.sums, ldexp(1.0, sum_exponent<Q>(plan)), o0, o1, o2));
     SG_CUDA_TRY(cudaGetLastError());
     sg_timing_end(ws, SG_STAGE_DIRECT, st);
     return SG_OK;
@@ -1054,7 +1071,7 @@ sg_status build_tables(sg_plan *plan, sg_near_tab &nt)
     L.first[L.n] = F.nclass;
     if (F.nclass == 0) return SG_OK;
     const int grid = (int)std::min<int64_t>(((int64_t)F.nclass * NEAR_CELLS + 127) / 128, 1 << 16);
-    k_near_table<Q><<<grid, 128>>>((float2 *)nt.data, L, plan->geom.G, plan->geom.z);
+    k_near_table<Q><<<grid, 128>>>((float2 *)nt.data, L, ldexp(plan->geom.G, -sum_exponent<Q>(plan)), plan->geom.z);
     e = cudaGetLastError();
     if (e != cudaSuccess) {
         drop_tables<Q>(plan, nt);

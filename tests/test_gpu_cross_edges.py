@@ -104,3 +104,28 @@ def test_every_near_pair_in_the_corner_form(sg, shape, kind):
     err = np.sqrt(sum(np.sum((a - b) ** 2) for a, b in zip(g, ref)) / sum(np.sum(b ** 2) for b in ref))
     print("rel L2 %s %s: %.2e" % (shape, kind, err))
     assert err < TOL
+
+
+@pytest.mark.parametrize("kind", ["force", "potential"])
+@pytest.mark.parametrize("exponent", [-40, -20, 30, 60, 70])
+def test_units_of_length_change_no_bit(sg, kind, exponent):
+    """Lengths times 2^e with slopes over 2^e: the force is the same and the potential
+    2^e times it, bit for bit (from 2^-40, below which the patches' own FP32 spectra
+    lose bits, to 2^70, where G H^2 is beyond FP32)."""
+    import torch
+    from paper_2001_02765_gb300 import workloads as W
+    from tests._lib import to_dev
+    base = [(lev,) + p for lev, p in enumerate(W.centred_nested_patches(32, 3))]
+    n = sum(p[1] * p[2] for p in base)
+    rng = np.random.Generator(np.random.PCG64(1))
+    s, x, y = (rng.uniform(-1, 1, n).astype(np.float32).astype(np.float64) for _ in range(3))
+    out = []
+    for e in (0, exponent):
+        f = 2.0 ** e
+        plan = sg.Plan([(l, nx, ny, x0 * f, y0 * f, h * f) for l, nx, ny, x0, y0, h in base],
+                       cross_mode=sg.SG_CROSS_DIRECT)
+        r = getattr(plan, kind)(*[to_dev(a, np.float32) for a in (s, x / f, y / f)])
+        torch.cuda.synchronize()
+        out.append([t.double() / (f if kind == "potential" else 1.0) for t in (r if isinstance(r, tuple) else (r,))])
+        plan.close()
+    assert all(torch.equal(a, b) for a, b in zip(*out))
