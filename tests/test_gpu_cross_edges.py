@@ -45,17 +45,17 @@ def test_plan_tuner_times_a_solve_of_a_real_density(sg):
     solve timed from Python and for noise)."""
     import torch
     from paper_2001_02765_gb300 import workloads as W
-    patches = [(lev,) + p for lev, p in enumerate(W.centred_nested_patches(256, 4))]
-    plan = sg.Plan(patches, cross_mode=sg.SG_CROSS_DIRECT)
+    patches = [(lev,) + p for lev, p in enumerate(W.centred_nested_patches(128, 3))]
+    plan = sg.Plan(patches, cross_mode=sg.SG_CROSS_DIRECT, z=patches[-1][5])
     best = sg.sg_plan_autotune(plan.handle, 5)
     g = torch.Generator(device="cuda").manual_seed(3)
     f = [torch.rand(plan.ncells, device="cuda", generator=g) for _ in range(3)]
-    plan.force(*f)
+    plan.force3(*f)
     ms = []
     for _ in range(9):
         e = [torch.cuda.Event(enable_timing=True) for _ in range(2)]
         e[0].record()
-        plan.force(*f)
+        plan.force3(*f)
         e[1].record()
         e[1].synchronize()
         ms.append(e[0].elapsed_time(e[1]))
