@@ -100,6 +100,7 @@ struct sg_server {
     std::vector<double> latency_ms;
     std::mutex mu;
     std::condition_variable wake;      // to the worker
+    std::atomic<bool> event{false};    // a submission or completion since the worker last looked
     std::condition_variable finished;  // to waiters
     std::thread worker;
     bool stop = false;
@@ -107,12 +108,22 @@ struct sg_server {
 
 namespace {
 
+// Wake the worker. It may be launching, with nobody waiting on `wake`: the flag keeps
+// the event until it looks again. (Without it a completion during a launch was seen
+// at the next poll, a millisecond later: 128 solves of 200^2, 8 in flight, 37 us each
+// instead of 23.5 with the lock held during launches.)
+void notify(sg_server *s)
+{
+    s->event.store(true);
+    s->wake.notify_one();
+}
+
 void CUDART_CB on_done(void *p)
 {
     sg_request *r = (sg_request *)p;
     r->t_done = now_s();
     r->state.store(RQ_GPU_DONE);
-    r->server->wake.notify_one();
+    notify(r->server);
 }
 
 // Finish a request whose GPU work completed (called with the lock held).
@@ -250,7 +261,7 @@ void CUDART_CB on_group_done(void *p)
         r->t_done = t;
         r->state.store(RQ_GPU_DONE);
     }
-    s->wake.notify_one();
+    notify(s);
 }
 
 // Pack the members' pass arguments into the slot's pinned staging, copy them
@@ -402,7 +413,7 @@ void worker_main(sg_server *s)
             }
         }
         if (s->stop && s->running.empty()) break;
-        s->wake.wait_for(lock, std::chrono::milliseconds(1));
+        s->wake.wait_for(lock, std::chrono::milliseconds(1), [s] { return s->event.exchange(false); });
     }
 }
 
@@ -473,7 +484,7 @@ sg_status sg_server_destroy(sg_server *s)
         s->queue.clear();
         s->stop = true;
     }
-    s->wake.notify_one();
+    notify(s);
     s->worker.join();
     for (auto &kv : s->live) delete kv.second;
     for (cudaStream_t st : s->streams) {
@@ -529,7 +540,7 @@ sg_status sg_submit(sg_server *s, sg_plan *plan, const void *sigma, const void *
         s->submitted++;
         *ticket = r->ticket;
     }
-    s->wake.notify_one();
+    notify(s);
     return SG_OK;
 }
 

@@ -18,6 +18,7 @@ def host(tmp_path_factory):
     return lambda scenario: subprocess.run([exe, scenario], capture_output=True, text=True, timeout=120)
 
 
-def test_failed_group_keeps_arrival_order(host):
-    r = host("failed_group_keeps_arrival_order")
+@pytest.mark.parametrize("scenario", ["failed_group_keeps_arrival_order", "completions_during_a_launch_are_noticed"])
+def test_admission(host, scenario):
+    r = host(scenario)
     assert r.returncode == 0, r.stderr
