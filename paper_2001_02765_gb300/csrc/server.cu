@@ -121,9 +121,10 @@ void notify(sg_server *s)
 void CUDART_CB on_done(void *p)
 {
     sg_request *r = (sg_request *)p;
+    sg_server *s = r->server;  // once the state is stored the request may be finished, reported and freed
     r->t_done = now_s();
     r->state.store(RQ_GPU_DONE);
-    notify(r->server);
+    notify(s);
 }
 
 // Finish a request whose GPU work completed (called with the lock held).
