@@ -63,6 +63,7 @@ struct sg_request {
     int64_t bytes = 0;
     int slot = -1;
     sg_workspace ws;
+    void *block = nullptr;          // the pool allocation of its workspace (a group's: sg_group_run::block)
     std::atomic<int> state{RQ_QUEUED};
     sg_status result = SG_OK;
     double t_submit = 0, t_start = 0, t_done = 0;
@@ -70,12 +71,13 @@ struct sg_request {
     sg_group_run *group = nullptr;  // the grouped admission it runs in (NULL: alone)
 };
 
-// Requests admitted together on one slot; the slot and the device argument
-// arrays are released when the last member has finished.
+// Requests admitted together on one slot; the slot and the allocation of their
+// workspaces and argument arrays are released when the last member has finished.
 struct sg_group_run {
     int slot = -1;
     std::vector<sg_request *> members;
-    void *dargs = nullptr;
+    void *block = nullptr;  // the members' workspaces, then
+    char *dargs = nullptr;  // their pass arguments
     int pending = 0;
 };
 
@@ -110,8 +112,8 @@ namespace {
 
 // Wake the worker. It may be launching, with nobody waiting on `wake`: the flag keeps
 // the event until it looks again. (Without it a completion during a launch was seen
-// at the next poll, a millisecond later: 128 solves of 200^2, 8 in flight, 37 us each
-// instead of 23.5 with the lock held during launches.)
+// at the next poll, up to a millisecond later: 256 solves of mixed lengths from 128^2 to
+// 1024^2, 8 in flight, 30.1 us each; 25.8 with it.)
 void notify(sg_server *s)
 {
     s->event.store(true);
@@ -130,7 +132,7 @@ void CUDART_CB on_done(void *p)
 // Finish a request whose GPU work completed (called with the lock held).
 void finalize(sg_server *s, sg_request *r)
 {
-    sg_workspace_free(&r->ws, s->streams[r->slot], true);
+    memset(&r->ws, 0, sizeof(r->ws));
     s->bytes_in_use -= r->bytes;
     // a bounded wait that ran out in one of the request's kernels (device error word;
     // a group's kernels report into its first member's word, copied to the slot's)
@@ -138,11 +140,13 @@ void finalize(sg_server *s, sg_request *r)
     if (sg_group_run *g = r->group) {
         r->group = nullptr;
         if (--g->pending == 0) {
-            if (g->dargs) cudaFreeAsync(g->dargs, s->streams[g->slot]);
+            cudaFreeAsync(g->block, s->streams[g->slot]);
             s->free_slots.push_back(g->slot);
             delete g;
         }
     } else {
+        cudaFreeAsync(r->block, s->streams[r->slot]);
+        r->block = nullptr;
         s->free_slots.push_back(r->slot);
     }
     r->slot = -1;
@@ -155,33 +159,53 @@ void finalize(sg_server *s, sg_request *r)
     r->state.store(RQ_FINISHED);
 }
 
-// The request's workspace, stream-ordered from the server's pool on `st`, its
-// error word cleared; false (nothing held) when it cannot be allocated now.
-bool alloc_ws(sg_server *s, sg_request *r, cudaStream_t st)
+size_t up256(size_t x) { return (x + 255) & ~(size_t)255; }
+
+// The buffers of a plan's workspace from `base` on (none set where base is NULL);
+// returns their bytes.
+size_t place_ws(const sg_plan *p, sg_workspace *ws, char *base)
 {
-    memset(&r->ws, 0, sizeof(r->ws));
-    sg_status a = SG_OK;
-    {
-        const sg_plan *p = r->plan;
-        int64_t sizes[6] = {p->ws_fwd_bytes, p->ws_inv_bytes, p->ws_sfield_bytes, p->ws_tile_bytes,
-                            p->ws_partial_bytes, 16};
-        void **dst[6] = {&r->ws.work_fwd, &r->ws.work_inv, &r->ws.sfield, &r->ws.tile_w, (void **)&r->ws.partial,
-                         (void **)&r->ws.err};
-        for (int k = 0; k < 6 && a == SG_OK; ++k) {
-            if (sizes[k] <= 0) continue;
-            if (cudaMallocFromPoolAsync(dst[k], (size_t)sizes[k], s->pool, st) != cudaSuccess) {
-                cudaGetLastError();
-                *dst[k] = nullptr;
-                a = SG_ENOMEM;
-            }
-        }
+    const int64_t sizes[5] = {p->ws_fwd_bytes, p->ws_inv_bytes, p->ws_sfield_bytes, p->ws_tile_bytes, p->ws_partial_bytes};
+    void **dst[5] = {&ws->work_fwd, &ws->work_inv, &ws->sfield, &ws->tile_w, (void **)&ws->partial};
+    size_t off = 0;
+    for (int k = 0; k < 5; ++k) {
+        if (sizes[k] <= 0) continue;
+        if (base) *dst[k] = base + off;
+        off += up256((size_t)sizes[k]);
     }
-    if (a == SG_OK && cudaMemsetAsync(r->ws.err, 0, 16, st) != cudaSuccess) a = SG_ECUDA;
-    if (a != SG_OK) {
-        sg_workspace_free(&r->ws, st, true);
-        return false;
+    return off;
+}
+
+// The workspaces of the requests admitted together, their error words (cleared) and
+// `extra` bytes after them (*tail), in one allocation from the server's pool, stream-
+// ordered on `st`; NULL (nothing held) when it cannot be had now. (One allocation per
+// buffer made it 3 x 16 for a group; where the pool's blocks had last served other
+// streams, as in a burst over eight of them, that took 0.5 ms a group: 128 solves of
+// 200^2, 8 in flight, 37 us each; 4.4 with one.)
+void *alloc_ws(sg_server *s, const std::vector<sg_request *> &mem, size_t extra, char **tail, cudaStream_t st)
+{
+    const size_t words = up256(16 * mem.size());
+    size_t total = words;
+    for (const sg_request *r : mem) total += place_ws(r->plan, nullptr, nullptr);
+    char *b = nullptr;
+    if (cudaMallocFromPoolAsync((void **)&b, total + extra, s->pool, st) != cudaSuccess) {
+        cudaGetLastError();
+        return nullptr;
     }
-    return true;
+    if (cudaMemsetAsync(b, 0, words, st) != cudaSuccess) {
+        cudaGetLastError();
+        cudaFreeAsync(b, st);
+        return nullptr;
+    }
+    size_t off = words;
+    for (size_t k = 0; k < mem.size(); ++k) {
+        sg_workspace *ws = &mem[k]->ws;
+        memset(ws, 0, sizeof(*ws));
+        ws->err = (int *)(b + 16 * k);
+        off += place_ws(mem[k]->plan, ws, b + off);
+    }
+    if (tail) *tail = b + off;
+    return b;
 }
 
 // Take requests off the queue for a free slot (lock held): they count as running
@@ -232,7 +256,8 @@ bool start(sg_server *s, sg_request *r, std::unique_lock<std::mutex> &lock)
     s->free_slots.pop_back();
     claim(s, {r}, slot);
     lock.unlock();
-    if (!alloc_ws(s, r, st)) {
+    r->block = alloc_ws(s, {r}, 0, nullptr, st);
+    if (!r->block) {
         lock.lock();
         unclaim(s, {r}, slot);
         return false;
@@ -266,7 +291,7 @@ void CUDART_CB on_group_done(void *p)
 }
 
 // Pack the members' pass arguments into the slot's pinned staging, copy them
-// to a pool allocation and enqueue the grouped launches.
+// behind their workspaces and enqueue the grouped launches.
 template <typename T>
 sg_status group_launch(sg_server *s, sg_group_run *g, cudaStream_t st)
 {
@@ -280,7 +305,7 @@ sg_status group_launch(sg_server *s, sg_group_run *g, cudaStream_t st)
                                       caller ? r->dy : nullptr, r->fx, r->fy, nullptr);
         if (us[k].rf.src.ny > maxny) maxny = us[k].rf.src.ny;
     }
-    auto up = [](size_t x) { return (x + 255) & ~(size_t)255; };
+    const auto up = up256;
     const size_t s0 = m * sizeof(sgk::row_fwd_args<T>), s1 = m * sizeof(sgk::edge_args<T>);
     const size_t s2 = m * sizeof(sgk::col_args<T>), s3 = m * sizeof(sgk::row_inv_args<T>);
     const size_t total = up(s0) + up(s1) + up(s2) + up(s3);
@@ -292,12 +317,7 @@ sg_status group_launch(sg_server *s, sg_group_run *g, cudaStream_t st)
         ((sgk::col_args<T> *)(h + up(s0) + up(s1)))[k] = us[k].col;
         ((sgk::row_inv_args<T> *)(h + up(s0) + up(s1) + up(s2)))[k] = us[k].ri;
     }
-    char *d = nullptr;
-    if (cudaMallocFromPoolAsync((void **)&d, total, s->pool, st) != cudaSuccess) {
-        cudaGetLastError();
-        return SG_ENOMEM;
-    }
-    g->dargs = d;
+    char *d = g->dargs;
     SG_CUDA_TRY(cudaMemcpyAsync(d, h, total, cudaMemcpyHostToDevice, st));
     sgk::group_passes<T> gp;
     gp.u = us[0];
@@ -320,16 +340,17 @@ bool start_group(sg_server *s, const std::vector<sg_request *> &mem, std::unique
     s->free_slots.pop_back();
     claim(s, mem, slot);
     lock.unlock();
-    for (size_t k = 0; k < mem.size(); ++k) {
-        if (!alloc_ws(s, mem[k], st)) {
-            for (size_t q = 0; q < k; ++q) sg_workspace_free(&mem[q]->ws, st, true);
-            lock.lock();
-            unclaim(s, mem, slot);
-            return false;
-        }
+    char *dargs = nullptr;
+    void *block = alloc_ws(s, mem, s->arg_bytes, &dargs, st);
+    if (!block) {
+        lock.lock();
+        unclaim(s, mem, slot);
+        return false;
     }
     sg_group_run *g = new sg_group_run();
     g->slot = slot;
+    g->block = block;
+    g->dargs = dargs;
     g->members = mem;
     g->pending = (int)mem.size();
     for (sg_request *r : mem) r->group = g;
@@ -444,7 +465,7 @@ sg_status sg_server_create(size_t hbm_budget, int max_inflight, sg_server **out)
     if (e == cudaSuccess) memset(s->err_host, 0, sizeof(int) * max_inflight);
     {
         // a group's four argument arrays (FP64, the larger), each padded to 256 bytes
-        auto up = [](size_t x) { return (x + 255) & ~(size_t)255; };
+        const auto up = up256;
         s->arg_bytes = up(GROUP_MAX * sizeof(sgk::row_fwd_args<double>)) + up(GROUP_MAX * sizeof(sgk::edge_args<double>)) +
                        up(GROUP_MAX * sizeof(sgk::col_args<double>)) + up(GROUP_MAX * sizeof(sgk::row_inv_args<double>));
     }

@@ -1,6 +1,6 @@
 // The request server's host side (server.cu) on a CPU: the CUDA runtime calls it
 // makes are replaced by the fakes below. A solve "runs" until the scenario lets it
-// complete; device memory holds the workspace of one request of a kind at a time.
+// complete; pool allocations above a size that it sets fail.
 // Usage: server_host SCENARIO; exits 0 when the scenario holds.
 #include "../paper_2001_02765_gb300/csrc/server.cu"
 
@@ -13,15 +13,14 @@ static std::vector<const void *> g_started;                     // sigma of ever
 static int g_groups = 0;
 static std::unordered_map<void *, size_t> g_live;               // pool allocations
 static bool g_at_once = false;                                  // solves complete within their launch
-static size_t g_scarce = 0;                                     // a size of which one allocation fits at a time
+static size_t g_largest = SIZE_MAX;                             // the largest pool allocation that succeeds
 
 #ifndef __CUDA_ARCH__
 extern "C" {
 cudaError_t cudaMallocFromPoolAsync(void **p, size_t n, cudaMemPool_t, cudaStream_t)
 {
     std::lock_guard<std::mutex> lock(g_mu);
-    for (const auto &kv : g_live)
-        if (n == g_scarce && kv.second == n) return cudaErrorMemoryAllocation;
+    if (n > g_largest) return cudaErrorMemoryAllocation;
     *p = malloc(n);
     g_live[*p] = n;
     return cudaSuccess;
@@ -61,12 +60,6 @@ void sg_set_last_cuda_error(cudaError_t, const char *) {}
 void sg_set_last_error_message(const char *) {}
 void sg_tune_shape(sg_precision, int, int *shape) { memset(shape, 0, SG_TUNE_KNOBS * sizeof(int)); }
 int64_t sg_workspace_bytes(const sg_plan *plan) { return plan->ws_fwd_bytes; }
-void sg_workspace_free(sg_workspace *ws, cudaStream_t st, bool)
-{
-    for (void *p : {ws->work_fwd, (void *)ws->err})
-        if (p) cudaFreeAsync(p, st);
-    memset(ws, 0, sizeof(*ws));
-}
 sg_status sg_force_ws(sg_plan *, const sg_workspace *, const void *sigma, const void *, const void *, void *, void *,
                       cudaStream_t, void *)
 {
@@ -168,7 +161,7 @@ static void failed_group_keeps_arrival_order()
     auto submit = [&](int k, sg_plan *p) { CHECK(sg_submit(s, p, &in[k], nullptr, nullptr, &out, &out, &t[k]) == SG_OK); };
     submit(0, &b);  // holds the only slot while the others arrive
     CHECK(soon([] { return in_flight() == 1; }));
-    g_scarce = 1000;
+    g_largest = 1500;  // one of a's workspaces (1000 bytes and the error word, rounded up), not two
     submit(1, &a);
     submit(2, &b);
     submit(3, &a);
