@@ -1190,13 +1190,13 @@ def oracle_fft_route(wl, reps=3):
             "target_cells_per_s": wl["targets"] / med, "seconds": med}
 
 
-# DRAM bytes (read + write) per launch of a stage's kernel from the ncu capture
-# of the current kernel build (see profiles/); None when not captured for it.
-# amr3 col_conv: the stage's column-transform and column-MAC launches, one each
-# per solve (profiles/amr3_levels_launches.md).
-TRAFFIC = {("spiral1024", "col_conv"): 33.810e6 + 0.014e6,
-           ("amr3", "col_conv"): (11.131e6 + 3.899e6) + (226.635e6 + 6.682e6),
-           ("amr3", "cross_direct"): 3.907e6 + 11.629e6}
+# DRAM bytes (read + write) per solve of a stage's kernels, from ncu captures at
+# commit 6306850 (profiles/spiral1024_passes.md, amr3_levels.md, k_near_far_amr3.md);
+# None when not captured. amr3 col_conv: the column transforms and the column MAC;
+# cross_direct: near and far field, and their addition.
+TRAFFIC = {("spiral1024", "col_conv"): 33.78e6 + 0.07e6,
+           ("amr3", "col_conv"): (11.13e6 + 6.18e6) + (226.61e6 + 9.51e6),
+           ("amr3", "cross_direct"): (10.51e6 + 0.01e6) + 6.56e6}
 
 
 def _pad(n):

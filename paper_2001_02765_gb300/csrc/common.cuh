@@ -142,7 +142,7 @@ struct __align__(32) sg_dvec4 {
 #define SG_CL_CELLS 4
 #define SG_CL_LEVELS 10         // clusters of a patch: 2048 / 4 = 2^9 per side, ten levels
 // Near tables: targets up to 2^SG_NT_GMAX times narrower than the source cells
-// (4^g positions of 6.9 KB each: 7 MB at 5), keyed by log2 of the source cell
+// (4^g positions of 6.9 KB each, 10.4 KB off the plane: 7 and 10.6 MB at 5), keyed by log2 of the source cell
 // width in lattice units (below SG_NT_STEPS) and the width ratio's exponent (-1 .. SG_NT_GMAX).
 #define SG_NT_GMAX 5
 #define SG_NT_KEYS (SG_NT_GMAX + 2)
