@@ -26,8 +26,8 @@
 // (it grows like the square root of the number of corners).
 //
 // The mid-plane potential (sg_potential on hierarchies of this path) is the
-// same sum with the kernel 1/r: its corner form, far-field moments and
-// kernels follow the force's (see the potential section below).
+// same sum with the kernel 1/r: its corner form and kernels follow the force's
+// (see the potential section below).
 #include "common.cuh"
 
 #include <math.h>
